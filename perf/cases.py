@@ -21,6 +21,14 @@ from paper_2501_08192_b200 import binding as P
 
 HEAD = 128
 EPS, THETA = 1e-5, 500000.0
+_streams = []
+
+
+def _stream():
+    """The program's stream: one for all of its calls."""
+    if not _streams:
+        _streams.append(torch.cuda.Stream())
+    return _streams[0]
 
 
 def _case(name, entry, layers, hidden, q_heads, kv_heads, ffn, tp, max_batch, batch, ctx_min, ctx,
@@ -142,7 +150,7 @@ WEIGHTS = ("w_q", "w_k", "w_v", "w_o", "w_gate", "w_up", "w_down", "g_attn", "g_
 def prepare(case, seed):
     cfg, ctx = _config(case), _contexts(case, seed)
     B, H = case["batch"], case["hidden"]
-    state = {"entry": case["entry"], "stream": torch.cuda.Stream(), "layers": [], "ios": [], "outputs": []}
+    state = {"entry": case["entry"], "stream": _stream(), "layers": [], "ios": [], "outputs": []}
     ctx_dev = torch.from_numpy(ctx).cuda()
     before = None
     for i in range(case["layers"]):
