@@ -53,6 +53,22 @@ bool make_map_2d(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 3-D 16-bit tensor map over activation planes: `planes` planes of `rows` rows of `cols` contiguous elements;
+// the box takes the first box_rows rows of every plane (64 x box_rows x planes), 128-byte swizzle.
+bool make_planes_map(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint32_t planes, uint32_t box_rows)
+{
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn)
+        return false;
+    cuuint64_t dims[3] = {cols, rows, planes};
+    cuuint64_t strides[2] = {cols * 2, rows * cols * 2};
+    cuuint32_t box[3] = {64, box_rows, planes};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // 2-D uint8 tensor map: `rows` rows of `cols` contiguous bytes, box (box_cols x box_rows), 128-byte swizzle.
 bool make_u8_map_2d(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint32_t box_cols, uint32_t box_rows)
 {
@@ -130,8 +146,8 @@ struct preserve_layer {
     CUtensorMap wmap[4];
     CUtensorMap wmap256[4];      // box of 256 rows (valid when has256[i])
     bool has256[4];
-    CUtensorMap xmap[4];         // x, o, x2, a as B operands
-    int nb_pad;
+    CUtensorMap xmap[8][4];      // x, o, x2, a as B operands, for a batch tile of 16 * (first index + 1) rows
+    int nb_pad;                  // max_batch rounded up to 16: rows per plane of the workspaces
 
     // K/V maps (re-encoded when the cache pointers change)
     const void *k_ptr, *v_ptr;
@@ -383,9 +399,11 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
         GemmTcArgs a = {};
         a.w_map = L->wmap[which];
         a.w_map256 = L->has256[which] ? &L->wmap256[which] : nullptr;
-        a.x_map = L->xmap[which];
         (void)x;
-        a.B = B; a.NB = L->nb_pad; a.N = d.n[which]; a.K = d.k[which];
+        // The batch tile follows the step's batch, not max_batch: a server sized for 128 sequences that holds
+        // 20 otherwise multiplies, fetches and hands over 128 columns in every projection.
+        a.B = B; a.NB = (B + 15) / 16 * 16; a.N = d.n[which]; a.K = d.k[which];
+        a.x_map = L->xmap[a.NB / 16 - 1][which];
         a.epi = epi;
         a.status = L->status;
         a.trace = trace;
@@ -401,6 +419,7 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
         a.w8 = L->w8 ? 1 : 0;
         a.scales = L->w8 ? L->scales + L->soff[which] : nullptr;
         a.w8_codes = L->w8 ? L->arena + L->off[which] : nullptr;
+        a.w8_tiles = L->w8 ? gemm_tc_w8_tiles(L->nb_pad, a.N, which >= 1) : 0;    // as the codes were packed
         CK(L, launch_gemm_tc(a, L->sm_count, s));
         return PRESERVE_OK;
     }
@@ -1175,14 +1194,15 @@ int preserve_layer_init(const preserve_layer_config_t *cfg, const preserve_layer
     CKI(cudaMalloc(&L->trace_buf, sizeof(long long) * PRESERVE_TRACE_SLOTS * PRESERVE_N_KERNELS));
 
     if (L->tensor_path) {
-        // activations as the B operand: [2 * nb_pad, K] = hi rows then lo rows, one box covers both
+        // activations as the B operand: the first NB rows of each plane, hi rows then lo rows, in one box
         const void *xb[4] = {L->x, L->o, L->x2, L->a};
         for (int i = 0; i < 4; ++i) {
             // x (two fp16 planes: hi rows, lo rows) feeds the QKV projection; o, x2 and a are one fp16 plane each
-            const uint32_t brows = (uint32_t)(i >= 1 ? L->nb_pad : 2 * L->nb_pad);
             // (int8 weights are fetched by plain bulk copies: no map over them)
-            const bool wok = L->w8 || make_map_2d(&L->wmap[i], L->arena + L->off[i], d.k[i], d.n[i], 64, 128);
-            if (!wok || !make_map_2d(&L->xmap[i], xb[i], d.k[i], brows, 64, brows)) {
+            bool ok = L->w8 || make_map_2d(&L->wmap[i], L->arena + L->off[i], d.k[i], d.n[i], 64, 128);
+            for (int nb = 16; ok && nb <= L->nb_pad; nb += 16)
+                ok = make_planes_map(&L->xmap[nb / 16 - 1][i], xb[i], d.k[i], L->nb_pad, i >= 1 ? 1 : 2, nb);
+            if (!ok) {
                 preserve_layer_destroy(L);
                 return PRESERVE_EARCH;
             }

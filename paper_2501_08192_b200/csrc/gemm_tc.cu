@@ -308,10 +308,10 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 uint64_t *bar = (kEarly && first_fill) ? &fullb[st_] : &full[st_];
                 if (kEarly && first_fill)
                     mbar_expect_tx(bar, b_bytes);
-                tma_load_2d(b_dst, &p.x_map, kb_ * kBlk, 0, bar);
-                tma_load_2d(b_dst + b_bytes / 2, &p.x_map, kb_ * kBlk + kTcBlockK, 0, bar);
+                tma_load_3d(b_dst, &p.x_map, kb_ * kBlk, 0, 0, bar);
+                tma_load_3d(b_dst + b_bytes / 2, &p.x_map, kb_ * kBlk + kTcBlockK, 0, 0, bar);
             } else {
-                tma_load_2d(b_dst, &p.x_map, kb_ * kBlk, 0, &full[st_]);
+                tma_load_3d(b_dst, &p.x_map, kb_ * kBlk, 0, 0, &full[st_]);
             }
         };
         for (int i = prod; i < pre; i += NP)
@@ -943,9 +943,9 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     // rows) weighs about as much as a weight tile: halves the L2->SM traffic of the activations, which
     // every CTA re-reads.  With a single fp16 plane of 64 rows it does not: one tile per CTA then gives
     // twice the CTAs (two per SM) and measured 1-1.5 us less on the O and down projections of config 4.
-    const int mt = a.w8 ? gemm_tc_w8_tiles(a.NB, a.N, a.x_fp16 == 1)
+    const int mt = a.w8 ? a.w8_tiles
                         : ((planes * a.NB >= 96 && a.N % (2 * kTcTileM) == 0 && a.w_map256) ? 2 : 1);
-    if (a.w8 && (!a.w8_codes || !a.scales))
+    if (a.w8 && (!a.w8_codes || !a.scales || mt < 1 || mt > 2))
         return cudaErrorInvalidValue;
     p.w8_codes = static_cast<const uint8_t *>(a.w8_codes);
     p.mt = mt;

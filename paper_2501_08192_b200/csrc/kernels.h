@@ -170,8 +170,8 @@ cudaError_t launch_gemv(const GemvArgs &a, int sm_count, cudaStream_t s);
 struct GemmTcArgs {
     CUtensorMap w_map;    // dims (K, N), box (64, 128), 128B swizzle
     const CUtensorMap *w_map256;  // optional: same tensor with box (64, 256), for two weight tiles per CTA
-    CUtensorMap x_map;    // dims (K, 2*NB): hi rows then lo rows; box (64, 2*NB), 128B swizzle - or, with x_fp16,
-                          // dims (K, NB): one fp16 plane, box (64, NB)
+    CUtensorMap x_map;    // dims (K, rows, planes), box (64, NB, planes), 128B swizzle: the first NB rows of the hi and
+                          // the lo plane - or, with x_fp16 = 1, of the one fp16 plane
     int x_fp16;           // 0: two bf16 planes; 2: two fp16 planes (hi rows then lo rows); 1: the activations are one fp16 plane (inputs that come out of an RMSNorm: bounded,
                           // 11 significant bits suffice) instead of bf16 hi + lo planes
     int B, NB, N, K;      // NB = batch rows per plane (multiple of 16)
@@ -185,7 +185,8 @@ struct GemmTcArgs {
     // and multiplies every accumulator row by its scale
     int w8;
     const float *scales;  // w8: [N] in packed row order
-    const void *w8_codes; // w8: the packed codes (launch_pack_rows_w8 with gemm_tc_w8_tiles() rows per block)
+    const void *w8_codes; // w8: the packed codes (launch_pack_rows_w8 with w8_tiles * 128 rows per block)
+    int w8_tiles;         // w8: 128-row tiles per packed block and CTA (gemm_tc_w8_tiles of the largest batch)
 };
 // int8 weights: 128-row weight tiles per CTA for a matrix of N rows and a padded batch of NB (the packed
 // layout depends on it)

@@ -362,3 +362,29 @@ def test_info_reports_plan_and_bytes():
         assert info.sm_count > 0 and info.l2_bytes > 0 and info.uses_tensor_path == 0
     finally:
         dl.close()
+
+
+@pytest.mark.parametrize("flags", [0, P.FLAG_INT8_WEIGHTS], ids=["bf16", "w8"])
+@pytest.mark.parametrize("batches", [(128, (1, 16, 17, 33, 127)), (40, (40, 32, 5, 40))], ids=["max128", "max40"])
+def test_batch_tile_follows_the_step_batch(oracle, batches, flags):
+    """Tensor path with fewer sequences than max_batch: every width of the batch tile (its edges, and one layer
+    going from wide to narrow and back), same tolerance; two KV heads' caches behind the batch stay untouched."""
+    most, steps = batches
+    shape = I.small_shape(name=f"tile_{most}", batch=most, hidden=1024, ffn=640, ctx=70, ctx_min=3, seed=61)
+    t = I.make_layers(shape, 1)[0]
+    dl = G.DeviceLayer(shape, t, flags=flags)
+    try:
+        for B in steps:
+            part = dict(t, **{n: t[n][:B] for n in ("residual_in", "k_cache", "v_cache", "ctx_len")},
+                        **{n: t[n][:, :B] for n in ("partials_in", "attn_peer_partials")})
+            ref = oracle.layer_step(replace(shape, batch=B), part, int8_weights=bool(flags))
+            out = [G.GuardedOut((B, shape.hidden)) for _ in range(3)]
+            io = dl.layer.make_io(B, dl.ctx_dev, dl.ctx_host, dl.partials, dl.peers, dl.residual, dl.k_cache,
+                                  dl.v_cache, *[o.t for o in out])
+            dl.layer.decode_step(io)
+            assert dl.layer.last_status() == P.PRESERVE_OK
+            for name, o in zip(("h2", "mlp_partial", "attn_partial"), out):
+                G.assert_close(G.cuda_to_f32(o.t), ref[name], f"batch {B}:{name}")
+                assert o.guards_intact()
+    finally:
+        dl.close()
