@@ -341,6 +341,15 @@ __device__ __forceinline__ void trace_end(long long *t)
     }
 }
 
+// True in one lane of the (converged) warp.  The compiler knows the branch to be taken by a single thread, which a
+// test of the lane index does not tell it.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t is;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
+    return is != 0;
+}
+
 // Programmatic dependent launch: wait for the producer grid's memory to be
 // visible / allow the dependent grid to start launching.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
