@@ -260,6 +260,11 @@ __device__ __forceinline__ void sts_f32x2(uint32_t addr, float2 v)
 {
     asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
+// One arrival on an mbarrier of another CTA of the cluster (release: this thread's earlier accesses come first).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+}
 // Cluster barrier split in two; the arrive carries no data (it only keeps shared memory alive), so
 // it needs no release.
 __device__ __forceinline__ void cluster_arrive_relaxed()

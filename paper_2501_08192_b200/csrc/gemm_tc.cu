@@ -20,8 +20,7 @@
 //   warps 2.. : epilogue (8 or 16 warps) - tcgen05.ld the accumulator (lane = output row; the warps of
 //               a TMEM lane group share the column chunks), split-K reduction across the cluster as a
 //               one-sided reduce-scatter in rank order (every rank finishes NB / splits columns:
-//               st.async pieces for narrow batches, bulk shared-memory copies for wide ones; reads
-//               through distributed shared memory only where the receive area does not fit), fused
+//               st.async pieces for narrow batches, bulk shared-memory copies for wide ones), fused
 //               epilogue (epilogue.cuh)
 // The kernel is instantiated per (epilogue kind, hand-over form): the tail of one instantiation is
 // a few KB of instructions, which matters for a kernel that runs for microseconds.
@@ -32,13 +31,10 @@
 // Every mbarrier wait is bounded; a wait that gives up records a status code,
 // poisons the rest of the CTA's work, and the CTA still reaches every barrier
 // and frees its TMEM.
-#include <cooperative_groups.h>
 #include <cstdlib>
 #include <type_traits>
 
 #include "epilogue.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace prsv {
 
@@ -61,8 +57,8 @@ struct GemmTcParams {
     int kblocks;        // K / 64 (int8 weights: K / 128 - a stage carries 128 k)
     int splits;         // cluster size along k
     int stages;
-    int push;           // split-K reduction by one-sided hand-over: 1 = st.async, 2 = bulk copies (0: every rank reads all ranks)
-    int recv_off;       // push: offset of the receive area behind the ring
+    int push;           // split-K reduction by one-sided hand-over: 1 = st.async, 2 = bulk copies (0: no split)
+    int recv_off;       // push: offset of the receive area, behind the ring - or (2) in it, behind the staged partial tiles
     int tmem_cols;
     uint32_t idesc;
     EpilogueArgs epi;
@@ -186,14 +182,14 @@ __device__ __forceinline__ void tc_ld_wait(uint32_t (&a)[16], uint32_t (&b)[16])
                  : "memory");
 }
 
-// KIND: the epilogue; PUSH: the split-K hand-over (0 pull, 1 st.async, 2 bulk copies) - template
+// KIND: the epilogue; PUSH: the split-K hand-over (0 none, 1 st.async, 2 bulk copies) - template
 // arguments, so that each instantiation carries a single tail and its instructions stay close together.
 template <int KIND, int PUSH, bool W8 = false, bool EARLY = false>
 __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_constant__ GemmTcParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ uint64_t full[kTcMaxStages], empty[kTcMaxStages], accum_bar, push_bar;
+    __shared__ uint64_t full[kTcMaxStages], empty[kTcMaxStages], accum_bar, push_bar, ready_bar;
     __shared__ uint64_t conv[kTcMaxW8Slots], slot_free[kTcMaxW8Slots];   // int8 weights: a widened tile is complete / has been consumed
     // int8 weights: the activation tiles of the ring's FIRST fill complete a barrier of their own, so that
     // those codes - which land while the kernel in front is still running - are widened before the
@@ -244,6 +240,8 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         if (PUSH && p.splits > 1) {
             // this rank will receive NB / splits columns of every other rank's partial tile
             mbar_init(&push_bar, 1);
+            if (PUSH == 2)
+                mbar_init(&ready_bar, p.splits - 1);     // one arrival per peer whose receive area is free
         }
         mbar_fence_init();
         poisoned = 0;
@@ -594,14 +592,20 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         // copy per (owner, m) moves the owner's columns - a contiguous slice - into the owner's receive
         // area [source slot][m][column][row], signalling the owner's barrier with the bytes.  The owner
         // waits for its area, sums the sources in rank order (its own share straight from its ring)
-        // and applies the epilogue.  The cluster barrier that keeps the senders' shared memory alive
-        // until the copies have landed is split: arrive once this rank's area is complete, wait at
-        // the very end, so its latency hides behind the epilogue.
-        cg::cluster_group cluster = cg::this_cluster();
+        // and applies the epilogue.  Where the receive area behind the ring would leave the ring under four
+        // stages, it lies in the ring instead, behind the staged tiles: a rank may then be written to
+        // once its own MMAs have read the ring, which it tells every peer by an arrival on that peer's
+        // ready barrier before it stages its tiles.  The cluster barrier that keeps the senders' shared
+        // memory alive until the copies have landed is split: arrive once this rank's area is complete,
+        // wait at the very end, so its latency hides behind the epilogue.
         const int cols = p.NB / p.splits;
         float *recv = reinterpret_cast<float *>(smem + p.recv_off);
+        const bool in_ring = p.recv_off < p.stages * stage_bytes;
         cluster_wait();       // (the arrival at the top of the kernel: every rank's receive barrier exists)
         if (is_epi) {
+            // (behind the wait for the accumulators: the ring has been read)
+            if (in_ring && warp == 2 && lane < p.splits && lane != s)
+                mbar_arrive_cluster(cluster_map(&ready_bar, lane));
             // two chunks (four TMEM loads) in flight per wait
             const uint32_t red_row = smem_u32(red) + (uint32_t)row * 4u;
             for (int j = sub; j < p.mt * nchunks; j += 2 * kSubs) {
@@ -644,7 +648,9 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             // the (splits - 1) * mt copies go out side by side
             const int n_ewarps = kSubs * 4;
             const int e = lane < 8 ? (warp - 2) + lane * n_ewarps : 1 << 30;
-            if (e < (p.splits - 1) * p.mt) {
+            if (e < (p.splits - 1) * p.mt && in_ring && !mbar_wait(&ready_bar, 0, p.status, ST_TIMEOUT_MMA)) {
+                poisoned = 1;      // (a peer that is this late gets nothing: its own wait records it)
+            } else if (e < (p.splits - 1) * p.mt) {
                 const int slot_q = e / p.mt, m = e % p.mt;
                 const int q = slot_q < s ? slot_q : slot_q + 1;      // owner
                 const int my_slot = s < q ? s : s - 1;               // where the owner keeps this rank's share
@@ -779,83 +785,6 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             else
                 finish(std::integral_constant<int, 8>());
         }
-    } else if (PUSH == 0 && p.splits > 1) {
-        // Split-K across the cluster, reduce-scatter style: every rank publishes its partial tiles in
-        // its own shared memory, then finishes NB / splits of the batch columns - reading that slice
-        // from all ranks in rank order - so the reduction and the epilogue work are spread over the
-        // whole cluster.
-        cg::cluster_group cluster = cg::this_cluster();
-        if (is_epi) {
-            for (int j = sub; j < p.mt * nchunks; j += kSubs) {      // the lane group's warps share the chunks
-                const int m = j / nchunks, c = j % nchunks;
-                float v[16];
-                load_chunk(m, c, v);
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    red[((size_t)m * p.NB + c * 16 + i) * kTcTileM + row] = v[i];
-            }
-        }
-        cluster.sync();
-        if (is_epi) {
-            const float *remote[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                remote[q] = cluster.map_shared_rank(red, q < p.splits ? q : 0) + row;
-            const int cols = p.NB / p.splits;             // columns finished by this rank (>= 2, even)
-            const int n_pairs = p.mt * cols / 2;
-            // The remote loads of a block of column pairs (16 values per rank slot in flight) are
-            // issued before the first pair of the block is finished: distributed shared memory has a
-            // latency of ~800 cycles, so a thread that fetched pair by pair would spend that long on
-            // each of its mt * cols / 2 pairs.
-            auto run = [&](auto sp_tag) {
-                constexpr int SP = decltype(sp_tag)::value;
-                constexpr int D = 16 / SP;                 // pairs per block
-                // (this warp's pairs: sub, sub + kSubs, ...)
-                for (int it0 = sub; it0 < n_pairs; it0 += D * kSubs) {
-                    float buf[D][2][SP];
-#pragma unroll
-                    for (int d = 0; d < D; ++d) {
-                        const int it = it0 + d * kSubs;
-                        if (it < n_pairs) {
-                            const int m = it / (cols / 2), b0 = s * cols + 2 * (it % (cols / 2));
-#pragma unroll
-                            for (int q = 0; q < SP; ++q) {
-                                buf[d][0][q] = remote[q][((size_t)m * p.NB + b0 + 0) * kTcTileM];
-                                buf[d][1][q] = remote[q][((size_t)m * p.NB + b0 + 1) * kTcTileM];
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int d = 0; d < D; ++d) {
-                        const int it = it0 + d * kSubs;
-                        if (it < n_pairs) {
-                            const int m = it / (cols / 2), b0 = s * cols + 2 * (it % (cols / 2));
-                            const int pair = ((tile * p.mt + m) * kTcTileM + row) >> 1;
-                            float mine[2] = {0.f, 0.f};
-#pragma unroll
-                            for (int q = 0; q < SP; ++q) {       // rank order
-                                mine[0] += buf[d][0][q];
-                                mine[1] += buf[d][1][q];
-                            }
-                            // rows 2r and 2r + 1 (adjacent lanes) form the output pair: the even lane finishes
-                            // column b0, the odd lane column b0 + 1, each with one value from its neighbour -
-                            // one exchange and one epilogue call for the whole warp
-                            const float recv = __shfl_xor_sync(0xffffffffu, par ? mine[0] : mine[1], 1);
-                            const int b = b0 + par;
-                            if (b < p.B && !poisoned)
-                                apply_epilogue_t<KIND>(p.epi, tabs, b, true, p.N, b, pair, par ? recv : mine[0], par ? mine[1] : recv);
-                        }
-                    }
-                }
-            };
-            if (p.splits == 2)
-                run(std::integral_constant<int, 2>());
-            else if (p.splits == 4)
-                run(std::integral_constant<int, 4>());
-            else
-                run(std::integral_constant<int, 8>());
-        }
-        cluster.sync();        // peers' shared memory must outlive the reads
     } else if (is_epi) {
         for (int j = sub; j < p.mt * nchunks; j += kSubs) {
             const int m = j / nchunks, c = j % nchunks;
@@ -930,6 +859,64 @@ int gemm_tc_w8_tiles(int NB, int N, int x_fp16)
     return (N % (2 * kTcTileM) == 0 && 2 * acc + 2 * 2 * 64 <= 512) ? 2 : 1;
 }
 
+// How a GEMM is cut into CTAs when each takes `mt` weight tiles.
+struct TcGeometry {
+    int tiles, stage_bytes, stages, per_sm, splits, w8_slots;
+    bool w8_two;
+    size_t tile_bytes, smem_cap;      // one CTA's partial tiles; shared memory a CTA may use
+    // bulk hand-over: the staged tiles and the other ranks' shares of this rank's columns
+    size_t bulk_bytes(int sp) const { return tile_bytes + tile_bytes / sp * (sp - 1); }
+};
+static bool tc_geometry(const GemmTcArgs &a, int sm_count, int mt, TcGeometry &g)
+{
+    const int planes = a.x_fp16 == 1 ? 1 : 2;
+    const int kblocks = a.K / (a.w8 ? 2 * kTcBlockK : kTcBlockK);
+    g.tiles = a.N / (kTcTileM * mt);
+    // int8 weights: a stage holds the codes (half a 16-bit tile) and the activations; the widened tiles
+    // live in tensor memory behind the accumulators (as many as fit, at most four), so the whole of
+    // shared memory is ring: a deep ring is what keeps enough int8 bytes in flight.  One CTA per SM
+    // (tensor memory is per SM).
+    g.stage_bytes = mt * kATileBytes + planes * a.NB * (a.w8 ? 2 * kTcBlockK : kTcBlockK) * 2;
+    // Two CTAs per SM when each needs at most half of tensor memory (accumulators + at least two widened
+    // tiles in 256 columns) and half of shared memory still holds three stages; else one.
+    g.w8_slots = 0;
+    g.w8_two = false;
+    if (a.w8) {
+        const int acc = mt * planes * a.NB;
+        g.w8_two = acc + 2 * mt * 64 <= 256 && (100 * 1024) / g.stage_bytes >= 3;
+        g.w8_slots = ((g.w8_two ? 256 : 512) - acc) / (mt * 64);
+        g.w8_slots = g.w8_slots > kTcMaxW8Slots ? kTcMaxW8Slots : g.w8_slots;
+        if (g.w8_slots < 2)
+            return false;
+    }
+    // Ring depth, CTAs per SM and cluster splits.  Two CTAs per SM (rings <= 100 KiB) whenever that
+    // leaves >= 4 stages: measured better than one CTA with a ring twice as deep, because the second
+    // CTA streams while the first is in its epilogue.  The grid (tiles x splits) must fit the
+    // co-resident slots (a second wave doubles the kernel); splits are a power of two <= 8 that leave
+    // every rank >= 2 k-blocks and whose hand-over fits shared memory.
+    g.stages = (200 * 1024) / g.stage_bytes;
+    g.per_sm = 1;
+    if (a.w8 ? g.w8_two : (100 * 1024) / g.stage_bytes >= 4) {
+        g.stages = (100 * 1024) / g.stage_bytes;
+        g.per_sm = 2;
+    }
+    if (g.stages > kTcMaxStages) g.stages = kTcMaxStages;
+    if (g.stages < 2)
+        return false;
+    g.tile_bytes = (size_t)mt * a.NB * kTcTileM * 4;
+    g.smem_cap = (size_t)(g.per_sm == 2 ? 108 : 225) * 1024;
+    const int slots = sm_count * g.per_sm;
+    g.splits = 1;
+    while (g.splits < 8 && g.tiles * g.splits * 2 <= slots && kblocks / (g.splits * 2) >= 2) g.splits *= 2;
+    while (g.splits > 1 && g.bulk_bytes(g.splits) + 1024 > g.smem_cap) g.splits /= 2;
+    // Sixteen ranks (a cluster size the device has to be asked for) when even eight leave half of the
+    // SMs without a CTA; only with the bulk hand-over, whose owners may hold a single column.
+    if (g.splits == 8 && g.tiles * 16 <= slots && g.tiles * 8 * 5 <= sm_count * 3 && kblocks / 16 >= 2 &&
+        g.bulk_bytes(16) + 1024 <= g.smem_cap)
+        g.splits = 16;
+    return true;
+}
+
 cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
 {
     if (a.NB < 16 || a.NB > 128 || a.NB % 16 || a.N % kTcTileM || a.K % (a.w8 ? 2 * kTcBlockK : kTcBlockK) || a.B > a.NB)
@@ -946,67 +933,41 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     const int planes = a.x_fp16 == 1 ? 1 : 2;
     p.planes = planes;
     p.f16 = a.x_fp16 ? 1 : 0;
-    // Two 128-row weight tiles per CTA share one activation tile when the activation tile (planes * NB
-    // rows) weighs about as much as a weight tile: halves the L2->SM traffic of the activations, which
-    // every CTA re-reads.  With a single fp16 plane of 64 rows it does not: one tile per CTA then gives
-    // twice the CTAs (two per SM) and measured 1-1.5 us less on the O and down projections of config 4.
-    const int mt = a.w8 ? a.w8_tiles
-                        : ((planes * a.NB >= 96 && a.N % (2 * kTcTileM) == 0 && a.w_map256) ? 2 : 1);
+    // Two 128-row weight tiles per CTA share one activation tile, which halves the L2->SM traffic of the
+    // activations every CTA re-reads - and double the partial tile that the CTA's epilogue has to stage,
+    // send and finish.  They pay only where the activation tile outweighs a weight tile (two planes of 80
+    // rows and more): with pairs from 96 rows up four 70B-shaped TP=8 layers at batch 128 take 420.7 us,
+    // with single tiles 387.2 (tail of each GEMM 7 -> 3.5 us, the gate/up stream 20 -> 27 us); TP=4
+    // at batch 64 266.7 -> 265.8 us.  Nor do they pay where the matrix is so small that pairs leave half of the
+    // SMs without a CTA and single tiles fill more of them (QKV of that shard at batch 128: 40 CTAs 21 us, 80
+    // CTAs 14.5 us).
+    int mt = a.w8 ? a.w8_tiles : ((planes * a.NB >= 160 && a.N % (2 * kTcTileM) == 0 && a.w_map256) ? 2 : 1);
     if (a.w8 && (!a.w8_codes || !a.scales || mt < 1 || mt > 2))
+        return cudaErrorInvalidValue;
+    TcGeometry g;
+    bool fits = tc_geometry(a, sm_count, mt, g);
+    if (!a.w8 && mt == 2 && (!fits || g.tiles * g.splits * 2 < sm_count)) {
+        TcGeometry one;
+        if (tc_geometry(a, sm_count, 1, one) && (!fits || one.tiles * one.splits > g.tiles * g.splits)) {
+            g = one;
+            mt = 1;
+            fits = true;
+        }
+    }
+    if (!fits)
         return cudaErrorInvalidValue;
     p.w8_codes = static_cast<const uint8_t *>(a.w8_codes);
     p.mt = mt;
     if (mt == 2 && !a.w8)
         p.w_map = *a.w_map256;
-    const int tiles = a.N / (kTcTileM * mt);
-    // int8 weights: a stage holds the codes (half a 16-bit tile) and the activations; the widened tiles
-    // live in tensor memory behind the accumulators (as many as fit, at most four), so the whole of
-    // shared memory is ring: a deep ring is what keeps enough int8 bytes in flight.  One CTA per SM
-    // (tensor memory is per SM).
-    const int stage_bytes = mt * kATileBytes + planes * a.NB * (a.w8 ? 2 * kTcBlockK : kTcBlockK) * 2;
-    // Two CTAs per SM when each needs at most half of tensor memory (accumulators + at least two widened
-    // tiles in 256 columns) and half of shared memory still holds three stages; else one.
-    int w8_slots = 0;
-    bool w8_two = false;
-    if (a.w8) {
-        const int acc = mt * planes * a.NB;
-        w8_two = acc + 2 * mt * 64 <= 256 && (100 * 1024) / stage_bytes >= 3;
-        w8_slots = ((w8_two ? 256 : 512) - acc) / (mt * 64);
-        w8_slots = w8_slots > kTcMaxW8Slots ? kTcMaxW8Slots : w8_slots;
-        if (w8_slots < 2)
-            return cudaErrorInvalidValue;
-    }
+    const int tiles = g.tiles, stage_bytes = g.stage_bytes, per_sm = g.per_sm, splits = g.splits, w8_slots = g.w8_slots;
+    const size_t tile_bytes = g.tile_bytes, smem_cap = g.smem_cap;
+    int stages = g.stages;
     p.w8_slots = w8_slots;
     // (measured: pays for narrow batches - two CTAs per SM, few stages per CTA - and costs ~1 % on wide ones)
-    p.w8_early = a.w8 && w8_two;
-    const int a16_bytes = 0;
+    p.w8_early = a.w8 && g.w8_two;
     p.w8 = a.w8;
     p.wscale = a.scales;
-    // Ring depth, CTAs per SM and cluster splits.  Two CTAs per SM (rings <= 100 KiB) whenever that
-    // leaves >= 4 stages: measured better than one CTA with a ring twice as deep, because the second
-    // CTA streams while the first is in its epilogue.  The grid (tiles x splits) must fit the
-    // co-resident slots (a second wave doubles the kernel); splits are a power of two <= 8 that leave
-    // every rank >= 2 k-blocks.
-    int stages = (200 * 1024 - a16_bytes) / stage_bytes, per_sm = 1;
-    if (a.w8 ? w8_two : (100 * 1024 - a16_bytes) / stage_bytes >= 4) {
-        stages = (100 * 1024 - a16_bytes) / stage_bytes;
-        per_sm = 2;
-    }
-    if (stages > kTcMaxStages) stages = kTcMaxStages;
-    if (stages < 2)
-        return cudaErrorInvalidValue;
-    const int slots = sm_count * per_sm;
-    int splits = 1;
-    while (splits < 8 && tiles * splits * 2 <= slots && p.kblocks / (splits * 2) >= 2) splits *= 2;
-    // Sixteen ranks (a cluster size the device has to be asked for) when even eight leave half of the
-    // SMs without a CTA; only with the bulk hand-over, whose owners may hold a single column.
-    const size_t need16 = (size_t)mt * a.NB * kTcTileM * 4 / 16 * 15;
-    const bool sixteen = splits == 8 && tiles * 16 <= slots && tiles * 8 * 5 <= sm_count * 3 && p.kblocks / 16 >= 2 &&
-                         a.NB % 16 == 0 &&
-                         (size_t)3 * stage_bytes + a16_bytes + need16 + 1024 <= (size_t)(per_sm == 2 ? 108 : 225) * 1024;
-    if (sixteen)
-        splits = 16;
-    p.stages = stages;
     p.splits = splits;
     int cols = 32;
     while (cols < mt * planes * a.NB + w8_slots * mt * 64) cols *= 2;
@@ -1017,38 +978,34 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     p.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)((planes * a.NB) >> 3) << 17) |
               ((uint32_t)(kTcTileM >> 4) << 24);
 
-    // one-sided split-K reduction when the receive area (one partial tile per CTA) is small - every
-    // thread then hands over one or two 16-byte pieces per owner; wide batches keep the pull form,
-    // whose remote accesses are full 128-byte rows - and fits behind the ring
-    const size_t recv_bytes = (size_t)mt * a.NB * kTcTileM * 4;
-    const size_t smem_cap = (per_sm == 2 ? 108 : 225) * 1024;
+    // The split-K hand-over: st.async pieces when the receive area (one partial tile per CTA) is small -
+    // every thread then hands over one or two 16-byte pieces per owner - else bulk copies.
     p.push = 0;
-    if (splits > 1 && splits <= 8 && recv_bytes <= 16 * 1024) {
-        int st = stages;
-        while (st > 3 && (size_t)st * stage_bytes + a16_bytes + recv_bytes + 1024 > smem_cap) --st;
-        if ((size_t)st * stage_bytes + a16_bytes + recv_bytes + 1024 <= smem_cap) {
-            stages = st;
-            p.stages = st;
+    size_t recv_alloc = 0;
+    if (splits > 1 && splits <= 8 && tile_bytes <= 16 * 1024) {
+        while (stages > 3 && (size_t)stages * stage_bytes + tile_bytes + 1024 > smem_cap) --stages;
+        if ((size_t)stages * stage_bytes + tile_bytes + 1024 <= smem_cap) {
             p.push = 1;
+            recv_alloc = tile_bytes;
         }
     }
-    // wide batches: the same by bulk copies (receive area: the other ranks' shares of this rank's columns)
-    size_t recv_alloc = p.push ? recv_bytes : 0;
+    bool in_ring = false;
     if (splits > 1 && !p.push) {
-        const size_t need = recv_bytes / splits * (splits - 1);
-        int st = stages;
-        while (st > 3 && (size_t)st * stage_bytes + a16_bytes + need + 1024 > smem_cap) --st;
-        if ((size_t)st * stage_bytes + a16_bytes + need + 1024 <= smem_cap) {
-            stages = st;
-            p.stages = st;
-            p.push = 2;
-            recv_alloc = need;
+        p.push = 2;
+        const size_t share = tile_bytes / splits * (splits - 1);
+        const int beside = (int)((smem_cap - 1024 - share) / stage_bytes);      // stages that fit beside the area
+        in_ring = beside < 4;
+        if (!in_ring) {
+            stages = stages < beside ? stages : beside;
+            recv_alloc = share;
         }
     }
-    p.recv_off = stages * stage_bytes + a16_bytes;
-    size_t smem = (size_t)stages * stage_bytes + a16_bytes + recv_alloc + 1024;
-    const size_t red_bytes = (size_t)mt * a.NB * kTcTileM * 4 + 1024;
-    if (smem < red_bytes) smem = red_bytes;
+    p.stages = stages;
+    p.recv_off = in_ring ? (int)tile_bytes : stages * stage_bytes;
+    size_t smem = (size_t)stages * stage_bytes + recv_alloc + 1024;
+    const size_t least = in_ring ? g.bulk_bytes(splits) : p.push == 2 ? tile_bytes : 0;
+    if (smem < least + 1024)
+        smem = least + 1024;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(tiles, splits, 1);
     // epilogue warps: 16 when the CTA has the SM to itself and enough column pairs per thread to share,
