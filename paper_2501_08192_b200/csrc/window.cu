@@ -26,6 +26,7 @@ namespace prsv {
 
 constexpr int kWinMaxChunks = 2;   // 8-element chunks per thread
 constexpr int kWinMaxCluster = 8;  // CTAs per row
+constexpr int kWinMaxCtas = 256;   // rows are cut into fewer, larger CTAs where there are many rows
 
 struct WindowParams {
     const uint4 *parts[kMaxParts];
@@ -81,7 +82,8 @@ __device__ __forceinline__ uint4 ld_volatile_v4(const void *p)
 // instructions, which the second finds in the instruction caches.)
 // LEAN, for big batches (hundreds of CTAs): one chunk per thread and the step's input buffers are only
 // hinted into L2 before the wait and loaded after it, so that a CTA holds few registers while it
-// waits - the grid then fits beside the early-launched GEMM CTAs in one wave instead of several.
+// waits - the grid then fits beside the early-launched GEMM CTAs in one wave instead of several.  For the same
+// reason the partial buffers come in bursts of four and the gain last (at most 64 registers; at 42 it spills).
 // COMM: the real communication window - the partial-sum buffers are the ranks' exchange buffers
 // (one-shot all-reduce: every rank reads every rank's buffer through peer-mapped pointers with plain
 // 128-bit loads and adds them in rank order, so all ranks obtain the same bits).  Arrival protocol,
@@ -94,7 +96,7 @@ __device__ __forceinline__ uint4 ld_volatile_v4(const void *p)
 // buffer only after it has passed window B of the same layer, by which time every peer has
 // announced its window-B buffer and therefore finished reading window A.
 template <bool LEAN, bool COMM = false>
-__global__ void __launch_bounds__(512) k_window_reduce_rmsnorm(const __grid_constant__ WindowParams p)
+__global__ void __launch_bounds__(512, LEAN ? 2 : 1) k_window_reduce_rmsnorm(const __grid_constant__ WindowParams p)
 {
     constexpr int kWinMaxChunks = LEAN ? 1 : prsv::kWinMaxChunks;
     const bool RESID_F32 = p.resid_f32 != 0, PART0_F32 = p.part0_f32 != 0;
@@ -106,12 +108,17 @@ __global__ void __launch_bounds__(512) k_window_reduce_rmsnorm(const __grid_cons
     uint4 gn[kWinMaxChunks];
     float ss = 0.f;
 
-    // the gain does not depend on the previous kernel: fetch it before waiting
+    // the gain does not depend on the previous kernel: fetch it before waiting (LEAN: behind the sums, where
+    // its registers are free again)
+    auto load_gain = [&]() {
 #pragma unroll
-    for (int c = 0; c < kWinMaxChunks; ++c) {
-        const int ch = threadIdx.x + c * blockDim.x;
-        gn[c] = ch < chunks ? ld_cached(p.gain + gain_off + ch) : make_uint4(0, 0, 0, 0);
-    }
+        for (int c = 0; c < kWinMaxChunks; ++c) {
+            const int ch = threadIdx.x + c * blockDim.x;
+            gn[c] = ch < chunks ? ld_cached(p.gain + gain_off + ch) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    if constexpr (!LEAN)
+        load_gain();
 
     trace_start(p.trace);
     pdl_launch_dependents();   // the next kernel may start fetching its weights now
@@ -133,7 +140,9 @@ __global__ void __launch_bounds__(512) k_window_reduce_rmsnorm(const __grid_cons
     // unless they are handed over in fp32 by an earlier kernel of the step) do not depend on the
     // previous kernel either: their loads - the only ones that go to HBM - are issued before the
     // wait, up to 8 partial buffers per chunk.
-    uint4 pre[kWinMaxChunks][8], pre_res[kWinMaxChunks];
+    constexpr int kBurst = LEAN ? 4 : 8;
+    uint4 pre[kWinMaxChunks][kBurst], pre_res[kWinMaxChunks];
+    auto load_part = [&](int j, size_t at) { return COMM ? ld_volatile_v4(p.parts[j] + at) : ld_stream(p.parts[j] + at); };
     auto load_inputs = [&]() {
 #pragma unroll
         for (int c = 0; c < kWinMaxChunks; ++c) {
@@ -142,9 +151,9 @@ __global__ void __launch_bounds__(512) k_window_reduce_rmsnorm(const __grid_cons
                 if (!RESID_F32)
                     pre_res[c] = ld_stream(reinterpret_cast<const uint4 *>(p.resid) + row_off + ch);
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
+                for (int j = 0; j < kBurst; ++j)
                     if (j < p.n_parts && !(PART0_F32 && j == 0))
-                        pre[c][j] = COMM ? ld_volatile_v4(p.parts[j] + row_off + ch) : ld_stream(p.parts[j] + row_off + ch);
+                        pre[c][j] = load_part(j, row_off + ch);
             }
         }
     };
@@ -223,21 +232,21 @@ __global__ void __launch_bounds__(512) k_window_reduce_rmsnorm(const __grid_cons
                 v[c][4] += b.x; v[c][5] += b.y; v[c][6] += b.z; v[c][7] += b.w;
             }
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
+            for (int j = 0; j < kBurst; ++j)
                 if (j < p.n_parts && !(PART0_F32 && j == 0)) {
                     const uint4 r = pre[c][j];
                     v[c][0] += bf_lo(r.x); v[c][1] += bf_hi(r.x); v[c][2] += bf_lo(r.y); v[c][3] += bf_hi(r.y);
                     v[c][4] += bf_lo(r.z); v[c][5] += bf_hi(r.z); v[c][6] += bf_lo(r.w); v[c][7] += bf_hi(r.w);
                 }
-            // (more than 8 partial buffers: the rest in bursts of 8)
-            for (int q0 = 8; q0 < p.n_parts; q0 += 8) {
-                uint4 r[8];
+            // (more partial buffers than one burst: the rest in bursts)
+            for (int q0 = kBurst; q0 < p.n_parts; q0 += kBurst) {
+                uint4 r[kBurst];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
+                for (int j = 0; j < kBurst; ++j)
                     if (q0 + j < p.n_parts)
-                        r[j] = ld_stream(p.parts[q0 + j] + row_off + ch);
+                        r[j] = load_part(q0 + j, row_off + ch);
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
+                for (int j = 0; j < kBurst; ++j)
                     if (q0 + j < p.n_parts) {
                         v[c][0] += bf_lo(r[j].x); v[c][1] += bf_hi(r[j].x); v[c][2] += bf_lo(r[j].y); v[c][3] += bf_hi(r[j].y);
                         v[c][4] += bf_lo(r[j].z); v[c][5] += bf_hi(r[j].z); v[c][6] += bf_lo(r[j].w); v[c][7] += bf_hi(r[j].w);
@@ -249,6 +258,8 @@ __global__ void __launch_bounds__(512) k_window_reduce_rmsnorm(const __grid_cons
         }
     }
 
+    if constexpr (LEAN)
+        load_gain();
     // block reduction of the sum of squares (fixed tree: bit-stable run to run)
     __shared__ float warp_sums[32];
     __shared__ float total;
@@ -404,16 +415,21 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
     p.delay_ns = a.delay_ns;
     p.status = a.status;
     // CTAs per row: as many (a power of two, at most 8) as leave every CTA at least 128 threads of
-    // one 8-element chunk each
+    // one 8-element chunk each, and at most 256 CTAs in all: at batch 128 the 1024 CTAs of eight per row took 6 us
+    // to start one after another behind the O projection (two per row: window B 10.7 -> 7.8 us, window A 9.3 -> 6.0,
+    // four 70B-shaped TP=8 layers 378.1 -> 372.6 us; batch 64 and below within 0.1 %).  With few rows more CTAs
+    // are better: at batch 16 four per row cost 1 %, two 2.5 %.
     int cl = 1;
-    while (cl < kWinMaxCluster && (a.H / 8) % (cl * 2) == 0 && (a.H / 8) / (cl * 2) >= 128)
+    while (cl < kWinMaxCluster && (a.H / 8) % (cl * 2) == 0 && (a.H / 8) / (cl * 2) >= 128 &&
+           ((a.H / 8) / cl > 512 || a.B * cl * 2 <= kWinMaxCtas))
         cl *= 2;
     p.cluster = cl;
     const int chunks = a.H / 8 / cl;
-    // LEAN (inputs read after the wait) for big batches, and whenever an input buffer may still be
+    // LEAN (inputs read after the wait, at most 64 registers: 389.1 -> 378.1 us there) for big batches, counted in
+    // threads (32768 = batch 32 at hidden 8192), and whenever an input buffer may still be
     // written by an earlier kernel of the same call
     const bool comm = a.comm_rank >= 0;
-    const bool lean = (a.B * cl > 256 || a.inputs_after_wait || comm) && chunks <= 512;
+    const bool lean = ((long long)a.B * (a.H / 8) > 32768 || a.inputs_after_wait || comm) && chunks <= 512;
     if ((a.inputs_after_wait || comm) && !lean)
         return cudaErrorInvalidValue;
     if (comm && (a.n_parts > 8 || a.part0_is_f32 || a.comm_rank >= a.n_parts))
