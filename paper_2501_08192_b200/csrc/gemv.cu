@@ -19,13 +19,12 @@
 // their L2 latency is paid once per burst).  Grids never exceed what is
 // co-resident (two CTAs per SM); a projection with few row-block groups is split
 // further along k, which shortens the activation slice every CTA reads after the wait.
-// Two arithmetic variants:
-//   - CUDA cores (batch <= 4): 2 x batch fp32 accumulators per lane, finished by
-//     a warp-shuffle reduction over the four lanes that share a row;
-//   - mma.sync m16n8k16 (5 <= batch <= 15): at batch 8 the fp32 FMA pipe would
-//     need ~8 FMAs per weight and co-limit the stream, so the 16x32 tile feeds
-//     warp MMAs with the batch as the n = 8 operand.
-// Activations arrive as hi + lo bf16 planes (x = hi + lo).
+// The 16x32 tile feeds warp MMAs (mma.sync m16n8k16, fp32 accumulation) with the batch as the n = 8
+// operand.  Activations arrive as hi + lo bf16 planes (x = hi + lo): two n tiles per eight batch rows -
+// or, up to batch 4, one tile whose columns 0-3 are the hi plane and 4-7 the lo plane of the same rows.
+// (On the fp32 pipe batch 3 needed ~180 instructions per tile and warp, most of them unpacking and
+// adding the planes, and eight activation loads per lane instead of one, in bursts of two tiles: a layer
+// of hidden 2688, ffn 1824 took 42.9 us at batch 3, now 28.4; the O projection's stream 4.9 -> 1.8 us.)
 // Split-K partial sums are added in a fixed order, so results are bit-stable: warps
 // through shared memory; cluster ranks one-sidedly - ranks 1.. store their sums
 // into rank 0's shared memory (st.async + mbarrier complete_tx) and rank 0
@@ -75,21 +74,20 @@ __device__ __forceinline__ uint32_t s8x2_to_bf16x2(uint32_t w, int shift)
     const int a = (int)(w << (24 - shift)) >> 24, b = (int)(w << (16 - shift)) >> 24;
     return pack_bf16((float)a, (float)b);
 }
-__device__ __forceinline__ float s8_to_f32(uint32_t w, int byte) { return (float)((int)(w << (24 - 8 * byte)) >> 24); }
-
 // RB = 16-row blocks per warp: with two, every activation fragment a warp loads is used for two
 // weight tiles, which halves the activation traffic from L2 (for batch 8 it is otherwise as large
 // as the weight stream itself, and an SM takes in only ~50 GB/s in total).
 // W8: the weights are int8 codes - a 1 KiB tile then covers 16 rows x 64 k (a lane's 16 bytes per row
 // are k = 16 t .. 16 t + 15), the codes are widened to bf16 (exactly) in registers, and every output
 // is multiplied by its row's scale in front of the epilogue.
-template <int NB, bool MMA, int RB, bool W8 = false>
+// PACK (batch <= 4): both planes of the activations in one n tile.
+template <int NB, bool PACK, int RB, bool W8 = false>
 __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid_constant__ GemvParams p)
 {
-    constexpr int NTB = MMA ? NB / 8 : 1;   // n-tiles that cover the batch
-    constexpr int NT = 2 * NTB;             // hi planes then lo planes of the activations
+    constexpr int NTB = PACK ? 1 : NB / 8;  // n-tiles that cover the batch
+    constexpr int NT = PACK ? 1 : 2 * NTB;  // hi planes then lo planes of the activations
     constexpr int XF = W8 ? 2 : 1;          // uint4 of activations per tile, lane and (batch row, plane): 8 k each
-    constexpr int NX = (MMA ? NT : 2 * NB) * XF;   // activation fragments (uint4) per tile
+    constexpr int NX = NT * XF;             // activation fragments (uint4) per tile and lane
     __shared__ float red[kGemvWarps][RB * 16][NB];       // per-warp partials
     __shared__ float cta_part[kGemvWarps * RB][16][NB];  // per-row-block CTA partials (read across the cluster)
     __shared__ uint64_t bars[kGemvWarps][kRingSlots];
@@ -178,25 +176,14 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
     load_epilogue_tables(p.epi, tabs, p.b0, p.B);    // inputs of the step: safe before the wait
     const int xrow = p.K >> 3;                       // uint4 per activation row
     auto load_x = [&](int c, uint4 (&xq)[NX]) {
-        if constexpr (MMA) {
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                const int b = (nt % NTB) * 8 + g;
-                const uint4 *plane = p.x + (nt >= NTB ? p.x_plane : 0);
+        for (int nt = 0; nt < NT; ++nt) {
+            const int b = PACK ? g & 3 : (nt % NTB) * 8 + g;
+            const uint4 *plane = p.x + ((PACK ? g >= 4 : nt >= NTB) ? p.x_plane : 0);
 #pragma unroll
-                for (int f = 0; f < XF; ++f)
-                    xq[nt * XF + f] = b < p.B ? ld_cached(plane + (size_t)(p.b0 + b) * xrow + c * (4 * XF) + t * XF + f)
-                                              : make_uint4(0, 0, 0, 0);
-            }
-        } else {
-#pragma unroll
-            for (int b = 0; b < NB; ++b)
-#pragma unroll
-                for (int f = 0; f < XF; ++f) {
-                    const size_t o = (size_t)(p.b0 + b) * xrow + c * (4 * XF) + t * XF + f;
-                    xq[b * XF + f] = b < p.B ? ld_cached(p.x + o) : make_uint4(0, 0, 0, 0);
-                    xq[(NB + b) * XF + f] = b < p.B ? ld_cached(p.x + p.x_plane + o) : make_uint4(0, 0, 0, 0);
-                }
+            for (int f = 0; f < XF; ++f)
+                xq[nt * XF + f] = b < p.B ? ld_cached(plane + (size_t)(p.b0 + b) * xrow + c * (4 * XF) + t * XF + f)
+                                          : make_uint4(0, 0, 0, 0);
         }
     };
 
@@ -217,43 +204,23 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
     bool ok = true;
     bool push_short = false;      // rank 0: the wait for the other ranks' partial sums ran out
     for (int grp = blockIdx.x; grp < p.groups; grp += gridDim.x) {
-        float acc[RB][MMA ? NT : 2 * NB][MMA ? 4 : 1];
+        float acc[RB][NT][4];
 #pragma unroll
         for (int r = 0; r < RB; ++r)
 #pragma unroll
-            for (int i = 0; i < (MMA ? NT : 2 * NB); ++i)
+            for (int i = 0; i < NT; ++i)
 #pragma unroll
-                for (int j = 0; j < (MMA ? 4 : 1); ++j)
+                for (int j = 0; j < 4; ++j)
                     acc[r][i][j] = 0.f;
 
-        // eight weights of row g (wl) and of row g + 8 (wh) against the same eight k of every batch row
-        auto fma8 = [&](float (&a_)[MMA ? NT : 2 * NB][MMA ? 4 : 1], const float (&l)[8], const float (&h)[8],
-                        const uint4 (&xq)[NX], int f) {
-            if constexpr (!MMA) {
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    const uint4 &xh = xq[b * XF + f], &xl = xq[(NB + b) * XF + f];     // x = hi + lo, exact in fp32
-                    const float x0 = bf_lo(xh.x) + bf_lo(xl.x), x1 = bf_hi(xh.x) + bf_hi(xl.x);
-                    const float x2 = bf_lo(xh.y) + bf_lo(xl.y), x3 = bf_hi(xh.y) + bf_hi(xl.y);
-                    const float x4 = bf_lo(xh.z) + bf_lo(xl.z), x5 = bf_hi(xh.z) + bf_hi(xl.z);
-                    const float x6 = bf_lo(xh.w) + bf_lo(xl.w), x7 = bf_hi(xh.w) + bf_hi(xl.w);
-                    float a = a_[2 * b][0], c = a_[2 * b + 1][0];
-                    a = fmaf(l[0], x0, a); a = fmaf(l[1], x1, a); a = fmaf(l[2], x2, a); a = fmaf(l[3], x3, a);
-                    a = fmaf(l[4], x4, a); a = fmaf(l[5], x5, a); a = fmaf(l[6], x6, a); a = fmaf(l[7], x7, a);
-                    c = fmaf(h[0], x0, c); c = fmaf(h[1], x1, c); c = fmaf(h[2], x2, c); c = fmaf(h[3], x3, c);
-                    c = fmaf(h[4], x4, c); c = fmaf(h[5], x5, c); c = fmaf(h[6], x6, c); c = fmaf(h[7], x7, c);
-                    a_[2 * b][0] = a; a_[2 * b + 1][0] = c;
-                }
-            }
-        };
-        auto compute = [&](float (&a_)[MMA ? NT : 2 * NB][MMA ? 4 : 1], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
-            if constexpr (MMA && !W8) {
+        auto compute = [&](float (&a_)[NT][4], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
+            if constexpr (!W8) {
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) {
                     mma_bf16_16816(a_[nt], wl.x, wh.x, wl.y, wh.y, xq[nt].x, xq[nt].y);
                     mma_bf16_16816(a_[nt], wl.z, wh.z, wl.w, wh.w, xq[nt].z, xq[nt].w);
                 }
-            } else if constexpr (MMA && W8) {
+            } else {
                 // word j of wl / wh = codes of k = 16 t + 4 j .. + 3: one m16n8k16 MMA per word
                 const uint32_t lw[4] = {wl.x, wl.y, wl.z, wl.w}, hw[4] = {wh.x, wh.y, wh.z, wh.w};
 #pragma unroll
@@ -265,22 +232,6 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                         const uint4 &xv = xq[nt * 2 + (j >> 1)];
                         mma_bf16_16816(a_[nt], a0, a1, a2, a3, (j & 1) ? xv.z : xv.x, (j & 1) ? xv.w : xv.y);
                     }
-                }
-            } else if constexpr (!W8) {
-                const float l[8] = {bf_lo(wl.x), bf_hi(wl.x), bf_lo(wl.y), bf_hi(wl.y), bf_lo(wl.z), bf_hi(wl.z), bf_lo(wl.w), bf_hi(wl.w)};
-                const float h[8] = {bf_lo(wh.x), bf_hi(wh.x), bf_lo(wh.y), bf_hi(wh.y), bf_lo(wh.z), bf_hi(wh.z), bf_lo(wh.w), bf_hi(wh.w)};
-                fma8(a_, l, h, xq, 0);
-            } else {
-                const uint32_t lw[4] = {wl.x, wl.y, wl.z, wl.w}, hw[4] = {wh.x, wh.y, wh.z, wh.w};
-#pragma unroll
-                for (int f = 0; f < 2; ++f) {
-                    float l[8], h[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        l[i] = s8_to_f32(lw[2 * f + (i >> 2)], i & 3);
-                        h[i] = s8_to_f32(hw[2 * f + (i >> 2)], i & 3);
-                    }
-                    fma8(a_, l, h, xq, f);
                 }
             }
         };
@@ -333,22 +284,21 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
         // ---- warp partial -> shared memory: red[warp][row block of the warp * 16 + row][b]
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
-            if constexpr (MMA) {
+            if constexpr (PACK) {
+                // columns 2t, 2t + 1: lanes t < 2 hold the hi plane's products, lanes t + 2 the lo plane's
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float v = acc[r][0][j] + __shfl_xor_sync(0xffffffffu, acc[r][0][j], 2);
+                    if (t < 2)
+                        red[warp][r * 16 + g + 8 * (j >> 1)][2 * t + (j & 1)] = v;
+                }
+            } else {
 #pragma unroll
                 for (int nt = 0; nt < NTB; ++nt) {
                     red[warp][r * 16 + g][nt * 8 + 2 * t] = acc[r][nt][0] + acc[r][NTB + nt][0];
                     red[warp][r * 16 + g][nt * 8 + 2 * t + 1] = acc[r][nt][1] + acc[r][NTB + nt][1];
                     red[warp][r * 16 + g + 8][nt * 8 + 2 * t] = acc[r][nt][2] + acc[r][NTB + nt][2];
                     red[warp][r * 16 + g + 8][nt * 8 + 2 * t + 1] = acc[r][nt][3] + acc[r][NTB + nt][3];
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 2 * NB; ++i) {
-                    float v = acc[r][i][0];
-                    v += __shfl_xor_sync(0xffffffffu, v, 1);
-                    v += __shfl_xor_sync(0xffffffffu, v, 2);
-                    if (t == 0)
-                        red[warp][r * 16 + g + 8 * (i & 1)][i >> 1] = v;
                 }
             }
         }
@@ -460,12 +410,12 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
     trace_end(p.trace);
 }
 
-template <int NB, bool MMA, int RB, bool W8>
+template <int NB, bool PACK, int RB, bool W8>
 static cudaError_t launch_variant(GemvParams &p, int sm_count, int pdl, cudaStream_t s)
 {
     static PerDeviceSize smem_limit;      // per instantiation and device
     {
-        cudaError_t e = ensure_dynamic_smem(k_gemv_splitk<NB, MMA, RB, W8>, smem_limit, kGemvSmemBytes + 32 * 1024 + 128);
+        cudaError_t e = ensure_dynamic_smem(k_gemv_splitk<NB, PACK, RB, W8>, smem_limit, kGemvSmemBytes + 32 * 1024 + 128);
         if (e != cudaSuccess)
             return e;
     }
@@ -523,7 +473,7 @@ static cudaError_t launch_variant(GemvParams &p, int sm_count, int pdl, cudaStre
     }
     cfg.attrs = at;
     cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, k_gemv_splitk<NB, MMA, RB, W8>, p);
+    return cudaLaunchKernelEx(&cfg, k_gemv_splitk<NB, PACK, RB, W8>, p);
 }
 
 template <bool W8>
@@ -531,12 +481,9 @@ static cudaError_t launch_by_batch(GemvParams &p, int B, int sm_count, int pdl, 
 {
     // two row blocks per warp whenever the matrix has enough row blocks to still fill the SMs
     const bool two = p.row_blocks % 2 == 0 && p.row_blocks >= 32;
-    if (B == 1) return two ? launch_variant<1, false, 2, W8>(p, sm_count, pdl, s) : launch_variant<1, false, 1, W8>(p, sm_count, pdl, s);
-    if (B == 2) return two ? launch_variant<2, false, 2, W8>(p, sm_count, pdl, s) : launch_variant<2, false, 1, W8>(p, sm_count, pdl, s);
-    // (int8 weights double the activation fragments a lane holds per tile: batch 3-4 takes the MMA form there)
-    if (B <= 4 && !W8) return two ? launch_variant<4, false, 2, false>(p, sm_count, pdl, s) : launch_variant<4, false, 1, false>(p, sm_count, pdl, s);
-    if (B <= 8) return two ? launch_variant<8, true, 2, W8>(p, sm_count, pdl, s) : launch_variant<8, true, 1, W8>(p, sm_count, pdl, s);
-    return two ? launch_variant<16, true, 2, W8>(p, sm_count, pdl, s) : launch_variant<16, true, 1, W8>(p, sm_count, pdl, s);
+    if (B <= 4) return two ? launch_variant<4, true, 2, W8>(p, sm_count, pdl, s) : launch_variant<4, true, 1, W8>(p, sm_count, pdl, s);
+    if (B <= 8) return two ? launch_variant<8, false, 2, W8>(p, sm_count, pdl, s) : launch_variant<8, false, 1, W8>(p, sm_count, pdl, s);
+    return two ? launch_variant<16, false, 2, W8>(p, sm_count, pdl, s) : launch_variant<16, false, 1, W8>(p, sm_count, pdl, s);
 }
 
 cudaError_t launch_gemv(const GemvArgs &a, int sm_count, cudaStream_t s)
