@@ -10,11 +10,8 @@
 // tile) x one slice of k.
 //   warp 0 (+ lane 0 of the first one or two epilogue warps): TMA producers - W tile (128 or 256 rows
 //               x 64, 128B swizzle) and x tile (2 NB x 64) into a multi-stage shared-memory ring,
-//               mbarrier full/empty.  One thread can start a bulk copy only every ~0.4 us whatever
-//               its size (measured: a single issuing thread moves 43 GB/s in 16 KiB copies, 131 GB/s
-//               in 64 KiB copies, and threads of different warps add up), so one producer alone caps
-//               a CTA near 50-70 GB/s - below an SM's share of HBM; the ring's stage uses are
-//               therefore dealt round-robin to several issuing threads
+//               mbarrier full/empty; the ring's stage uses are dealt round-robin to the issuing threads
+//               (three instead of one measured < 1 %)
 //   warp 1    : allocates TMEM, issues tcgen05.mma (kind::f16, bf16 in, fp32
 //               accumulate in TMEM), tcgen05.commit frees ring slots
 //   warps 2.. : epilogue (8 or 16 warps) - tcgen05.ld the accumulator (lane = output row; the warps of
@@ -859,6 +856,7 @@ int gemm_tc_w8_tiles(int NB, int N, int x_fp16)
     return (N % (2 * kTcTileM) == 0 && 2 * acc + 2 * 2 * 64 <= 512) ? 2 : 1;
 }
 
+namespace {
 // How a GEMM is cut into CTAs when each takes `mt` weight tiles.
 struct TcGeometry {
     int tiles, stage_bytes, stages, per_sm, splits, w8_slots;
@@ -867,7 +865,7 @@ struct TcGeometry {
     // bulk hand-over: the staged tiles and the other ranks' shares of this rank's columns
     size_t bulk_bytes(int sp) const { return tile_bytes + tile_bytes / sp * (sp - 1); }
 };
-static bool tc_geometry(const GemmTcArgs &a, int sm_count, int mt, TcGeometry &g)
+bool tc_geometry(const GemmTcArgs &a, int sm_count, int mt, TcGeometry &g)
 {
     const int planes = a.x_fp16 == 1 ? 1 : 2;
     const int kblocks = a.K / (a.w8 ? 2 * kTcBlockK : kTcBlockK);
@@ -916,6 +914,7 @@ static bool tc_geometry(const GemmTcArgs &a, int sm_count, int mt, TcGeometry &g
         g.splits = 16;
     return true;
 }
+}  // namespace
 
 cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
 {
