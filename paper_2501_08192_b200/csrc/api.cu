@@ -340,7 +340,7 @@ struct StepPlan {
     uint64_t kv_bytes, alg_bytes;
     bool pf_a, pf_b;
     int pdl;
-    int attn_grid, attn_tpi, attn_items_per_stream;
+    int attn_grid, attn_tpi, attn_items_per_stream, attn_cluster;
 };
 
 int check_step(preserve_layer *L, const preserve_step_io_t *io, StepPtrs *sp)
@@ -496,6 +496,7 @@ void plan_step(preserve_layer *L, const StepPtrs &sp, StepPlan *pl)
     pl->pf_b = (L->only == -1 || L->only == -3) && pl->planned[1][0] + pl->planned[1][1] > 0;
     plan_attention(sp.ctx_len_host, B, c.n_kv_heads, L->sm_count, &pl->attn_grid, &pl->attn_tpi,
                    L->kv8 ? attention_kv8_stages() : 3, L->kv8 ? 3.0 : 1.5);
+    pl->attn_cluster = plan_attention_cluster(sp.ctx_len_host, B, c.n_q_heads, c.n_kv_heads, L->sm_count);
     pl->attn_items_per_stream = (int)((max_tiles_seq + pl->attn_tpi - 1) / pl->attn_tpi);
     // (the merge kernel sizes its CTAs from this, between 4 and 32 warps: clamp here so that the
     // number that enters the graph signature changes as rarely as the launch does)
@@ -669,6 +670,7 @@ int enqueue_step(preserve_layer *L, const StepPtrs &sp, const StepPlan &pl, bool
         a.o_fp16 = L->tensor_path ? 1 : 0;
         a.ctx_len = sp.ctx_len;
         a.B = B; a.nq = c.n_q_heads; a.nkv = c.n_kv_heads; a.cap = cap;
+        a.cluster = pl.attn_cluster;
         a.grid = pl.attn_grid;
         a.tiles_per_item = pl.attn_tpi;
         a.max_items_per_stream = pl.attn_items_per_stream;
@@ -845,7 +847,7 @@ void step_signature(const preserve_layer *L, const StepPtrs &sp, const StepPlan 
     put((uint64_t)L->window_delay_ns | (uint64_t)L->pf_chunk << 32);
     put((uint64_t)L->prefetch_ctas);
     put((uint64_t)pl.attn_grid | (uint64_t)pl.attn_tpi << 32);
-    put((uint64_t)pl.attn_items_per_stream);
+    put((uint64_t)pl.attn_items_per_stream | (uint64_t)pl.attn_cluster << 32);
     putp(L->comm);
     putp(L->ext_attn_sum);
 }

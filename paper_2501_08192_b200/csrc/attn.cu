@@ -22,6 +22,7 @@
 // k_attn_merge then combines the partials of a sequence in fixed order.  Nothing
 // depends on timing, so results are bit-stable.
 #include <cstdlib>
+#include <type_traits>
 
 #include "../../include/preserve.h"
 #include <cuda_fp16.h>
@@ -45,6 +46,7 @@ struct AttnParams {
     int B, nq, nkv, G, cap;
     int tiles_per_item;
     int max_items;
+    int cl;                 // CTAs per cluster (CL)
     float scale_log2;       // log2(e) / sqrt(d)
     float *part_o;          // [item][G][d] CTA partials (unnormalised, relative to the item's max)
     float *part_ml;         // [item][G][2] (max, sum)
@@ -76,11 +78,13 @@ __device__ __forceinline__ float *comb_row(uint8_t *stage, int w, int r)
 __device__ __forceinline__ int comb_col2(int r, int c) { return c ^ ((r & 3) << 2); }
 
 // NARROW: groups of up to 8 query heads (keys as MMA rows in the QK product), else up to 16.
-template <bool NARROW>
+// CL: one cluster per (sequence, kv head), the partials merged inside (attn_common.cuh).
+template <bool NARROW, bool CL = false>
 __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const __grid_constant__ AttnParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     AttnSmem &sm = *reinterpret_cast<AttnSmem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ typename std::conditional<CL, ClusterRecv, int>::type rc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int streams = p.B * p.nkv;
 
@@ -95,13 +99,22 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
     }
     trace_start(p.trace);
     pdl_launch_dependents();
-    build_item_table(p, sm.item_base);       // sequence lengths are inputs of the step: no dependency
-    __syncthreads();
+    if constexpr (CL) {
+        if (threadIdx.x == 0)
+            cluster_recv_init(rc, p.G, p.cl);
+        if (blockIdx.x == 0 && warp == 0)
+            cluster_check_items(p.ctx_len, p.B, p.nkv, p.tiles_per_item, p.max_items, p.status);
+        __syncthreads();
+        cluster_arrive_relaxed();
+    } else {
+        build_item_table(p, sm.item_base);       // sequence lengths are inputs of the step: no dependency
+        __syncthreads();
+    }
     // The partial buffers hold max_items entries, sized from the host copy of the lengths.  Device
     // lengths that disagree with it must not write past them: the surplus items are dropped (the
     // result is then wrong, and the status word says why).
-    int total_items = sm.item_base[streams];
-    if (total_items > p.max_items) {
+    int total_items = CL ? (int)gridDim.x : sm.item_base[streams];
+    if (!CL && total_items > p.max_items) {
         total_items = p.max_items;
         if (threadIdx.x == 0)
             atomicCAS(p.status, ST_OK, ST_ITEMS_OVERFLOW);
@@ -117,11 +130,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
             uint32_t it = 0;
             bool ok = true, waited = false;
             for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-                const int sidx = find_stream(sm.item_base, streams, item);
-                const int chunk = item - sm.item_base[sidx];
+                const int sidx = CL ? item / p.cl : find_stream(sm.item_base, streams, item);
+                const int chunk = CL ? item % p.cl : item - sm.item_base[sidx];
                 const int nt = tiles_of(p.ctx_len[sidx / p.nkv]);
-                const int t0 = chunk * p.tiles_per_item;
-                const int t1 = min(nt, t0 + p.tiles_per_item);
+                const int t0 = CL ? cluster_first_tile(nt, chunk, p.cl) : chunk * p.tiles_per_item;
+                const int t1 = CL ? cluster_first_tile(nt, chunk + 1, p.cl) : min(nt, t0 + p.tiles_per_item);
                 for (int tile = t0; tile < t1; ++tile, ++it) {
                     const int st = it % kStages;
                     const uint32_t ph = (it / kStages) & 1;
@@ -141,6 +154,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
                 }
             }
         }
+        if constexpr (CL) {
+            __syncwarp();
+            cluster_wait();
+        }
         return;
     }
 
@@ -153,13 +170,13 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
     pdl_wait();    // q comes from the QKV projection
     trace_waited(p.trace);
     for (int item = blockIdx.x; item < total_items; item += gridDim.x) {
-        const int sidx = find_stream(sm.item_base, streams, item);
+        const int sidx = CL ? item / p.cl : find_stream(sm.item_base, streams, item);
         const int b = sidx / p.nkv, kvh = sidx % p.nkv;
-        const int chunk = item - sm.item_base[sidx];
+        const int chunk = CL ? item % p.cl : item - sm.item_base[sidx];
         const int n_keys = p.ctx_len[b] + 1;
         const int nt = tiles_of(p.ctx_len[b]);
-        const int t0 = chunk * p.tiles_per_item;
-        const int t1 = min(nt, t0 + p.tiles_per_item);
+        const int t0 = CL ? cluster_first_tile(nt, chunk, p.cl) : chunk * p.tiles_per_item;
+        const int t1 = CL ? cluster_first_tile(nt, chunk + 1, p.cl) : min(nt, t0 + p.tiles_per_item);
 
         constexpr bool narrow = NARROW;
         // Q fragments: rows = query heads of the group (zero beyond G)
@@ -409,7 +426,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
             }
         }
         consumer_barrier();
-        const int n_items_stream = sm.item_base[sidx + 1] - sm.item_base[sidx];
+        auto store_o = [&](int r, int d, float o0, float o1) {
+            const size_t oi = ((size_t)b * p.nq + (size_t)kvh * p.G + r) * kHeadDim + d;
+            if (p.o_fp16) {
+                *reinterpret_cast<__half2 *>(reinterpret_cast<__half *>(p.o_out) + oi) = __floats2half2_rn(o0, o1);
+            } else {
+                uint32_t hi, lo;
+                split_bf16x2(o0, o1, hi, lo);
+                *reinterpret_cast<uint32_t *>(p.o_out + oi) = hi;
+                *reinterpret_cast<uint32_t *>(p.o_out + p.o_plane + oi) = lo;
+            }
+        };
+        const int n_items_stream = CL ? 0 : sm.item_base[sidx + 1] - sm.item_base[sidx];
+        if constexpr (CL)
+            cluster_wait();          // (the arrival in the prologue: every rank's receive barrier exists)
         // two head dims per consumer thread, the heads of one parity per half of the threads
         const int d2 = threadIdx.x & 63;
         for (int r = threadIdx.x >> 6; r < p.G; r += 2) {
@@ -428,23 +458,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
                 acc.y += v.y * c;
                 lsum += sm.comb_ml[w][r][1] * c;
             }
-            if (n_items_stream == 1) {
+            if constexpr (CL) {
+                cluster_send(rc, p.G, p.cl, chunk, r, d2, acc, M, lsum);
+            } else if (n_items_stream == 1) {
                 // the item is the whole sequence: finish here
-                const float o0 = acc.x / lsum, o1 = acc.y / lsum;
-                const size_t oi = ((size_t)b * p.nq + (size_t)kvh * p.G + r) * kHeadDim + 2 * d2;
-                if (p.o_fp16) {
-                    *reinterpret_cast<__half2 *>(reinterpret_cast<__half *>(p.o_out) + oi) = __floats2half2_rn(o0, o1);
-                } else {
-                    uint32_t hi, lo;
-                    split_bf16x2(o0, o1, hi, lo);
-                    *reinterpret_cast<uint32_t *>(p.o_out + oi) = hi;
-                    *reinterpret_cast<uint32_t *>(p.o_out + p.o_plane + oi) = lo;
-                }
+                store_o(r, 2 * d2, acc.x / lsum, acc.y / lsum);
             } else {
                 *reinterpret_cast<float2 *>(p.part_o + ((size_t)item * p.G + r) * kHeadDim + 2 * d2) = acc;
                 if (d2 == 0)
                     *reinterpret_cast<float2 *>(p.part_ml + ((size_t)item * p.G + r) * 2) = make_float2(M, lsum);
             }
+        }
+        if constexpr (CL) {
+            cluster_finish(rc, p.G, p.cl, chunk, threadIdx.x, p.status, p.trace, store_o);
+            return;
         }
         consumer_barrier();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -603,6 +630,26 @@ void plan_attention(const int32_t *ctx_len_host, int batch, int nkv, int sm_coun
     *tiles_per_item = best;
 }
 
+int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count)
+{
+    if (nq / nkv > kMaxClusterGroup)
+        return 0;
+    // Eight CTAs per (sequence, kv head), or four where eight would exceed one CTA per SM, and at most four tiles
+    // each (2047 or 1023 cached tokens).  The merge kernel's launch, hand-over and read of the partials go:
+    // us per layer, items / clusters: batch 1, ctx 512 24.5 / 24.2; batch 3, ctx up to 777 28.5 / 27.6; batch 7,
+    // ctx 160 72.8 / 70.6; batch 10, ctx up to 1084 46.3 / 45.0.  Sixteen CTAs lose: they only find a place together once
+    // the kernel in front has ended (batch 1: 24.6), and beyond four tiles the items' finer split wins
+    // (batch 8, ctx 4096, sixteen CTAs of five tiles 33.4 against 32.4).
+    int cl = 8;
+    while (cl >= 4 && batch * nkv * cl > sm_count) cl /= 2;
+    if (cl < 4)
+        return 0;
+    for (int b = 0; b < batch; ++b)
+        if ((ctx_len_host[b] + 1 + kTileKeys - 1) / kTileKeys > 4 * cl)
+            return 0;
+    return cl;
+}
+
 cudaError_t launch_attention(const AttnArgs &a, cudaStream_t s)
 {
     if (a.B * a.nkv > kMaxStreams || a.nq % a.nkv || a.nq / a.nkv > 16)
@@ -625,9 +672,17 @@ cudaError_t launch_attention(const AttnArgs &a, cudaStream_t s)
     p.status = a.status;
     p.trace = a.trace;
     p.inject = a.inject;
+    p.cl = a.cluster;
 
-    const size_t smem = attn_smem_bytes(a.B * a.nkv);
-    if (!a.kv8) {
+    const size_t smem = attn_smem_bytes(a.cluster ? 0 : a.B * a.nkv);
+    if (a.cluster && (p.G > kMaxClusterGroup || a.cluster > kMaxAttnCluster || (a.cluster & (a.cluster - 1))))
+        return cudaErrorInvalidValue;
+    if (!a.kv8 && a.cluster) {
+        static PerDeviceSize lim_cl;
+        cudaError_t e = ensure_dynamic_smem(k_attn_decode_splitkv<true, true>, lim_cl, smem);
+        if (e != cudaSuccess)
+            return e;
+    } else if (!a.kv8) {
         static PerDeviceSize lim_narrow, lim_wide;      // per device: the attribute belongs to one device
         cudaError_t e = ensure_dynamic_smem(k_attn_decode_splitkv<true>, lim_narrow, attn_smem_bytes(kMaxStreams));
         if (e == cudaSuccess)
@@ -635,21 +690,29 @@ cudaError_t launch_attention(const AttnArgs &a, cudaStream_t s)
         if (e != cudaSuccess)
             return e;
     }
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.grid);
+    cfg.gridDim = dim3(a.cluster ? a.B * a.nkv * a.cluster : a.grid);
     cfg.blockDim = dim3(kAttnThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = pdl_attr(at, a.pdl);
+    if (a.cluster) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[cfg.numAttrs].val.clusterDim.x = a.cluster;
+        at[cfg.numAttrs].val.clusterDim.y = 1;
+        at[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
     const int phases = a.phases ? a.phases : 3;
     cudaError_t e = cudaSuccess;
     if ((phases & 1) && a.kv8)
         e = launch_attention_kv8_kernel(a, cfg);
     else if (phases & 1)
-        e = p.G <= 8 ? cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv<true>, p)
-                     : cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv<false>, p);
+        e = a.cluster ? cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv<true, true>, p)
+            : p.G <= 8 ? cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv<true>, p)
+                       : cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv<false>, p);
     if (e != cudaSuccess)
         return e;
     if (a.mid_event) {
@@ -657,7 +720,7 @@ cudaError_t launch_attention(const AttnArgs &a, cudaStream_t s)
         if (e != cudaSuccess)
             return e;
     }
-    if (!(phases & 2))
+    if (!(phases & 2) || a.cluster)       // (clusters merge inside the kernel)
         return cudaSuccess;
     // one warp per item partial of the longest sequence (at least the four that write the head dims)
     int warps = a.max_items_per_stream < 4 ? 4 : (a.max_items_per_stream > kMergeMaxWarps ? kMergeMaxWarps

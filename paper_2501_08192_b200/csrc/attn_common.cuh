@@ -59,4 +59,94 @@ __device__ __forceinline__ int find_stream(const int *item_base, int streams, in
     return lo;
 }
 
+// ---- Short caches: one cluster per (sequence, kv head) instead of work items and a merge kernel.  Rank r of
+// the cluster takes the r-th of `cl` equal runs of the sequence's tiles; the ranks' partials meet by one-sided
+// stores (rank q finishes elements [q L, (q + 1) L) of the group's G x 128 outputs, L = G * 128 / cl), and the
+// result leaves the kernel merged.
+constexpr int kMaxAttnCluster = 8;
+constexpr int kMaxClusterGroup = 8;
+struct ClusterRecv {
+    float o[kMaxClusterGroup * 128];                          // [source rank][L]
+    float ml[kMaxAttnCluster * kMaxClusterGroup][2];          // [source rank][head]
+    uint64_t bar;
+    int gave_up;
+};
+__device__ __forceinline__ void cluster_recv_init(ClusterRecv &rc, int G, int cl)      // one thread, before the CTA's barrier
+{
+    mbar_init(&rc.bar, 1);
+    mbar_fence_init();
+    mbar_expect_tx(&rc.bar, (uint32_t)(G * 128 * 4 + cl * G * 8));
+    rc.gave_up = 0;
+}
+// balanced runs, the longer ones first (rank 0 is never empty)
+__device__ __forceinline__ int cluster_first_tile(int nt, int rank, int cl) { return (nt * rank + cl - 1) / cl; }
+// head dims 2 * d2, 2 * d2 + 1 of head r, relative to this rank's maximum M with weight sum l
+__device__ __forceinline__ void cluster_send(ClusterRecv &rc, int G, int cl, int rank, int r, int d2, float2 acc, float M, float l)
+{
+    const int L = G * 128 / cl, e = r * 128 + 2 * d2, q = e / L;
+    st_async_v2(cluster_map(&rc.o[rank * L + e - q * L], q), acc, cluster_map(&rc.bar, q));
+    if (d2 < cl)
+        st_async_v2(cluster_map(rc.ml[rank * G + r], d2), make_float2(M, l), cluster_map(&rc.bar, d2));
+}
+// Waits for every rank's share of this rank's elements, adds them in rank order and hands each finished pair to
+// store(head, first dim, value, value).  Called by all consumer threads (tid < 128).  In the timeline this part is the
+// merge: the attention's slots end where it begins.
+template <typename Store>
+__device__ __forceinline__ void cluster_finish(ClusterRecv &rc, int G, int cl, int rank, int tid, int *status, long long *trace, Store store)
+{
+    long long *tr = trace ? trace + kTraceSlots : nullptr;
+    trace_end(trace);
+    trace_start(tr);
+    if (!mbar_wait(&rc.bar, 0, status, ST_TIMEOUT_FULL)) {
+        *reinterpret_cast<volatile int *>(&rc.gave_up) = 1;
+        trace_waited(tr);
+    } else {
+        trace_waited(tr);
+        const int L = G * 128 / cl;
+        for (int i = 2 * tid; i < L; i += 2 * kConsumerWarps * 32) {
+            const int e = rank * L + i, r = e >> 7;
+            float M = -INFINITY;
+            for (int c = 0; c < cl; ++c)
+                M = fmaxf(M, rc.ml[c * G + r][0]);
+            float2 acc = make_float2(0.f, 0.f);
+            float l = 0.f;
+            for (int c = 0; c < cl; ++c) {                    // rank order
+                const float mc = rc.ml[c * G + r][0];
+                const float w = mc == -INFINITY ? 0.f : exp2f(mc - M);
+                const float2 v = *reinterpret_cast<const float2 *>(&rc.o[c * L + i]);
+                acc.x += v.x * w;
+                acc.y += v.y * w;
+                l += rc.ml[c * G + r][1] * w;
+            }
+            store(r, e & 127, acc.x / l, acc.y / l);
+        }
+    }
+    // A CTA that gave up may be about to leave before every peer has stored into it, and a store into the shared
+    // memory of a CTA that has exited is a fault: it stays until every peer has left or reached this point
+    // too, then gives the stores in flight a bounded time to land.  (The barrier counts only threads that have
+    // not exited; a CTA that received everything simply leaves.)
+    consumer_barrier();
+    if (*reinterpret_cast<volatile int *>(&rc.gave_up)) {
+        cluster_arrive_relaxed();
+        cluster_wait();
+        if (tid == 0)
+            mbar_wait(&rc.bar, 0, status, ST_TIMEOUT_FULL);
+        consumer_barrier();
+    }
+    trace_end(tr);
+}
+// The overflow report of the item form: device lengths that need more items than the plan has room for are
+// reported although this form has no buffer they could overrun.  (One warp of one CTA.)
+__device__ __forceinline__ void cluster_check_items(const int *ctx_len, int B, int nkv, int tiles_per_item, int max_items, int *status)
+{
+    int n = 0;
+    for (int b = threadIdx.x & 31; b < B; b += 32)
+        n += nkv * ((tiles_of(ctx_len[b]) + tiles_per_item - 1) / tiles_per_item);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        n += __shfl_xor_sync(0xffffffffu, n, o);
+    if (n > max_items && (threadIdx.x & 31) == 0)
+        atomicCAS(status, ST_OK, ST_ITEMS_OVERFLOW);
+}
+
 }  // namespace prsv

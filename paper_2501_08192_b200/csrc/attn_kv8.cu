@@ -26,6 +26,7 @@
 //     codes and scales to the cache for the following steps;
 //   - groups of at most 8 query heads per KV head (keys as MMA rows).
 #include <cuda_fp16.h>
+#include <type_traits>
 
 #include "../../include/preserve.h"
 #include "attn_common.cuh"
@@ -58,6 +59,7 @@ struct AttnKv8Params {
     int B, nq, nkv, G, cap, scale_cap;
     int tiles_per_item;
     int max_items;
+    int cl;                 // CTAs per cluster (CL)
     float scale_log2;
     float *part_o;
     float *part_ml;
@@ -135,10 +137,12 @@ __device__ __forceinline__ uint32_t quantize_row_128(float4 u, float &scale)
     return code(u.x) | (code(u.y) << 8) | (code(u.z) << 16) | (code(u.w) << 24);
 }
 
+template <bool CL>
 __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(const __grid_constant__ AttnKv8Params p)
 {
     extern __shared__ uint8_t smem_raw[];
     AttnKv8Smem &sm = *reinterpret_cast<AttnKv8Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ typename std::conditional<CL, ClusterRecv, int>::type rc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int streams = p.B * p.nkv;
 
@@ -153,10 +157,19 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(con
     }
     trace_start(p.trace);
     pdl_launch_dependents();
-    build_item_table(p, sm.item_base);       // sequence lengths are inputs of the step: no dependency
-    __syncthreads();
-    int total_items = sm.item_base[streams];
-    if (total_items > p.max_items) {         // device lengths disagree with the host copy: never write past the partials
+    if constexpr (CL) {
+        if (threadIdx.x == 0)
+            cluster_recv_init(rc, p.G, p.cl);
+        if (blockIdx.x == 0 && warp == 0)
+            cluster_check_items(p.ctx_len, p.B, p.nkv, p.tiles_per_item, p.max_items, p.status);
+        __syncthreads();
+        cluster_arrive_relaxed();
+    } else {
+        build_item_table(p, sm.item_base);       // sequence lengths are inputs of the step: no dependency
+        __syncthreads();
+    }
+    int total_items = CL ? (int)gridDim.x : sm.item_base[streams];
+    if (!CL && total_items > p.max_items) {         // device lengths disagree with the host copy: never write past the partials
         total_items = p.max_items;
         if (threadIdx.x == 0)
             atomicCAS(p.status, ST_OK, ST_ITEMS_OVERFLOW);
@@ -173,11 +186,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(con
             uint32_t it = 0;
             bool ok = true, waited = false;
             for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-                const int sidx = find_stream(sm.item_base, streams, item);
-                const int chunk = item - sm.item_base[sidx];
+                const int sidx = CL ? item / p.cl : find_stream(sm.item_base, streams, item);
+                const int chunk = CL ? item % p.cl : item - sm.item_base[sidx];
                 const int nt = tiles_of(p.ctx_len[sidx / p.nkv]);
-                const int t0 = chunk * p.tiles_per_item;
-                const int t1 = min(nt, t0 + p.tiles_per_item);
+                const int t0 = CL ? cluster_first_tile(nt, chunk, p.cl) : chunk * p.tiles_per_item;
+                const int t1 = CL ? cluster_first_tile(nt, chunk + 1, p.cl) : min(nt, t0 + p.tiles_per_item);
                 for (int tile = t0; tile < t1; ++tile, ++it) {
                     const int st = it % kStages8;
                     const uint32_t ph = (it / kStages8) & 1;
@@ -198,6 +211,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(con
                 }
             }
         }
+        if constexpr (CL) {
+            __syncwarp();
+            cluster_wait();
+        }
         return;
     }
 
@@ -213,13 +230,13 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(con
     const int lkey = warp * 16 + (((lane >> 3) & 1) << 3) + (lane & 7);
     const int lsw = lkey & 7, lch = lane >> 4;
     for (int item = blockIdx.x; item < total_items; item += gridDim.x) {
-        const int sidx = find_stream(sm.item_base, streams, item);
+        const int sidx = CL ? item / p.cl : find_stream(sm.item_base, streams, item);
         const int b = sidx / p.nkv, kvh = sidx % p.nkv;
-        const int chunk = item - sm.item_base[sidx];
+        const int chunk = CL ? item % p.cl : item - sm.item_base[sidx];
         const int n_keys = p.ctx_len[b] + 1;
         const int nt = tiles_of(p.ctx_len[b]);
-        const int t0 = chunk * p.tiles_per_item;
-        const int t1 = min(nt, t0 + p.tiles_per_item);
+        const int t0 = CL ? cluster_first_tile(nt, chunk, p.cl) : chunk * p.tiles_per_item;
+        const int t1 = CL ? cluster_first_tile(nt, chunk + 1, p.cl) : min(nt, t0 + p.tiles_per_item);
 
         // Q fragments (the B operand of S^T = K Q^T), query head g, as one fp16 plane.  The k index
         // of the MMA runs over the head dims in the order the int8 ldmatrix delivers them: for the
@@ -429,7 +446,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(con
             }
         }
         consumer_barrier();
-        const int n_items_stream = sm.item_base[sidx + 1] - sm.item_base[sidx];
+        auto store_o = [&](int r, int d, float o0, float o1) {
+            const size_t oi = ((size_t)b * p.nq + (size_t)kvh * p.G + r) * kHeadDim + d;
+            if (p.o_fp16) {
+                *reinterpret_cast<__half2 *>(reinterpret_cast<__half *>(p.o_out) + oi) = __floats2half2_rn(o0, o1);
+            } else {
+                uint32_t hi, lo;
+                split_bf16x2(o0, o1, hi, lo);
+                *reinterpret_cast<uint32_t *>(p.o_out + oi) = hi;
+                *reinterpret_cast<uint32_t *>(p.o_out + p.o_plane + oi) = lo;
+            }
+        };
+        const int n_items_stream = CL ? 0 : sm.item_base[sidx + 1] - sm.item_base[sidx];
+        if constexpr (CL)
+            cluster_wait();          // (the arrival in the prologue: every rank's receive barrier exists)
         // two head dims per consumer thread, the heads of one parity per half of the threads
         const int d2 = threadIdx.x & 63;
         for (int r = threadIdx.x >> 6; r < p.G; r += 2) {
@@ -448,23 +478,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(con
                 acc.y += v.y * c;
                 lsum += sm.comb_ml[w][r][1] * c;
             }
-            if (n_items_stream == 1) {
+            if constexpr (CL) {
+                cluster_send(rc, p.G, p.cl, chunk, r, d2, acc, M, lsum);
+            } else if (n_items_stream == 1) {
                 // the item is the whole sequence: finish here
-                const float o0 = acc.x / lsum, o1 = acc.y / lsum;
-                const size_t oi = ((size_t)b * p.nq + (size_t)kvh * p.G + r) * kHeadDim + 2 * d2;
-                if (p.o_fp16) {
-                    *reinterpret_cast<__half2 *>(reinterpret_cast<__half *>(p.o_out) + oi) = __floats2half2_rn(o0, o1);
-                } else {
-                    uint32_t hi, lo;
-                    split_bf16x2(o0, o1, hi, lo);
-                    *reinterpret_cast<uint32_t *>(p.o_out + oi) = hi;
-                    *reinterpret_cast<uint32_t *>(p.o_out + p.o_plane + oi) = lo;
-                }
+                store_o(r, 2 * d2, acc.x / lsum, acc.y / lsum);
             } else {
                 *reinterpret_cast<float2 *>(p.part_o + ((size_t)item * p.G + r) * kHeadDim + 2 * d2) = acc;
                 if (d2 == 0)
                     *reinterpret_cast<float2 *>(p.part_ml + ((size_t)item * p.G + r) * 2) = make_float2(M, lsum);
             }
+        }
+        if constexpr (CL) {
+            cluster_finish(rc, p.G, p.cl, chunk, threadIdx.x, p.status, p.trace, store_o);
+            return;
         }
         consumer_barrier();      // the combine rows are free for the next item
     }
@@ -508,13 +535,21 @@ cudaError_t launch_attention_kv8_kernel(const AttnArgs &a, const cudaLaunchConfi
     p.status = a.status;
     p.trace = a.trace;
     p.inject = a.inject;
-    static PerDeviceSize lim;      // per device: the attribute belongs to one device
-    cudaError_t e = ensure_dynamic_smem(k_attn_decode_splitkv_kv8, lim, attn_kv8_smem_bytes(kMaxStreams));
+    p.cl = a.cluster;
+    static PerDeviceSize lim, lim_cl;      // per device: the attributes belong to one device
+    cudaLaunchConfig_t cfg = base_cfg;
+    if (a.cluster) {
+        cudaError_t e = ensure_dynamic_smem(k_attn_decode_splitkv_kv8<true>, lim_cl, attn_kv8_smem_bytes(0));
+        if (e != cudaSuccess)
+            return e;
+        cfg.dynamicSmemBytes = attn_kv8_smem_bytes(0);
+        return cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv_kv8<true>, p);
+    }
+    cudaError_t e = ensure_dynamic_smem(k_attn_decode_splitkv_kv8<false>, lim, attn_kv8_smem_bytes(kMaxStreams));
     if (e != cudaSuccess)
         return e;
-    cudaLaunchConfig_t cfg = base_cfg;
     cfg.dynamicSmemBytes = attn_kv8_smem_bytes(a.B * a.nkv);
-    return cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv_kv8, p);
+    return cudaLaunchKernelEx(&cfg, k_attn_decode_splitkv_kv8<false>, p);
 }
 
 }  // namespace prsv

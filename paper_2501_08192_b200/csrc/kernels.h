@@ -195,6 +195,7 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s);
 
 // ---- split-KV decode attention + merge
 struct AttnArgs {
+    int cluster;          // > 0: one cluster of this many CTAs per (sequence, kv head), merged in the kernel (grid unused)
     CUtensorMap k_map;    // dims (d, max_batch*nkv*cap), box (64, 64), 128B swizzle
     CUtensorMap v_map;
     const void *q;        // split bf16 [2][rows][nq,d]
@@ -238,6 +239,9 @@ int attention_kv8_stages();
 // tile streams in half the time, so the same fixed work weighs twice as much).
 void plan_attention(const int32_t *ctx_len_host, int batch, int nkv, int sm_count, int *grid, int *tiles_per_item,
                     int stages = 3, double item_cost = 1.5);
+// Short caches: CTAs per (sequence, kv head) when one cluster each, merging inside the kernel, beats the items of
+// plan_attention and the merge kernel; 0 = the items.
+int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count);
 // 2-D uint8 tensor map (rows x cols bytes, cols contiguous), box (box_cols x box_rows), 128-byte swizzle.
 bool encode_u8_map_2d(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint32_t box_cols,
                       uint32_t box_rows);

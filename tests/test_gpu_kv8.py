@@ -90,6 +90,17 @@ def test_int8_cache_matches_the_quantised_oracle(oracle, shape):
     kv8_check(oracle, shape)
 
 
+@pytest.mark.parametrize("shape", [
+    # the cluster form of the attention: its largest range, the first beyond it, fewer tiles than CTAs, four CTAs
+    I.small_shape(name="kv8_cl_32_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=2047, ctx_min=0, seed=262),
+    I.small_shape(name="kv8_cl_33_tiles", batch=1, n_q_heads=5, n_kv_heads=1, ctx=2048, seed=263),
+    I.small_shape(name="kv8_cl_g7", batch=2, n_q_heads=7, n_kv_heads=1, ctx=512, ctx_min=64, seed=264),
+    I.small_shape(name="kv8_cl4", batch=10, n_q_heads=12, n_kv_heads=2, ctx=1023, ctx_min=1, seed=265),
+], ids=lambda s: s.name)
+def test_int8_cluster_attention_matches_the_quantised_oracle(oracle, shape):
+    kv8_check(oracle, shape)
+
+
 @pytest.mark.parametrize("idx", [0, 1, 3, 4])
 def test_int8_cache_on_benchmark_configs(oracle, idx):
     bits = kv8_check(oracle, I.CONFIGS[idx], budget=16 << 20)

@@ -388,3 +388,23 @@ def test_batch_tile_follows_the_step_batch(oracle, batches, flags):
                 assert o.guards_intact()
     finally:
         dl.close()
+
+
+# attention with one cluster per (sequence, kv head): every sequence at most 32 tiles of 64 keys (8 CTAs of 4; 16 tiles
+# with 4 CTAs, from 19 sequence-heads up); the last tile of the range and the first beyond it, fewer tiles than
+# CTAs, groups whose 128 G outputs do not divide into whole heads, an empty cache
+CLUSTER_SHAPES = [
+    I.small_shape(name="cl_g3_32_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=2047, ctx_min=0, seed=62),
+    I.small_shape(name="cl_33_tiles", batch=1, n_q_heads=3, n_kv_heads=1, ctx=2048, seed=63),
+    I.small_shape(name="cl_g5_one_tile", batch=3, n_q_heads=5, n_kv_heads=1, ctx=63, ctx_min=0, seed=64),
+    I.small_shape(name="cl_g7_9_tiles", batch=2, n_q_heads=7, n_kv_heads=1, ctx=512, seed=65),
+    I.small_shape(name="cl4_16_tiles", batch=10, n_q_heads=12, n_kv_heads=2, ctx=1023, ctx_min=1, seed=66),
+    I.small_shape(name="cl4_17_tiles", batch=10, n_q_heads=2, n_kv_heads=2, ctx=1024, ctx_min=1000, seed=67),
+    I.small_shape(name="cl4_tensor", batch=20, n_q_heads=8, n_kv_heads=1, ctx=500, ctx_min=2, seed=68),
+    I.small_shape(name="cl_37_streams", batch=37, n_q_heads=1, n_kv_heads=1, ctx=130, ctx_min=60, seed=69),
+]
+
+
+@pytest.mark.parametrize("shape", CLUSTER_SHAPES, ids=[s.name for s in CLUSTER_SHAPES])
+def test_cluster_attention_matches_oracle(oracle, shape):
+    full_check(oracle, shape)
