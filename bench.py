@@ -382,8 +382,9 @@ def bench_config(P, I, torch, dist, args, idx, rank, local_rank, world, stream, 
                 "h2d_bytes_per_step": h2d * R, "d2h_bytes_per_step": d2h * R},
         "gpu_launches": (n_main + n_pf) * R * args.steps,
         "kernels_us": {n: round(float(v) * 1e3, 3) for n, v in zip(P.KERNEL_NAMES, kms)},
-        "kernels_gbs": {n: round(kb[i] / (float(kms[i]) * 1e-3) / 1e9, 1) for i, n in enumerate(P.KERNEL_NAMES)},
-        "kernels_frac_of_measured": {n: round(kb[i] / (float(kms[i]) * 1e-3) / 1e9 / peak, 3)
+        "kernels_gbs": {n: round(kb[i] / (float(kms[i]) * 1e-3) / 1e9, 1) if kms[i] > 2e-4 else None
+                        for i, n in enumerate(P.KERNEL_NAMES)},
+        "kernels_frac_of_measured": {n: round(kb[i] / (float(kms[i]) * 1e-3) / 1e9 / peak, 3) if kms[i] > 2e-4 else None
                                      for i, n in enumerate(P.KERNEL_NAMES)},
         "roofline": {"bound": "hbm", "kernel": P.KERNEL_NAMES[dom], "achieved": round(achieved, 1), "peak": peak,
                      "unit": "GB/s", "frac": round(achieved / peak, 4),
