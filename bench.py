@@ -11,8 +11,9 @@ time), prefetch on vs off.  A "step" is one pass of the whole hot path over a ro
 distinct layer instances of the workload (distinct weight arenas and KV-caches, R x (weights +
 KV) >= 4 x L2), so every layer-step starts with a cold L2; per-layer figures are the step's
 divided by R.  Without --config all five benchmark configurations run in one invocation: the
-top-level `value` / `config` / `roofline` are those of the largest single-GPU one (configs[3]:
-70B-shaped TP=4 shard, batch 64, ragged contexts), `per_config` carries all five.
+top-level `value` / `config` / `roofline` are those of the largest single-GPU one (the
+70B-shaped TP=4 shard, batch 64, ragged contexts), `per_config` has a short row for each of the five and
+--details FILE takes everything that was measured.
 `value` is the effective GB/s with the library's default prefetch setting and inputs resident in
 HBM; `e2e` is the same metric through the host-buffer entry point with host<->device copies
 inside the timed region.  With --gpus N each rank runs an independent shard replica (no
@@ -127,6 +128,34 @@ def max_over_ranks(ms: float, world: int, device: str = "cuda") -> float:
 def whole_job_gbs(alg_bytes_per_layer: int, layers_per_step: int, ms_per_step: float, world: int) -> float:
     """Aggregate effective bandwidth of `world` independent replicas that all take ms_per_step."""
     return alg_bytes_per_layer * layers_per_step * world / (ms_per_step * 1e-3) / 1e9
+
+
+LINE_BYTES = 6000            # upper limit on the printed result line
+
+
+def result_line(out: dict) -> str:
+    """The one line rank 0 prints: every figure of the headline workload and a short row per configuration.
+    Sweeps, models, streaming tables and int8 rows go to the --details file only: with them the line was tens
+    of kilobytes long and got cut by whoever captured it."""
+    o = {k: v for k, v in out.items() if k not in ("per_config", "streams", "prefetch", "kernels_gbs")}
+    o["prefetch"] = {k: v for k, v in out["prefetch"].items()
+                     if k not in ("sweep", "modelled_window", "meaning", "paper_context")}
+    o["per_config"] = []
+    for c in out["per_config"]:
+        row = {"name": c["name"], "us_per_layer": c["us_per_layer"], "gbs": c["gbs"],
+               "off_us": c["prefetch"]["off_us_per_layer"], "e2e_us": c["e2e"]["us_per_layer"]}
+        for v in ("int8_kv", "int8_weights", "int8_weights_and_kv"):
+            if v in c:
+                row[v + "_us"] = c[v]["early_launch_only_us_per_layer"]
+        o["per_config"].append(row)
+    line = json.dumps(o)
+    # (what is optional leaves first, should anything grow: the required figures always fit)
+    for k in ("real_window", "per_config", "read_bandwidth", "kernels_us", "prefetch"):
+        if len(line) <= LINE_BYTES:
+            break
+        o.pop(k, None)
+        line = json.dumps(o)
+    return line
 
 
 def rotation_size(shape, l2_bytes: int) -> int:
@@ -657,10 +686,9 @@ def run_ours(args):
         except Exception as e:      # noqa: BLE001  (the replicas' result above must survive)
             out["real_window"] = {"error": f"{type(e).__name__}: {e}"}
     if rank == 0:
-        print(json.dumps(out), flush=True)
-        det = os.path.join(ROOT, "gpurun_out")
-        if os.path.isdir(det):
-            with open(os.path.join(det, f"bench_n{world}.json"), "w") as f:
+        print(result_line(out), flush=True)
+        if args.details:
+            with open(args.details, "w") as f:
                 json.dump(out, f, indent=1)
     if world > 1:
         dist.destroy_process_group()
@@ -1019,6 +1047,8 @@ def main():
     ap.add_argument("--no-cpu-baseline", dest="cpu_baseline", action="store_false")
     ap.add_argument("--no-real-window", action="store_true",
                     help="N > 1: skip the measurement of the real communication window")
+    ap.add_argument("--details", default="", metavar="FILE",
+                    help="also write the full result (sweeps, models, streams, every configuration) to FILE as JSON")
     ap.add_argument("--dry-run", action="store_true", help="launch plumbing only (CPU, gloo); nothing is timed")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)

@@ -140,3 +140,30 @@ def test_exchange_block_handles_travel_and_a_leaving_rank_is_noticed_on_the_host
     assert out[("events", 0)] == [1, 2, "peer lost"]
     assert "step 2" in out[("message", 0)]
     assert out[("events", 1)][:2] == [1, 2] and out[("events", 1)][2] in ("peer lost", "no error")
+
+
+def test_result_line_is_short_and_complete():
+    """The printed line carries every required figure and stays far below what a capture cuts off, whatever the sweeps,
+    models and streaming tables weigh; what is optional leaves first."""
+    import json
+    import bench
+    big = [{"frac_of_l2": i / 10, "us_per_layer": 123.456, "note": "x" * 200} for i in range(40)]
+    prefetch = {"on_us_per_layer": 1.0, "off_us_per_layer": 2.0, "sweep": big, "modelled_window": big, "meaning": "y" * 900,
+                "paper_context": "z"}
+    e2e = {"value": 1.0, "unit": "GB/s", "us_per_layer": 3.0, "h2d_bytes_per_step": 5, "d2h_bytes_per_step": 6}
+    row = {"name": "n" * 30, "us_per_layer": 1.0, "gbs": 2.0, "prefetch": prefetch, "e2e": e2e, "model": {"sweep": big},
+           "int8_kv": {"early_launch_only_us_per_layer": 4.0, "rows": big}}
+    required = dict(metric=bench.METRIC, value=4400.1, unit="GB/s", n_gpus=1, steps=20, warmup=5, ms_per_step=0.27,
+                    higher_is_better=True, scaling="weak", vs_baseline=None, dtype="bf16 (fp32 accumulate)", data="synthetic",
+                    config={"workload": "w" * 120, "cold_l2": "c" * 200, "parallelism": "p"}, e2e=e2e, gpu_launches=320,
+                    clocks={"sm_mhz": 1965, "sm_max_mhz": 1965, "reasons": []}, roofline={"bound": "hbm", "frac": 0.8},
+                    cpu_baseline={"value": 0.9, "cores": 16})
+    out = dict(required, prefetch=prefetch, kernels_us={"k": 1.0}, kernels_gbs={"k": 1.0}, read_bandwidth={"hbm": 1.0},
+               streams=big, per_config=[dict(row) for _ in range(5)])
+    assert len(json.dumps(out)) > 20000
+    for extra in ({}, {"real_window": big}):
+        line = bench.result_line(dict(out, **extra))
+        assert "\n" not in line and len(line) <= bench.LINE_BYTES
+        got = json.loads(line)
+        assert all(got[k] == v for k, v in required.items())
+        assert [c["off_us"] for c in got["per_config"]] == [2.0] * 5 and got["prefetch"]["on_us_per_layer"] == 1.0
