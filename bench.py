@@ -61,7 +61,7 @@ def load_peaks():
         with open(path) as f:
             p = json.load(f)
         return float(p["hbm_gbs"]), "measured (MEASURED_PEAKS.json hbm_gbs, copy bandwidth)"
-    return 6650.0, "fallback (6.65 TB/s, earlier measurement on this pool)"
+    return 6650.0, "fallback (6.65 TB/s, an earlier measurement)"
 
 
 class ClockSampler(threading.Thread):
@@ -383,7 +383,7 @@ def bench_config(P, I, torch, dist, args, idx, rank, local_rank, world, stream, 
     traffic = NCU_TRAFFIC.get((P.KERNEL_NAMES[dom], idx))
     res = {
         "config_index": idx, "name": shape.name,
-        "workload": f"configs[{idx}] {shape.name}: hidden {shape.hidden}, {shape.n_q_heads}q/{shape.n_kv_heads}kv heads, "
+        "workload": f"{shape.name}: hidden {shape.hidden}, {shape.n_q_heads}q/{shape.n_kv_heads}kv heads, "
                     f"ffn {shape.ffn}, batch {shape.batch}, ctx "
                     f"{'U[%d,%d]' % (shape.ctx_min, shape.ctx) if shape.ctx_min is not None else shape.ctx}, "
                     f"P={shape.tp_degree}",
@@ -697,7 +697,7 @@ def run_ours(args):
 # ------------------------------------------------------------------------ other modes
 def bench_real_window(P, I, torch, dist, args, rank, local_rank, world, stream):
     """N > 1: the communication window for real.  The ranks are the `world` shards of a
-    configs[1]-shaped layer (tp_degree = world) chained over a rotation of R layers; per layer-step
+    Llama-3-8B-shaped layer (tp_degree = world) chained over a rotation of R layers; per layer-step
     time with (a) the fused one-shot all-reduce window (peer reads in the window kernel), (b) the
     library-collective baseline (NCCL all-reduce + a one-buffer window, kernels queued one by one)
     and (c) the local stand-in, each with prefetch off / early launch only / on.  Every phase is
@@ -718,7 +718,7 @@ def bench_real_window(P, I, torch, dist, args, rank, local_rank, world, stream):
     wl = wl1 = comm = None
     try:
         R = rotation_size(base, l2)
-        # (Workload indexes I.CONFIGS: build from a patched copy of configs[1])
+        # (Workload indexes I.CONFIGS: build from a patched copy of that configuration)
         saved = I.CONFIGS
         I.CONFIGS = tuple(replace(c, tp_degree=world) if i == 1 else c for i, c in enumerate(saved))
         try:
@@ -843,7 +843,7 @@ def bench_real_window(P, I, torch, dist, args, rank, local_rank, world, stream):
     except Exception as e:      # noqa: BLE001
         err = f"{type(e).__name__}: {e}"
         res["error"] = err
-    res["workload"] = (f"{world} shards of a configs[1]-shaped layer (tp_degree {world}), rotation of {wl.R} layers, "
+    res["workload"] = (f"{world} shards of a Llama-3-8B-shaped layer (tp_degree {world}), rotation of {wl.R} layers, "
                        f"{steps * wl.R} layer-steps per setting, time = slowest rank")
     for w_ in (wl, wl1):
         if w_ is not None:
@@ -903,7 +903,7 @@ def run_timeline(P, I, torch, args, stream):
 
 
 def run_decode_loop(P, I, torch, args, stream):
-    """A 32-layer model made of configs[1] layers (linked chain: layer i + 1 consumes layer i's
+    """A 32-layer model made of Llama-3-8B-shaped TP=8 layers (linked chain: layer i + 1 consumes layer i's
     results), decoding tokens with every context advancing by one per token, against the same chain
     replayed with fixed contexts: us per token with prefetch off / early launch only / on, and the
     number of graphs captured along the way."""
@@ -963,7 +963,7 @@ def run_decode_loop(P, I, torch, args, stream):
     status = max(L.last_status() for L in wl.layers)
     print(json.dumps({"mode": "decode-loop", "layers": n_layers, "tokens": n_tokens,
                       "precision": "bf16" + (", int8 KV-cache" if args.int8_kv else "") + (", int8 weights" if args.int8_weights else ""),
-                      "workload": f"{n_layers} x configs[{idx}] {shape.name} (linked chain), contexts "
+                      "workload": f"{n_layers} x {shape.name} (linked chain), contexts "
                                   f"{int(start.min())}..{int(start.max())} advancing by one per token",
                       "results": res, "device_status": status}), flush=True)
     wl.close()
@@ -985,7 +985,7 @@ def cpu_baseline(shape, t, alg: int, budget_s: float, idx: int):
     dt = (time.perf_counter() - t0) / n
     return {"value": round(alg / dt / 1e9, 4), "unit": "GB/s", "us_per_layer": round(dt * 1e6, 1),
             "cores": O.num_threads(), "kind": "oracle",
-            "sample": f"{n} full layer-steps of configs[{idx}] ({shape.name}), one layer instance, after one untimed run"}
+            "sample": f"{n} full layer-steps of {shape.name}, one layer instance, after one untimed run"}
 
 
 def run_reference(args):
@@ -1011,12 +1011,12 @@ def run_reference(args):
         steps += 1
     ms = (time.perf_counter() - t0) * 1e3 / steps
     val = round(alg / (ms * 1e-3) / 1e9, 4)
-    sample = f"each step = one full layer-step of configs[{idx}] ({shape.name}) on one layer instance"
+    sample = f"each step = one full layer-step of {shape.name} on one layer instance"
     out = {"impl": "reference", "metric": METRIC, "value": val, "unit": "GB/s", "n_gpus": args.gpus,
            "steps": steps, "warmup": warm, "ms_per_step": round(ms, 3), "higher_is_better": True,
            "scaling": "weak", "vs_baseline": None, "dtype": "fp32 values, fp64 accumulation",
            "data": "synthetic (same seeded inputs as the CUDA arm)",
-           "config": {"workload": f"configs[{idx}] {shape.name}", "layers_per_step": 1,
+           "config": {"workload": shape.name, "layers_per_step": 1,
                       "algorithmic_bytes_per_layer": alg},
            "us_per_layer": round(ms * 1e3, 1),
            "cpu_baseline": {"value": val, "unit": "GB/s", "cores": O.num_threads(), "kind": "oracle", "sample": sample},
@@ -1032,7 +1032,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=10)
     ap.add_argument("--impl", default="ours", choices=("ours", "reference"))
     ap.add_argument("--config", type=int, default=-1,
-                    help="index into the five benchmark configurations (default: all five, configs[3] as the headline)")
+                    help="index into the five benchmark configurations (default: all five, the 70B-shaped batch-64 one as the headline)")
     ap.add_argument("--mode", default="bench", choices=("bench", "timeline", "decode-loop", "streams", "real-window"))
     ap.add_argument("--layers", type=int, default=32, help="decode-loop mode: layers of the chain")
     ap.add_argument("--rotation", type=int, default=0, help="layer instances per step (0 = sized from L2)")

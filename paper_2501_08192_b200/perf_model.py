@@ -167,7 +167,7 @@ def l2_size_sweep(hw: Hardware, ops: Sequence[Op], sizes_mib: Sequence[float]) -
 
 def b200_measured(hbm_gbs: float = 6900.0, l2_gbs: float = 18500.0, bf16_tflops: float = 1418.0,
                   l2_bytes: int = 132644864, kernel_overhead_us: float = 2.6, early_hides_us: float = 1.6) -> Hardware:
-    """This machine's B200 from measurements: bulk-copy read streams from HBM and from L2 (the stream
+    """A B200 from measurements: bulk-copy read streams from HBM and from L2 (the stream
     microbenchmark), sustained bf16 throughput, and the fixed per-kernel cost read off the kernel
     timelines (tail plus hand-over to the next kernel; early launch hides part of it).  No link: the
     single-GPU window is a local stand-in whose measured duration is passed to predict()."""
