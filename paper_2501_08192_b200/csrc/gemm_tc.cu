@@ -68,7 +68,7 @@ struct GemmTcParams {
     int producers;      // 1..kTcMaxProducers threads that issue the ring's TMA loads (stage uses dealt round-robin)
     int w8;             // the weight tiles arrive as int8 codes and are widened into tensor memory (the MMA's A operand)
     int w8_early;       // w8: the first ring fill's activation tiles complete their own barrier (codes widened before the wait)
-    int w8_slots;       // 2..kTcMaxW8Slots widened tiles in tensor memory (mt * 32 columns each) behind the accumulators
+    int w8_slots;       // 2..kTcMaxW8Slots widened tiles in tensor memory (mt * 64 columns each) behind the accumulators, at most `stages`
     const float *wscale;  // w8: one fp32 scale per packed weight row
     const uint8_t *w8_codes;  // w8: the codes, one contiguous block of mt * 128 rows x 64 bytes per (tile, k-block)
 };
@@ -480,6 +480,12 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         // The converter warps form groups of four, one warp per quadrant; group g widens the tile uses
         // g, g + G, ... on its own, so successive stages are widened concurrently (a single group
         // needs longer for one stage than the stage may take).
+        // A wait by parity means the phase it names only while the phase before that one is known to be over.  A
+        // group sees every G-th use only, so: G <= slots <= stages, and the slot is awaited before the stage.  The
+        // slot of use n says that the MMAs up to use n - slots are over (G <= slots: the group's wait before this
+        // one covered the slot's phase before), hence that the stage's use n - stages has landed.  Without it - three
+        // groups on a ring of two stages, the QKV projection from batch 97 up - a group passed the wait for
+        // a stage whose bytes were still to come, and the CTA could finish and exit ahead of its own loads.
         const int quad = warp & 3;
         int iq = 0, n_min = 1 << 30;     // this warp's index among its quadrant's converter warps; the groups
         for (int q2 = 0; q2 < 4; ++q2) {
@@ -492,7 +498,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 }
             n_min = n < n_min ? n : n_min;
         }
-        const int G = n_min;
+        const int G = n_min < p.w8_slots ? n_min : p.w8_slots;
         const bool f16 = p.f16 != 0;
         const int row = quad * 32 + lane;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(p.mt * acc_cols);
@@ -506,9 +512,10 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             if (turn == iq) {
                 int ok = 1;
                 if (lane == 0) {
-                    ok = mbar_wait(&full[st], ph, p.status, ST_TIMEOUT_FULL) ? 1 : 0;
-                    if (ok && reuse)
+                    if (reuse)
                         ok = mbar_wait(&slot_free[j], phj ^ 1, p.status, ST_TIMEOUT_EMPTY) ? 1 : 0;
+                    if (ok)
+                        ok = mbar_wait(&full[st], ph, p.status, ST_TIMEOUT_FULL) ? 1 : 0;
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) { poisoned = 1; break; }
@@ -1000,6 +1007,8 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
         }
     }
     p.stages = stages;
+    if (p.w8_slots > stages)      // (a stage is held until its MMAs are over: further slots would never be in use)
+        p.w8_slots = stages;
     p.recv_off = in_ring ? (int)tile_bytes : stages * stage_bytes;
     size_t smem = (size_t)stages * stage_bytes + recv_alloc + 1024;
     const size_t least = in_ring ? g.bulk_bytes(splits) : p.push == 2 ? tile_bytes : 0;

@@ -104,6 +104,10 @@ W8_SHAPES = [
     I.small_shape(name="w8_b33_ragged_g8", batch=33, ctx=300, ctx_min=1, n_q_heads=8, n_kv_heads=1, tp_degree=3, seed=116),
     I.small_shape(name="w8_b64", batch=64, hidden=1024, ffn=1152, ctx=64, seed=117),
     I.small_shape(name="w8_b128", batch=128, hidden=256, ffn=128, ctx=20, n_q_heads=2, n_kv_heads=2, seed=144),
+    # batch 97 up: the QKV ring has two stages, fewer than there are widening groups (four and eight uses per rank; 60: four stages)
+    I.small_shape(name="w8_h4096_b60", batch=60, hidden=4096, ffn=256, ctx=40, ctx_min=2, n_q_heads=4, n_kv_heads=1, seed=158),
+    I.small_shape(name="w8_h4096_b100", batch=100, hidden=4096, ffn=256, ctx=40, ctx_min=2, n_q_heads=4, n_kv_heads=1, seed=159),
+    I.small_shape(name="w8_h8192_b128", batch=128, hidden=8192, ffn=256, ctx=20, n_q_heads=8, n_kv_heads=1, seed=160),
     I.small_shape(name="w8_h8192_b40", batch=40, hidden=8192, ffn=256, ctx=50, ctx_min=3, n_q_heads=2, n_kv_heads=2,
                   tp_degree=3, seed=157),
 ]
