@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                 for (int j = 0; j < 4; ++j)
                     acc[r][i][j] = 0.f;
 
-        auto compute = [&](float (&a_)[NT][4], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
+        auto compute_into = [&](float (&a_)[NT][4], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
             if constexpr (!W8) {
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) {
@@ -233,6 +233,20 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                         mma_bf16_16816(a_[nt], a0, a1, a2, a3, (j & 1) ? xv.z : xv.x, (j & 1) ? xv.w : xv.y);
                     }
                 }
+            }
+        };
+
+        // PACK: every tile's products are summed by the tensor cores from zero and added to the running sum in fp32
+        // (the tensor cores' own accumulation truncates: over a warp's run it cost 2e-6 of the result, relative)
+        auto compute = [&](float (&a_)[NT][4], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
+            if constexpr (PACK) {
+                float d[NT][4] = {};
+                compute_into(d, wl, wh, xq);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    a_[0][j] += d[0][j];
+            } else {
+                compute_into(a_, wl, wh, xq);
             }
         };
 
