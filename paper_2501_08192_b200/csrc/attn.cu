@@ -228,6 +228,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
             }
 
             float corr[2];
+            // CL: P is taken relative to this tile's own maximum and the tile's products join the sums with the
+            // factor wgt, as if every tile were an item of its own - the largest weight of each tile and warp is then
+            // exactly one in bf16.  Relative to the running maximum, two to four tiles per rank put o up to 1.34 times as
+            // far from its float64 value as the one-tile items that short caches had before.
+            float wgt[2];
             uint32_t pa[4];
             if constexpr (narrow) {
                 // ---- up to 8 query heads: S^T = K Q^T, keys as the 16 MMA rows, heads as the 8 columns -
@@ -264,13 +269,17 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
                     corr[j] = m_new == -INFINITY ? 1.f : exp2f(m_run[j] - m_new);
                     m_run[j] = m_new;                       // (narrow: m_run / l_run belong to heads 2t, 2t + 1;
                     l_run[j] *= corr[j];                    //  l_run is this lane's share, summed at the end)
+                    if constexpr (CL)
+                        wgt[j] = mx[j] == -INFINITY ? 0.f : exp2f(mx[j] - m_new);
+                    else
+                        mx[j] = m_new;
                 }
                 float ph[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float m = m_run[j & 1];
+                    const float m = mx[j & 1];
                     ph[j] = m == -INFINITY ? 0.f : exp2f(v[j] - m);
-                    l_run[j & 1] += ph[j];
+                    l_run[j & 1] += CL ? ph[j] * wgt[j & 1] : ph[j];
                 }
                 // P^T (keys x heads) -> (heads x keys), the B fragment of P^T in O^T = V^T P^T: two 8 x 8 transposes
                 const uint32_t x0 = pack_bf16(ph[0], ph[1]), x1 = pack_bf16(ph[2], ph[3]);
@@ -360,7 +369,13 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
                     const uint32_t addr = rowaddr + (c >> 3) * kHalfBytes + ((cc ^ (key & 7)) << 4);
                     uint32_t r[4];     // transposed 8 x 8 blocks [keys 0-7 | 8-15] x [dims 0-7 | 8-15] of 16 head dims
                     ldmatrix_x4_trans(r, addr);
-                    if constexpr (narrow) {
+                    if constexpr (CL) {
+                        float d[4] = {0.f, 0.f, 0.f, 0.f};
+                        mma_bf16_16816(d, r[0], r[2], r[1], r[3], pa[0], pa[2]);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            o[c >> 1][j] = fmaf(d[j], wgt[j & 1], o[c >> 1][j]);
+                    } else if constexpr (narrow) {
                         mma_bf16_16816(o[c >> 1], r[0], r[2], r[1], r[3], pa[0], pa[2]);
                     } else {
                         mma_bf16_16816(o[c], pa[0], pa[1], pa[2], pa[3], r[0], r[1]);
