@@ -645,24 +645,32 @@ void plan_attention(const int32_t *ctx_len_host, int batch, int nkv, int sm_coun
     *tiles_per_item = best;
 }
 
-int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count)
+int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count, bool tensor_path)
 {
     if (nq / nkv > kMaxClusterGroup)
         return 0;
-    // Eight CTAs per (sequence, kv head), or four where eight would exceed one CTA per SM, and at most four tiles
-    // each (2047 or 1023 cached tokens).  The merge kernel's launch, hand-over and read of the partials go:
-    // us per layer, items / clusters: batch 1, ctx 512 24.5 / 24.2; batch 3, ctx up to 777 28.5 / 27.6; batch 7,
-    // ctx 160 72.8 / 70.6; batch 10, ctx up to 1084 46.3 / 45.0.  Sixteen CTAs lose: they only find a place together once
-    // the kernel in front has ended (batch 1: 24.6), and beyond four tiles the items' finer split wins
-    // (batch 8, ctx 4096, sixteen CTAs of five tiles 33.4 against 32.4).
+    // Eight CTAs per (sequence, kv head), or four where eight would exceed one CTA per SM.  The merge kernel's launch,
+    // hand-over and read of the partials go; the items' finer split and free placement are given up.  The lines, from
+    // layers with items / with clusters (four layers of an 8B-shaped TP=8 shard unless said, us; bf16 cache, int8 cache):
+    //   up to 20 tiles (16 with four CTAs), projections by GEMV: batch 1, ctx 511 112.8 / 110.4, 119.0 / 115.4; ctx 1023
+    //     113.8 / 112.1, 119.5 / 119.4; ctx 1200 114.3 / 113.1, 120.2 / 119.8; batch 8, ctx 511 126.1 / 121.3, 132.4 /
+    //     129.0; ctx 1200 127.0 / 127.0, 132.9 / 132.2; 0.993-1.11 times the speed over hidden 1024-8192, 1-8 kv heads.
+    //     Longer: batch 4, ctx 1535 118.7 / 119.0, 126.1 / 127.6; ctx 2047 118.3 / 121.7, 124.8 / 130.5.
+    //   two to four tiles in front of the tcgen05 GEMMs: batch 16, ctx 255 147.8 / 144.4, 152.0 / 152.1; batch 24 156.3 / 157.5,
+    //     163.1 / 160.1; batch 37 164.2 / 161.6, 168.8 / 165.2.  Longer: batch 20, ctx 767 162.3 / 169.9, 166.1 /
+    //     178.0 (half of the SMs without a CTA; batch 37 gains up to 5 % from ctx 400 to 1023, and is not worth a line).
+    //   one tile: an item is then the whole sequence, and nothing is left to merge: batch 16, ctx 60 138.0 / 143.5.
+    // Sixteen CTAs lose: they only find a place together once the kernel in front has ended (batch 1: 24.6 us a
+    // layer against 24.2 with eight).
     int cl = 8;
     while (cl >= 4 && batch * nkv * cl > sm_count) cl /= 2;
     if (cl < 4)
         return 0;
+    int longest = 0;
     for (int b = 0; b < batch; ++b)
-        if ((ctx_len_host[b] + 1 + kTileKeys - 1) / kTileKeys > 4 * cl)
-            return 0;
-    return cl;
+        longest = ctx_len_host[b] > longest ? ctx_len_host[b] : longest;
+    const int tiles = (longest + 1 + kTileKeys - 1) / kTileKeys;
+    return tiles >= 2 && tiles <= (tensor_path ? 4 : cl == 8 ? 20 : 16) ? cl : 0;
 }
 
 cudaError_t launch_attention(const AttnArgs &a, cudaStream_t s)
