@@ -144,8 +144,6 @@ struct preserve_layer {
 
     // tensor path
     CUtensorMap wmap[4];
-    CUtensorMap wmap256[4];      // box of 256 rows (valid when has256[i])
-    bool has256[4];
     CUtensorMap xmap[8][4];      // x, o, x2, a as B operands, for a batch tile of 16 * (first index + 1) rows
     int nb_pad;                  // max_batch rounded up to 16: rows per plane of the workspaces
 
@@ -398,7 +396,6 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
     if (L->tensor_path) {
         GemmTcArgs a = {};
         a.w_map = L->wmap[which];
-        a.w_map256 = L->has256[which] ? &L->wmap256[which] : nullptr;
         (void)x;
         // The batch tile follows the step's batch, not max_batch: a server sized for 128 sequences that holds
         // 20 otherwise multiplies, fetches and hands over 128 columns in every projection.
@@ -496,7 +493,7 @@ void plan_step(preserve_layer *L, const StepPtrs &sp, StepPlan *pl)
     pl->pf_b = (L->only == -1 || L->only == -3) && pl->planned[1][0] + pl->planned[1][1] > 0;
     plan_attention(sp.ctx_len_host, B, c.n_kv_heads, L->sm_count, &pl->attn_grid, &pl->attn_tpi,
                    L->kv8 ? attention_kv8_stages() : 3, L->kv8 ? 3.0 : 1.5);
-    pl->attn_cluster = plan_attention_cluster(sp.ctx_len_host, B, c.n_q_heads, c.n_kv_heads, L->sm_count);
+    pl->attn_cluster = plan_attention_cluster(sp.ctx_len_host, B, c.n_q_heads, c.n_kv_heads, L->sm_count, L->tensor_path);
     pl->attn_items_per_stream = (int)((max_tiles_seq + pl->attn_tpi - 1) / pl->attn_tpi);
     // (the merge kernel sizes its CTAs from this, between 4 and 32 warps: clamp here so that the
     // number that enters the graph signature changes as rarely as the launch does)
@@ -1208,8 +1205,6 @@ int preserve_layer_init(const preserve_layer_config_t *cfg, const preserve_layer
                 preserve_layer_destroy(L);
                 return PRESERVE_EARCH;
             }
-            L->has256[i] = !L->w8 && d.n[i] % 256 == 0 &&
-                           make_map_2d(&L->wmap256[i], L->arena + L->off[i], d.k[i], d.n[i], 64, 256);
         }
     }
     if ((c.flags & PRESERVE_FLAG_PERSIST_L2) && L->max_persist > 0) {

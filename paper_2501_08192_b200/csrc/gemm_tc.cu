@@ -6,10 +6,10 @@
 // 128 x 16-k slab of weights for every batch row at once and the CUDA cores stay
 // out of the weight stream entirely.
 //
-// Per CTA: one 128-row tile of the packed weights (two for wide batches, sharing one activation
+// Per CTA: one 128-row tile of the packed weights (int8 weights, wide batches: two that share one activation
 // tile) x one slice of k.
-//   warp 0 (+ lane 0 of the first one or two epilogue warps): TMA producers - W tile (128 or 256 rows
-//               x 64, 128B swizzle) and x tile (2 NB x 64) into a multi-stage shared-memory ring,
+//   warp 0 (+ lane 0 of the first one or two epilogue warps): TMA producers - W tile (128 rows x 64,
+//               128B swizzle) and x tile (2 NB x 64) into a multi-stage shared-memory ring,
 //               mbarrier full/empty; the ring's stage uses are dealt round-robin to the issuing threads
 //               (three instead of one measured < 1 %)
 //   warp 1    : allocates TMEM, issues tcgen05.mma (kind::f16, bf16 in, fp32
@@ -50,7 +50,7 @@ struct GemmTcParams {
     CUtensorMap w_map;
     CUtensorMap x_map;
     int B, NB, N, K;
-    int mt;             // 128-row weight tiles per CTA (1 or 2): two tiles share one activation tile
+    int mt;             // int8 weights: 128-row weight tiles per CTA (1, or 2 that share one activation tile)
     int kblocks;        // K / 64 (int8 weights: K / 128 - a stage carries 128 k)
     int splits;         // cluster size along k
     int stages;
@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
     constexpr int kBlk = W8 ? 2 * kTcBlockK : kTcBlockK;
     // int8 weights, narrow batches: the codes of the ring's first fill are widened before the activations exist
     constexpr bool kEarly = W8 && EARLY;
-    const int a_bytes = p.mt * kATileBytes;
+    const int mt = W8 ? p.mt : 1;     // 128-row weight tiles per CTA
+    const int a_bytes = mt * kATileBytes;
     const int b_bytes = p.planes * p.NB * kBlk * 2;
     const int stage_bytes = a_bytes + b_bytes;
     const int acc_cols = p.planes * p.NB;      // TMEM columns of one weight tile's accumulator
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
 
     // MMA-issuing threads (see run_mma): two for the int8 kernels with two weight tiles and sixteen epilogue warps
     // (the last of them is then not needed as a converter)
-    const int n_issuers = (W8 && p.mt == 2 && p.epi_warps == 16 && p.producers == 3) ? 2 : 1;
+    const int n_issuers = (W8 && mt == 2 && p.epi_warps == 16 && p.producers == 3) ? 2 : 1;
     trace_start(p.trace);
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         mbar_fence_init();
         poisoned = 0;
         if (PUSH && p.splits > 1)
-            mbar_expect_tx(&push_bar, (uint32_t)(p.splits - 1) * p.mt * kTcTileM * (p.NB / p.splits) * 4u);
+            mbar_expect_tx(&push_bar, (uint32_t)(p.splits - 1) * mt * kTcTileM * (p.NB / p.splits) * 4u);
         // The ring's first fill, weights only, right here: they never depend on earlier kernels, and a CTA
         // that becomes resident late - after the kernel in front has ended - should have its first bytes
         // under way before anything else of the prologue (tensor-memory allocation, tables, barriers
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                                    a_bytes, &full[i], pol);
                 else
                     tma_load_2d_hint(smem + (size_t)i * stage_bytes, &p.w_map, (kb0 + i) * kTcBlockK,
-                                     tile * p.mt * kTcTileM, &full[i], pol);
+                                     tile * mt * kTcTileM, &full[i], pol);
             }
         }
         tma_prefetch_desc(&p.x_map);
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             if constexpr (W8)
                 bulk_load_hint(a_dst, p.w8_codes + ((size_t)tile * p.kblocks + kb) * a_bytes, a_bytes, &full[st], pol);
             else
-                tma_load_2d_hint(a_dst, &p.w_map, kb * kTcBlockK, tile * p.mt * kTcTileM, &full[st], pol);
+                tma_load_2d_hint(a_dst, &p.w_map, kb * kTcBlockK, tile * mt * kTcTileM, &full[st], pol);
             load_b(st, kb, false);
             st += NP;
             while (st >= p.stages) {
@@ -368,7 +369,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                     if constexpr (W8) {
                         // widened tile of this use: 64 columns per weight tile (128 k), 8 per MMA; the activations
                         // are two 64-k boxes
-                        const uint32_t a_tmem = tmem_base + p.mt * acc_cols + (j * p.mt + m) * 64;
+                        const uint32_t a_tmem = tmem_base + mt * acc_cols + (j * mt + m) * 64;
                         const uint64_t bdesc2 = make_smem_desc(st_addr + a_bytes + b_bytes / 2);
 #pragma unroll
                         for (int k = 0; k < kBlk / 16; ++k)
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         if (lane == 0)
             run_producer(0);
     } else if (warp == 1) {
-        run_mma(0, n_issuers == 2 ? 1 : p.mt);
+        run_mma(0, n_issuers == 2 ? 1 : mt);
     }
     __syncwarp();
 
@@ -412,9 +413,9 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
     // their memory round trip would sit on the kernel's tail.
     float wsc[2] = {1.f, 1.f};
     if (W8 && is_epi) {
-        wsc[0] = p.wscale[(size_t)(tile * p.mt) * kTcTileM + row];
-        if (p.mt == 2)
-            wsc[1] = p.wscale[(size_t)(tile * p.mt + 1) * kTcTileM + row];
+        wsc[0] = p.wscale[(size_t)(tile * mt) * kTcTileM + row];
+        if (mt == 2)
+            wsc[1] = p.wscale[(size_t)(tile * mt + 1) * kTcTileM + row];
     }
     const int kSubs = ((int)blockDim.x / 32 - 2) / 4;    // warps per lane group
     const int par = lane & 1;
@@ -429,9 +430,9 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         int m = 0, cl = warp - 2;
         while (cl >= cols) { cl -= cols; ++m; }
         const int b = s * cols + cl;
-        if (m < p.mt && b < p.B) {
-            trig[0] = rope_trig(p.epi, tabs, tabs.pos[b], tile * p.mt + m, 2 * lane);
-            trig[1] = rope_trig(p.epi, tabs, tabs.pos[b], tile * p.mt + m, 2 * lane + 1);
+        if (m < mt && b < p.B) {
+            trig[0] = rope_trig(p.epi, tabs, tabs.pos[b], tile * mt + m, 2 * lane);
+            trig[1] = rope_trig(p.epi, tabs, tabs.pos[b], tile * mt + m, 2 * lane + 1);
         }
     } else if (is_epi && KIND == EPI_QKV && p.splits > 1 && PUSH == 1) {
         const int cols = p.NB / p.splits, hp = cols / 2;
@@ -439,17 +440,17 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         while (c2 >= hp) { c2 -= hp; ++m; }
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if (m < p.mt) {
+            if (m < mt) {
                 const int b = s * cols + 2 * c2 + par;
                 if (b < p.B)
-                    trig[k] = rope_trig(p.epi, tabs, tabs.pos[b], tile * p.mt + m, row >> 1);
+                    trig[k] = rope_trig(p.epi, tabs, tabs.pos[b], tile * mt + m, row >> 1);
                 c2 += kSubs;
                 while (c2 >= hp) { c2 -= hp; ++m; }
             }
     }
     // one finished pair of iteration k (k < 2 uses the factors above)
     auto finish_pair = [&](int k, int m, int b, float v0, float v1) {
-        const int pair = ((tile * p.mt + m) * kTcTileM + row) >> 1;
+        const int pair = ((tile * mt + m) * kTcTileM + row) >> 1;
         if constexpr (KIND == EPI_QKV) {
             const int pos = tabs.pos[b], hd = pair >> 6, i = pair & 63;
             const float2 cs = k == 0 ? trig[0] : (k == 1 ? trig[1] : rope_trig(p.epi, tabs, pos, hd, i));
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         const int G = n_min < p.w8_slots ? n_min : p.w8_slots;
         const bool f16 = p.f16 != 0;
         const int row = quad * 32 + lane;
-        const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(p.mt * acc_cols);
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(mt * acc_cols);
         const uint32_t src_lane = (uint32_t)row * 128;
         const uint32_t swz = (uint32_t)(row & 7);
         int st = 0, j = 0;
@@ -521,8 +522,8 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 if (!ok) { poisoned = 1; break; }
                 tc_fence_after();
                 const uint8_t *a8 = smem + (size_t)st * stage_bytes + src_lane;
-                const uint32_t slot_addr = lane_addr + (uint32_t)(j * p.mt * 64);
-                for (int mh = 0; mh < 2 * p.mt; ++mh) {      // (weight tile, half of its 128 k): four 16-byte groups
+                const uint32_t slot_addr = lane_addr + (uint32_t)(j * mt * 64);
+                for (int mh = 0; mh < 2 * mt; ++mh) {      // (weight tile, half of its 128 k): four 16-byte groups
                     const int m = mh >> 1, q0 = (mh & 1) * 4;
                     uint4 w[4];
 #pragma unroll
@@ -612,9 +613,9 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 mbar_arrive_cluster(cluster_map(&ready_bar, lane));
             // two chunks (four TMEM loads) in flight per wait
             const uint32_t red_row = smem_u32(red) + (uint32_t)row * 4u;
-            for (int j = sub; j < p.mt * nchunks; j += 2 * kSubs) {
+            for (int j = sub; j < mt * nchunks; j += 2 * kSubs) {
                 const int j1 = j + kSubs;
-                const bool two = j1 < p.mt * nchunks;
+                const bool two = j1 < mt * nchunks;
                 const int m0 = j / nchunks, c0 = j % nchunks;
                 const int m1 = two ? j1 / nchunks : m0, c1 = two ? j1 % nchunks : c0;
                 uint32_t h0[16], l0[16], h1[16], l1[16];
@@ -652,13 +653,13 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             // the (splits - 1) * mt copies go out side by side
             const int n_ewarps = kSubs * 4;
             const int e = lane < 8 ? (warp - 2) + lane * n_ewarps : 1 << 30;
-            if (e < (p.splits - 1) * p.mt && in_ring && !mbar_wait(&ready_bar, 0, p.status, ST_TIMEOUT_MMA)) {
+            if (e < (p.splits - 1) * mt && in_ring && !mbar_wait(&ready_bar, 0, p.status, ST_TIMEOUT_MMA)) {
                 poisoned = 1;      // (a peer that is this late gets nothing: its own wait records it)
-            } else if (e < (p.splits - 1) * p.mt) {
-                const int slot_q = e / p.mt, m = e % p.mt;
+            } else if (e < (p.splits - 1) * mt) {
+                const int slot_q = e / mt, m = e % mt;
                 const int q = slot_q < s ? slot_q : slot_q + 1;      // owner
                 const int my_slot = s < q ? s : s - 1;               // where the owner keeps this rank's share
-                bulk_copy_to_cluster(cluster_map(recv + ((size_t)(my_slot * p.mt + m) * cols) * kTcTileM, q),
+                bulk_copy_to_cluster(cluster_map(recv + ((size_t)(my_slot * mt + m) * cols) * kTcTileM, q),
                                      smem_u32(red + ((size_t)m * p.NB + q * cols) * kTcTileM),
                                      (uint32_t)cols * kTcTileM * 4u, cluster_map(&push_bar, q));
             }
@@ -679,12 +680,12 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 uint32_t base[SP], mstr[SP];
 #pragma unroll
                 for (int q = 0; q < SP; ++q) {
-                    base[q] = q == s ? red_a : recv_a + (uint32_t)((q < s ? q : q - 1) * p.mt * cols) * (kTcTileM * 4u);
+                    base[q] = q == s ? red_a : recv_a + (uint32_t)((q < s ? q : q - 1) * mt * cols) * (kTcTileM * 4u);
                     mstr[q] = (uint32_t)(q == s ? p.NB : cols) * (kTcTileM * 4u);
                 }
                 int m = 0, cl = warp - 2;
                 while (cl >= cols) { cl -= cols; ++m; }
-                for (int k = 0; m < p.mt; ++k) {
+                for (int k = 0; m < mt; ++k) {
                     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int q = 0; q < SP; ++q) {         // rank order
@@ -693,7 +694,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                     }
                     const int b = s * cols + cl;
                     if (b < p.B && !bad)
-                        apply_epilogue_quad_t<KIND>(p.epi, tabs, p.N, b, (tile * p.mt + m) * (kTcTileM / 2) + 2 * lane, acc, k == 0,
+                        apply_epilogue_quad_t<KIND>(p.epi, tabs, p.N, b, (tile * mt + m) * (kTcTileM / 2) + 2 * lane, acc, k == 0,
                                             trig[0], trig[1]);
                     cl += n_ew;
                     while (cl >= cols) { cl -= cols; ++m; }
@@ -726,10 +727,10 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         // rank order.  No cluster barrier and no remote loads on the critical path.
         const int cols = p.NB / p.splits;
         const uint32_t recv_a = smem_u32(smem + p.recv_off);
-        const uint32_t src_stride = (uint32_t)p.mt * kTcTileM * cols * 4u;          // bytes per source rank
+        const uint32_t src_stride = (uint32_t)mt * kTcTileM * cols * 4u;          // bytes per source rank
         cluster_wait();       // (the arrival at the top of the kernel: every rank's receive barrier exists)
         if (is_epi) {
-            for (int j = sub; j < p.mt * nchunks; j += kSubs) {
+            for (int j = sub; j < mt * nchunks; j += kSubs) {
                 const int m = j / nchunks, c = j % nchunks;
                 float v[16];
                 load_chunk(m, c, v);
@@ -765,7 +766,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 const int hp = cols / 2;                   // column pairs per m
                 int m = 0, c2 = sub;
                 while (c2 >= hp) { c2 -= hp; ++m; }
-                for (int k = 0; m < p.mt; ++k) {
+                for (int k = 0; m < mt; ++k) {
                     const uint32_t a = row_a + m * mstr + c2 * 8u;
                     float mine[2] = {0.f, 0.f};
 #pragma unroll
@@ -790,9 +791,9 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 finish(std::integral_constant<int, 8>());
         }
     } else if (is_epi) {
-        for (int j = sub; j < p.mt * nchunks; j += kSubs) {
+        for (int j = sub; j < mt * nchunks; j += kSubs) {
             const int m = j / nchunks, c = j % nchunks;
-            const int pair = ((tile * p.mt + m) * kTcTileM + row) >> 1;
+            const int pair = ((tile * mt + m) * kTcTileM + row) >> 1;
             float v[16];
             load_chunk(m, c, v);
 #pragma unroll
@@ -939,33 +940,19 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     const int planes = a.x_fp16 == 1 ? 1 : 2;
     p.planes = planes;
     p.f16 = a.x_fp16 ? 1 : 0;
-    // Two 128-row weight tiles per CTA share one activation tile, which halves the L2->SM traffic of the
-    // activations every CTA re-reads - and double the partial tile that the CTA's epilogue has to stage,
-    // send and finish.  They pay only where the activation tile outweighs a weight tile (two planes of 80
-    // rows and more): with pairs from 96 rows up four 70B-shaped TP=8 layers at batch 128 take 420.7 us,
-    // with single tiles 387.2 (tail of each GEMM 7 -> 3.5 us, the gate/up stream 20 -> 27 us); TP=4
-    // at batch 64 266.7 -> 265.8 us.  Nor do they pay where the matrix is so small that pairs leave half of the
-    // SMs without a CTA and single tiles fill more of them (QKV of that shard at batch 128: 40 CTAs 21 us, 80
-    // CTAs 14.5 us).
-    int mt = a.w8 ? a.w8_tiles : ((planes * a.NB >= 160 && a.N % (2 * kTcTileM) == 0 && a.w_map256) ? 2 : 1);
+    // 16-bit weights: one 128-row weight tile per CTA.  Two that share one activation tile halve the activations' traffic
+    // and double the partial tile that the CTA's epilogue has to stage, send and finish: at batch 96 and 128 four
+    // 70B-shaped TP=8 layers took 420.7 us with pairs, 387.2 without, and pairs for the two-plane QKV projection alone
+    // (from 80 rows up) still lost 2-5 % of a layer at batch 65-112 (hidden 8192, 8 q heads, batch 112: 183.9 -> 176.1 us
+    // per two layers; 32 q / 4 kv heads within 0.4 %) and nothing gained at batch 128.
+    const int mt = a.w8 ? a.w8_tiles : 1;
     if (a.w8 && (!a.w8_codes || !a.scales || mt < 1 || mt > 2))
         return cudaErrorInvalidValue;
     TcGeometry g;
-    bool fits = tc_geometry(a, sm_count, mt, g);
-    if (!a.w8 && mt == 2 && (!fits || g.tiles * g.splits * 2 < sm_count)) {
-        TcGeometry one;
-        if (tc_geometry(a, sm_count, 1, one) && (!fits || one.tiles * one.splits > g.tiles * g.splits)) {
-            g = one;
-            mt = 1;
-            fits = true;
-        }
-    }
-    if (!fits)
+    if (!tc_geometry(a, sm_count, mt, g))
         return cudaErrorInvalidValue;
     p.w8_codes = static_cast<const uint8_t *>(a.w8_codes);
     p.mt = mt;
-    if (mt == 2 && !a.w8)
-        p.w_map = *a.w_map256;
     const int tiles = g.tiles, stage_bytes = g.stage_bytes, per_sm = g.per_sm, splits = g.splits, w8_slots = g.w8_slots;
     const size_t tile_bytes = g.tile_bytes, smem_cap = g.smem_cap;
     int stages = g.stages;

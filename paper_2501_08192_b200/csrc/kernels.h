@@ -169,7 +169,6 @@ cudaError_t launch_gemv(const GemvArgs &a, int sm_count, cudaStream_t s);
 // ---- tcgen05 skinny GEMM (batch >= 16): W [N,K] K-major through TMA
 struct GemmTcArgs {
     CUtensorMap w_map;    // dims (K, N), box (64, 128), 128B swizzle
-    const CUtensorMap *w_map256;  // optional: same tensor with box (64, 256), for two weight tiles per CTA
     CUtensorMap x_map;    // dims (K, rows, planes), box (64, NB, planes), 128B swizzle: the first NB rows of the hi and
                           // the lo plane - or, with x_fp16 = 1, of the one fp16 plane
     int x_fp16;           // 0: two bf16 planes; 2: two fp16 planes (hi rows then lo rows); 1: the activations are one fp16 plane (inputs that come out of an RMSNorm: bounded,
@@ -180,7 +179,7 @@ struct GemmTcArgs {
     long long *trace;
     int pdl;
     int inject;
-    // int8 weights: the codes come from w8_codes by plain bulk copies (w_map / w_map256 are unused); the
+    // int8 weights: the codes come from w8_codes by plain bulk copies (w_map is unused); the
     // kernel widens every tile to the activations' 16-bit format into tensor memory (the MMA's A operand)
     // and multiplies every accumulator row by its scale
     int w8;
@@ -241,7 +240,7 @@ void plan_attention(const int32_t *ctx_len_host, int batch, int nkv, int sm_coun
                     int stages = 3, double item_cost = 1.5);
 // Short caches: CTAs per (sequence, kv head) when one cluster each, merging inside the kernel, beats the items of
 // plan_attention and the merge kernel; 0 = the items.
-int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count);
+int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count, bool tensor_path);
 // 2-D uint8 tensor map (rows x cols bytes, cols contiguous), box (box_cols x box_rows), 128-byte swizzle.
 bool encode_u8_map_2d(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint32_t box_cols,
                       uint32_t box_rows);
