@@ -415,21 +415,22 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
     p.delay_ns = a.delay_ns;
     p.status = a.status;
     // CTAs per row: as many (a power of two, at most 8) as leave every CTA at least 128 threads of
-    // one 8-element chunk each, and at most 256 CTAs in all: at batch 128 the 1024 CTAs of eight per row took 6 us
+    // one 8-element chunk each, and at most 256 CTAs in all (unless a slice would exceed 512 chunks): at batch 128 the 1024 CTAs of eight per row took 6 us
     // to start one after another behind the O projection (two per row: window B 10.7 -> 7.8 us, window A 9.3 -> 6.0,
     // four 70B-shaped TP=8 layers 378.1 -> 372.6 us; batch 64 and below within 0.1 %).  With few rows more CTAs
     // are better: at batch 16 four per row cost 1 %, two 2.5 %.
-    int cl = 1;
-    while (cl < kWinMaxCluster && (a.H / 8) % (cl * 2) == 0 && (a.H / 8) / (cl * 2) >= 128 &&
-           ((a.H / 8) / cl > 512 || a.B * cl * 2 <= kWinMaxCtas))
-        cl *= 2;
+    int cl = 1, uncut = 1;      // uncut: without the limit on the CTAs
+    while (uncut < kWinMaxCluster && (a.H / 8) % (uncut * 2) == 0 && (a.H / 8) / (uncut * 2) >= 128) uncut *= 2;
+    while (cl < uncut && ((a.H / 8) / cl > 512 || a.B * cl * 2 <= kWinMaxCtas)) cl *= 2;
     p.cluster = cl;
     const int chunks = a.H / 8 / cl;
-    // LEAN (inputs read after the wait, at most 64 registers: 389.1 -> 378.1 us there) for big batches, counted in
-    // threads (32768 = batch 32 at hidden 8192), and whenever an input buffer may still be
-    // written by an earlier kernel of the same call
+    // LEAN (inputs read after the wait, at most 64 registers: 389.1 -> 378.1 us there) for big batches, where the
+    // CTAs would be more than 256 without the limit above, and whenever an input buffer may still be
+    // written by an earlier kernel of the same call.  (Counted in threads instead, from 32768 up, it took in hidden 5120-7168
+    // at batch 37-64 and cost up to 7 % there: three layers of hidden 6144, batch 48 155.5 -> 166.2 us, hidden 7168,
+    // batch 56 179.0 -> 190.7; the two counts agree at hidden 2048, 4096 and 8192.)
     const bool comm = a.comm_rank >= 0;
-    const bool lean = ((long long)a.B * (a.H / 8) > 32768 || a.inputs_after_wait || comm) && chunks <= 512;
+    const bool lean = (a.B * uncut > kWinMaxCtas || a.inputs_after_wait || comm) && chunks <= 512;
     if ((a.inputs_after_wait || comm) && !lean)
         return cudaErrorInvalidValue;
     if (comm && (a.n_parts > 8 || a.part0_is_f32 || a.comm_rank >= a.n_parts))
