@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                 for (int j = 0; j < 4; ++j)
                     acc[r][i][j] = 0.f;
 
-        auto compute_into = [&](float (&a_)[NT][4], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
+        auto compute = [&](float (&a_)[NT][4], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
             if constexpr (!W8) {
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) {
@@ -236,20 +236,6 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
             }
         };
 
-        // PACK: every tile's products are summed by the tensor cores from zero and added to the running sum in fp32
-        // (the tensor cores' own accumulation truncates: over a warp's run it cost 2e-6 of the result, relative)
-        auto compute = [&](float (&a_)[NT][4], const uint4 &wl, const uint4 &wh, const uint4 (&xq)[NX]) {
-            if constexpr (PACK) {
-                float d[NT][4] = {};
-                compute_into(d, wl, wh, xq);
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    a_[0][j] += d[0][j];
-            } else {
-                compute_into(a_, wl, wh, xq);
-            }
-        };
-
         // ---- stream this warp's run through its ring
         for (int c0 = c_begin; ok && c0 < c_end; c0 += kBurst) {
             const int nb = min(kBurst, c_end - c0);
@@ -269,12 +255,22 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                         if (ok) {
                             const uint4 *wtile =
                                 reinterpret_cast<const uint4 *>(ring + slot * (kUnitChunks * 1024)) + lane * 2;
+                            // PACK: a unit's products are summed by the tensor cores from zero and added to the
+                            // running sum in fp32.  (The tensor cores' own accumulation truncates: over a
+                            // warp's whole run the SwiGLU output of hidden 8192 was 3.1e-6 off its float64 value, with
+                            // fp32 FMAs 2.4e-6, so 2.4e-6; the two-plane store alone is 2.3e-6.  0-0.5 % of a layer.)
+                            float d[NT][4] = {};
 #pragma unroll
                             for (int u = 0; u < kUnitChunks; ++u)
                                 if (uu * kUnitChunks + u < nb) {
                                     const uint4 wl = wtile[u * 64], wh = wtile[u * 64 + 1];
-                                    compute(acc[r], wl, wh, xq[uu * kUnitChunks + u]);
+                                    compute(PACK ? d : acc[r], wl, wh, xq[uu * kUnitChunks + u]);
                                 }
+                            if constexpr (PACK) {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    acc[r][0][j] += d[0][j];
+                            }
                         }
                         ++n_consumed;
                         __syncwarp();
