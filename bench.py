@@ -98,16 +98,17 @@ class ClockSampler(threading.Thread):
                 "reasons": reasons, "samples": len(sm)}
 
 
-def kernel_bytes(s, sum_ctx: int):
+def kernel_bytes(s, sum_ctx: int, merged: bool = False):
     """Algorithmic bytes per launch of each main-stream kernel (order: window A, QKV, split-KV
-    attention, merge, O, window B, gate/up, down).  Their sum is the layer-step's algorithmic bytes."""
+    attention, merge, O, window B, gate/up, down).  Their sum is the layer-step's algorithmic bytes.
+    merged: the attention merges its partials itself and writes the output; there is no merge kernel."""
     B, H, d, P_ = s.batch, s.hidden, s.head_dim, s.tp_degree
     BH, Bq, Bkv, BF = B * H * 2, B * s.n_q_heads * d * 2, B * s.n_kv_heads * d * 2, B * s.ffn * 2
     wqkv = 2 * H * (s.n_q_heads + 2 * s.n_kv_heads) * d
     wo, wgu, wdn = 2 * s.n_q_heads * d * H, 2 * H * 2 * s.ffn, 2 * s.ffn * H
     kv = 2 * sum_ctx * s.n_kv_heads * d * 2
     win = (P_ + 1) * BH + H * 2 + 2 * BH
-    return [win, wqkv + BH + Bq + 2 * Bkv, kv + Bq, Bq, wo + Bq + BH, win, wgu + BH + BF, wdn + BF + BH]
+    return [win, wqkv + BH + Bq + 2 * Bkv, kv + Bq + (Bq if merged else 0), 0 if merged else Bq, wo + Bq + BH, win, wgu + BH + BF, wdn + BF + BH]
 
 
 def algorithmic_bytes(s, sum_ctx: int) -> int:
@@ -350,11 +351,15 @@ def bench_config(P, I, torch, dist, args, idx, rank, local_rank, world, stream, 
     # instances (cold L2 by rotation) from a captured graph, CUDA events on the launching stream
     # around many replays.  Launches of one kernel are independent of each other, so this is the
     # kernel's own duration including its launch hand-over, not a dependency chain.
-    kms = np.full(len(P.KERNEL_NAMES), 1e-9)
+    kms = np.zeros(len(P.KERNEL_NAMES))
     with torch.cuda.stream(stream):
         chain_step()
         torch.cuda.synchronize()
+    merged = layers[0].attention_cluster_size() > 0       # no merge kernel: its slot stays empty
     for k in range(len(P.KERNEL_NAMES) if not args.no_kernels else 0):
+        if merged and P.KERNEL_NAMES[k] == "attn_merge":
+            continue
+
         def one():
             for L, io in zip(layers, ios):
                 L.run_kernel(io, k, stream)
@@ -372,13 +377,11 @@ def bench_config(P, I, torch, dist, args, idx, rank, local_rank, world, stream, 
     info = layers[0].get_info()
     n_pf = sum(1 for w in range(2) if sum(info.planned_bytes[w]) > 0)
 
-    # main-stream kernels per layer: a short cache's attention merges its partials itself, and the merge slot is empty
-    n_main = len(P.KERNEL_NAMES) if args.no_kernels else int((kms > 2e-4).sum())
-    kms = np.maximum(kms, 1e-9)
-
-    kb = kernel_bytes(shape, wl.sum_ctx)
+    n_main = len(P.KERNEL_NAMES) - (1 if merged else 0)
+    kb = kernel_bytes(shape, wl.sum_ctx, merged)
     dom = int(np.argmax(kms))
-    achieved = kb[dom] / (kms[dom] * 1e-3) / 1e9
+    rate = [kb[i] / (float(v) * 1e-3) / 1e9 if v > 0 else None for i, v in enumerate(kms)]
+    achieved = rate[dom] or 0.0
     best = min(sweep, key=lambda e: e["us_per_layer"]) if sweep else None
     traffic = NCU_TRAFFIC.get((P.KERNEL_NAMES[dom], idx))
     res = {
@@ -411,10 +414,8 @@ def bench_config(P, I, torch, dist, args, idx, rank, local_rank, world, stream, 
                 "h2d_bytes_per_step": h2d * R, "d2h_bytes_per_step": d2h * R},
         "gpu_launches": (n_main + n_pf) * R * args.steps,
         "kernels_us": {n: round(float(v) * 1e3, 3) for n, v in zip(P.KERNEL_NAMES, kms)},
-        "kernels_gbs": {n: round(kb[i] / (float(kms[i]) * 1e-3) / 1e9, 1) if kms[i] > 2e-4 else None
-                        for i, n in enumerate(P.KERNEL_NAMES)},
-        "kernels_frac_of_measured": {n: round(kb[i] / (float(kms[i]) * 1e-3) / 1e9 / peak, 3) if kms[i] > 2e-4 else None
-                                     for i, n in enumerate(P.KERNEL_NAMES)},
+        "kernels_gbs": {n: round(r, 1) if r else None for n, r in zip(P.KERNEL_NAMES, rate)},
+        "kernels_frac_of_measured": {n: round(r / peak, 3) if r else None for n, r in zip(P.KERNEL_NAMES, rate)},
         "roofline": {"bound": "hbm", "kernel": P.KERNEL_NAMES[dom], "achieved": round(achieved, 1), "peak": peak,
                      "unit": "GB/s", "frac": round(achieved / peak, 4),
                      "traffic": traffic[0] if traffic else None,

@@ -278,14 +278,17 @@ PRESERVE_API int preserve_decode_step_host(preserve_layer_t *layer, const preser
  * on that stream around each main-stream kernel, waits for the stream, and writes
  * PRESERVE_N_KERNELS durations in milliseconds: window A, QKV projection, split-KV
  * attention, attention merge, output projection, window B, gate/up projection,
- * down projection.  Results of the step are the same as preserve_decode_step's. */
+ * down projection.  Results of the step are the same as preserve_decode_step's.  Where the attention merges its
+ * partials itself (preserve_attention_cluster_size > 0) there is no merge kernel and its slot is empty: the time
+ * between two events. */
 #define PRESERVE_N_KERNELS 8
 PRESERVE_API int preserve_profile_step(preserve_layer_t *layer, const preserve_step_io_t *io, void *cuda_stream,
                                        float *kernel_ms);
 
 /* Queue ONE main-stream kernel of the step (index as in preserve_profile_step) with the
  * step's arguments, directly on `cuda_stream`, without prefetch.  For benchmarks that time a
- * kernel on its own; the buffers it reads must hold the results of an earlier full step. */
+ * kernel on its own; the buffers it reads must hold the results of an earlier full step.  (The merge of a step
+ * whose attention merges its partials itself: nothing is queued.) */
 PRESERVE_API int preserve_run_kernel(preserve_layer_t *layer, const preserve_step_io_t *io, int32_t which,
                                      void *cuda_stream);
 
@@ -311,6 +314,11 @@ PRESERVE_API int preserve_read_trace(preserve_layer_t *layer, int64_t *out);
 
 /* Sizes, device attributes and the last plan. */
 PRESERVE_API int preserve_layer_get_info(const preserve_layer_t *layer, preserve_info_t *info);
+
+/* How the attention of the handle's last queued step was cut: the CTAs of the cluster that each (sequence, KV head)
+ * got, merged inside the kernel; or 0 = work items, whose partials a merge kernel combines (also before the
+ * first step).  Depends on the batch, the sequence lengths and the heads. */
+PRESERVE_API int32_t preserve_attention_cluster_size(const preserve_layer_t *layer);
 
 /* Synchronises the device and returns the layer's device status word: PRESERVE_OK;
  * PRESERVE_ETIMEOUT if a bounded wait gave up (the step's results are then undefined, the

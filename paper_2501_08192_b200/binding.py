@@ -36,7 +36,7 @@ EXPORTS = (
     "preserve_last_status_code", "preserve_comm_create", "preserve_comm_export", "preserve_comm_import",
     "preserve_comm_set_peer", "preserve_comm_write", "preserve_comm_debug_arrive", "preserve_comm_epoch",
     "preserve_comm_destroy", "preserve_layer_set_comm", "preserve_layer_set_external_attention_sum",
-    "preserve_prefetch_window", "preserve_measure_stream_tma", "preserve_kv8_layout",
+    "preserve_prefetch_window", "preserve_measure_stream_tma", "preserve_kv8_layout", "preserve_attention_cluster_size",
 )
 NODE_COMM, NODE_MATMUL, NODE_ATTENTION, NODE_OTHER = 0, 1, 2, 3
 TRACE_SLOTS = 8
@@ -112,6 +112,7 @@ def lib() -> C.CDLL:
         L.preserve_graph_captures.argtypes = [C.c_void_p]
         L.preserve_graph_captures.restype = C.c_int64
         L.preserve_debug_set.argtypes = [C.c_void_p, C.c_int32, C.c_int64]
+        L.preserve_attention_cluster_size.argtypes = [C.c_void_p]
         L.preserve_attention_static_status.argtypes = []
         L.preserve_measure_stream.argtypes = [C.c_void_p, C.c_size_t, C.c_int32, C.c_int32, C.c_int32, C.c_int32,
                                               C.c_uint32, C.c_int32, C.c_void_p, C.c_void_p, C.POINTER(C.c_float)]
@@ -332,6 +333,10 @@ class Layer:
         return int(lib().preserve_graph_captures(self.handle))
 
     def set_prefetch_mechanism(self, mechanism: int, chunk_bytes: int = 4096, ctas: int = 128) -> None:
+    def attention_cluster_size(self) -> int:
+        """CTAs per (sequence, KV head) of the last step's attention where it merged its partials itself; else 0."""
+        return int(lib().preserve_attention_cluster_size(self.handle))
+
         _check(lib().preserve_set_prefetch_mechanism(self.handle, mechanism, chunk_bytes, ctas),
                "preserve_set_prefetch_mechanism")
 

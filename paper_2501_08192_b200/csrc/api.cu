@@ -170,6 +170,7 @@ struct preserve_layer {
     int plan_mode;
     uint64_t planned[2][3];
     uint64_t kv_bytes, alg_bytes;
+    int attn_cluster;            // of the last queued step
     int last_cuda;
     int prefetch_ctas;
 
@@ -513,6 +514,7 @@ int enqueue_step(preserve_layer *L, const StepPtrs &sp, const StepPlan &pl, bool
         for (int j = 0; j < 3; ++j)
             L->planned[w][j] = pl.planned[w][j];
     const int pdl = pl.pdl;
+    L->attn_cluster = pl.attn_cluster;
     const bool pf_a = pl.pf_a, pf_b = pl.pf_b;
 #define WANT(k) (L->only == -1 || L->only == (k))
 #define TRACE(k) (L->tracing ? L->trace_buf + PRESERVE_TRACE_SLOTS * (k) : nullptr)
@@ -892,6 +894,7 @@ int run_steps(preserve_layer *const *layers, StepPtrs *sps, int n, cudaStream_t 
             }
             CK(L0, cudaGraphLaunch(g.exec, s));
             return PRESERVE_OK;
+                L->attn_cluster = plans[i].attn_cluster;
         }
     // capture
     CK(L0, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -1256,6 +1259,8 @@ int preserve_debug_set(preserve_layer_t *L, int32_t what, int64_t value)
 {
     if (!L)
         return PRESERVE_EINVAL;
+int32_t preserve_attention_cluster_size(const preserve_layer_t *L) { return L ? L->attn_cluster : 0; }
+
     if (what == PRESERVE_DEBUG_WITHHOLD) {
         if (value < 0 || value > INJECT_ATTN_RING)
             return PRESERVE_EINVAL;

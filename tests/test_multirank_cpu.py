@@ -167,3 +167,13 @@ def test_result_line_is_short_and_complete():
         got = json.loads(line)
         assert all(got[k] == v for k, v in required.items())
         assert [c["off_us"] for c in got["per_config"]] == [2.0] * 5 and got["prefetch"]["on_us_per_layer"] == 1.0
+
+
+def test_merged_attention_books_its_output_on_the_attention():
+    """Where the attention merges its partials itself there is no merge kernel: the bytes move, their sum stays."""
+    import bench
+    from paper_2501_08192_b200 import inputs as I
+    for s in I.CONFIGS:
+        apart, merged = bench.kernel_bytes(s, 1000), bench.kernel_bytes(s, 1000, merged=True)
+        assert sum(apart) == sum(merged) and merged[3] == 0 and merged[2] == apart[2] + apart[3]
+        assert apart[:2] + apart[4:] == merged[:2] + merged[4:]
