@@ -510,11 +510,11 @@ int enqueue_step(preserve_layer *L, const StepPtrs &sp, const StepPlan &pl, bool
 
     L->kv_bytes = pl.kv_bytes;
     L->alg_bytes = pl.alg_bytes;
+    L->attn_cluster = pl.attn_cluster;
     for (int w = 0; w < 2; ++w)
         for (int j = 0; j < 3; ++j)
             L->planned[w][j] = pl.planned[w][j];
     const int pdl = pl.pdl;
-    L->attn_cluster = pl.attn_cluster;
     const bool pf_a = pl.pf_a, pf_b = pl.pf_b;
 #define WANT(k) (L->only == -1 || L->only == (k))
 #define TRACE(k) (L->tracing ? L->trace_buf + PRESERVE_TRACE_SLOTS * (k) : nullptr)
@@ -890,11 +890,11 @@ int run_steps(preserve_layer *const *layers, StepPtrs *sps, int n, cudaStream_t 
                 preserve_layer *L = layers[i];
                 L->kv_bytes = plans[i].kv_bytes;
                 L->alg_bytes = plans[i].alg_bytes;
+                L->attn_cluster = plans[i].attn_cluster;
                 memcpy(L->planned, plans[i].planned, sizeof(L->planned));
             }
             CK(L0, cudaGraphLaunch(g.exec, s));
             return PRESERVE_OK;
-                L->attn_cluster = plans[i].attn_cluster;
         }
     // capture
     CK(L0, cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -1255,12 +1255,12 @@ int preserve_set_prefetch_mechanism(preserve_layer_t *L, int32_t mechanism, uint
     return PRESERVE_OK;
 }
 
+int32_t preserve_attention_cluster_size(const preserve_layer_t *L) { return L ? L->attn_cluster : 0; }
+
 int preserve_debug_set(preserve_layer_t *L, int32_t what, int64_t value)
 {
     if (!L)
         return PRESERVE_EINVAL;
-int32_t preserve_attention_cluster_size(const preserve_layer_t *L) { return L ? L->attn_cluster : 0; }
-
     if (what == PRESERVE_DEBUG_WITHHOLD) {
         if (value < 0 || value > INJECT_ATTN_RING)
             return PRESERVE_EINVAL;
