@@ -111,8 +111,8 @@ def lib() -> C.CDLL:
         L.preserve_clear_status.argtypes = [C.c_void_p]
         L.preserve_graph_captures.argtypes = [C.c_void_p]
         L.preserve_graph_captures.restype = C.c_int64
-        L.preserve_debug_set.argtypes = [C.c_void_p, C.c_int32, C.c_int64]
         L.preserve_attention_cluster_size.argtypes = [C.c_void_p]
+        L.preserve_debug_set.argtypes = [C.c_void_p, C.c_int32, C.c_int64]
         L.preserve_attention_static_status.argtypes = []
         L.preserve_measure_stream.argtypes = [C.c_void_p, C.c_size_t, C.c_int32, C.c_int32, C.c_int32, C.c_int32,
                                               C.c_uint32, C.c_int32, C.c_void_p, C.c_void_p, C.POINTER(C.c_float)]
@@ -332,11 +332,11 @@ class Layer:
     def graph_captures(self) -> int:
         return int(lib().preserve_graph_captures(self.handle))
 
-    def set_prefetch_mechanism(self, mechanism: int, chunk_bytes: int = 4096, ctas: int = 128) -> None:
     def attention_cluster_size(self) -> int:
         """CTAs per (sequence, KV head) of the last step's attention where it merged its partials itself; else 0."""
         return int(lib().preserve_attention_cluster_size(self.handle))
 
+    def set_prefetch_mechanism(self, mechanism: int, chunk_bytes: int = 4096, ctas: int = 128) -> None:
         _check(lib().preserve_set_prefetch_mechanism(self.handle, mechanism, chunk_bytes, ctas),
                "preserve_set_prefetch_mechanism")
 
