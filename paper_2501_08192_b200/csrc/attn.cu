@@ -19,8 +19,10 @@
 // O += P V (V via ldmatrix.trans).  At the end of an item the four warps combine
 // their (max, sum, O) through the ring stage they consumed last and the CTA writes
 // ONE fp32 partial per item (or the final o when the item is the whole sequence).
-// k_attn_merge then combines the partials of a sequence in fixed order.  Nothing
-// depends on timing, so results are bit-stable.
+// k_attn_merge then combines the partials of a sequence in fixed order.  Short caches
+// (plan_attention_cluster) take one cluster of CTAs per (sequence, kv head) instead, whose ranks
+// hand their partials to one another through shared memory and write the merged o; there is no
+// merge kernel then.  Nothing depends on timing, so results are bit-stable.
 #include <cstdlib>
 #include <type_traits>
 
@@ -203,6 +205,12 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
             o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
         float m_run[2] = {-INFINITY, -INFINITY};
         float l_run[2] = {0.f, 0.f};
+        // CL: m_run is the reference of the sums, not their maximum (m_top): each tile's weights are taken relative to
+        // the tile's OWN maximum, as if it were an item of its own, so that its largest weight is exactly one in bf16 -
+        // unless the tile lies more than 2^20 below the largest so far and does not matter.  Relative to the running
+        // maximum, two to four tiles per rank put o up to 1.34 times as far from its float64 value as the
+        // one-tile items that short caches have otherwise (batch 1, 2047 tokens, hidden 8192: 3.0e-4 -> 4.0e-4).
+        float m_top[2] = {-INFINITY, -INFINITY};
 
         for (int tile = t0; ok && tile < t1; ++tile, ++it) {
             const int st = it % kStages;
@@ -228,11 +236,6 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
             }
 
             float corr[2];
-            // CL: P is taken relative to this tile's own maximum and the tile's products join the sums with the
-            // factor wgt, as if every tile were an item of its own - the largest weight of each tile and warp is then
-            // exactly one in bf16.  Relative to the running maximum, two to four tiles per rank put o up to 1.34 times as
-            // far from its float64 value as the one-tile items that short caches had before.
-            float wgt[2];
             uint32_t pa[4];
             if constexpr (narrow) {
                 // ---- up to 8 query heads: S^T = K Q^T, keys as the 16 MMA rows, heads as the 8 columns -
@@ -265,21 +268,21 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
                     mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], 4));
                     mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], 8));
                     mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], 16));
-                    const float m_new = fmaxf(m_run[j], mx[j]);
+                    float m_new = fmaxf(m_run[j], mx[j]);
+                    if constexpr (CL) {
+                        m_top[j] = fmaxf(m_top[j], mx[j]);
+                        m_new = fmaxf(mx[j], m_top[j] - 20.f);
+                    }
                     corr[j] = m_new == -INFINITY ? 1.f : exp2f(m_run[j] - m_new);
                     m_run[j] = m_new;                       // (narrow: m_run / l_run belong to heads 2t, 2t + 1;
                     l_run[j] *= corr[j];                    //  l_run is this lane's share, summed at the end)
-                    if constexpr (CL)
-                        wgt[j] = mx[j] == -INFINITY ? 0.f : exp2f(mx[j] - m_new);
-                    else
-                        mx[j] = m_new;
                 }
                 float ph[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float m = mx[j & 1];
+                    const float m = m_run[j & 1];
                     ph[j] = m == -INFINITY ? 0.f : exp2f(v[j] - m);
-                    l_run[j & 1] += CL ? ph[j] * wgt[j & 1] : ph[j];
+                    l_run[j & 1] += ph[j];
                 }
                 // P^T (keys x heads) -> (heads x keys), the B fragment of P^T in O^T = V^T P^T: two 8 x 8 transposes
                 const uint32_t x0 = pack_bf16(ph[0], ph[1]), x1 = pack_bf16(ph[2], ph[3]);
@@ -369,13 +372,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
                     const uint32_t addr = rowaddr + (c >> 3) * kHalfBytes + ((cc ^ (key & 7)) << 4);
                     uint32_t r[4];     // transposed 8 x 8 blocks [keys 0-7 | 8-15] x [dims 0-7 | 8-15] of 16 head dims
                     ldmatrix_x4_trans(r, addr);
-                    if constexpr (CL) {
-                        float d[4] = {0.f, 0.f, 0.f, 0.f};
-                        mma_bf16_16816(d, r[0], r[2], r[1], r[3], pa[0], pa[2]);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            o[c >> 1][j] = fmaf(d[j], wgt[j & 1], o[c >> 1][j]);
-                    } else if constexpr (narrow) {
+                    if constexpr (narrow) {
                         mma_bf16_16816(o[c >> 1], r[0], r[2], r[1], r[3], pa[0], pa[2]);
                     } else {
                         mma_bf16_16816(o[c], pa[0], pa[1], pa[2], pa[3], r[0], r[1]);
@@ -645,21 +642,21 @@ void plan_attention(const int32_t *ctx_len_host, int batch, int nkv, int sm_coun
     *tiles_per_item = best;
 }
 
-int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count, bool tensor_path)
+int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count, bool tensor_path, bool kv8)
 {
-    if (nq / nkv > kMaxClusterGroup)
+    if (nq / nkv > kMaxClusterGroup || tensor_path)
         return 0;
     // Eight CTAs per (sequence, kv head), or four where eight would exceed one CTA per SM.  The merge kernel's launch,
     // hand-over and read of the partials go; the items' finer split and free placement are given up.  The lines, from
-    // layers with items / with clusters (four layers of an 8B-shaped TP=8 shard unless said, us; bf16 cache, int8 cache):
-    //   up to 20 tiles (16 with four CTAs), projections by GEMV: batch 1, ctx 511 112.8 / 110.4, 119.0 / 115.4; ctx 1023
-    //     113.8 / 112.1, 119.5 / 119.4; ctx 1200 114.3 / 113.1, 120.2 / 119.8; batch 8, ctx 511 126.1 / 121.3, 132.4 /
-    //     129.0; ctx 1200 127.0 / 127.0, 132.9 / 132.2; 0.993-1.11 times the speed over hidden 1024-8192, 1-8 kv heads.
-    //     Longer: batch 4, ctx 1535 118.7 / 119.0, 126.1 / 127.6; ctx 2047 118.3 / 121.7, 124.8 / 130.5.
-    //   two to four tiles in front of the tcgen05 GEMMs: batch 16, ctx 255 147.8 / 144.4, 152.0 / 152.1; batch 24 156.3 / 157.5,
-    //     163.1 / 160.1; batch 37 164.2 / 161.6, 168.8 / 165.2.  Longer: batch 20, ctx 767 162.3 / 169.9, 166.1 /
-    //     178.0 (half of the SMs without a CTA; batch 37 gains up to 5 % from ctx 400 to 1023, and is not worth a line).
-    //   one tile: an item is then the whole sequence, and nothing is left to merge: batch 16, ctx 60 138.0 / 143.5.
+    // layers with items / with clusters (four layers of an 8B-shaped TP=8 shard, us; bf16 cache, int8 cache):
+    //   two to 20 tiles (16 with four CTAs): batch 1, ctx 511 112.8 / 110.4, 119.0 / 115.4; ctx 1200 114.3 / 113.1, 120.2 /
+    //     119.8; batch 8, ctx 100 124.3 / 122.3, 130.3 / 129.2; ctx 511 126.1 / 121.3, 132.4 / 129.0; ctx 1200 127.0 / 127.0,
+    //     132.9 / 132.2.  0.98-1.11 times the speed over hidden 1024-8192, 1-8 kv heads, the mean 1.02.
+    //   longer: batch 4, ctx 1535 118.7 / 119.0, 126.1 / 127.6; ctx 2047 118.3 / 121.7, 124.8 / 130.5.
+    //   one tile has nothing to merge: batch 8, ctx 63 118.6 / 121.6, 123.9 / 128.7.  (int8 cache: from three tiles up, so
+    //     that a sequence's 64th token changes no plan and captures no graph; two tiles gain 1 % there.)
+    //   in front of the tcgen05 GEMMs they mostly lose: batch 20, ctx 767 162.3 / 169.9, 166.1 / 178.0; batch 16, ctx 63
+    //     137.0 / 144.9, 143.2 / 151.7, ctx 200 147.2 / 145.1, 152.5 / 151.6; batch 37, ctx 767 180.9 / 177.1, 180.1 / 181.0.
     // Sixteen CTAs lose: they only find a place together once the kernel in front has ended (batch 1: 24.6 us a
     // layer against 24.2 with eight).
     int cl = 8;
@@ -670,7 +667,7 @@ int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int n
     for (int b = 0; b < batch; ++b)
         longest = ctx_len_host[b] > longest ? ctx_len_host[b] : longest;
     const int tiles = (longest + 1 + kTileKeys - 1) / kTileKeys;
-    return tiles >= 2 && tiles <= (tensor_path ? 4 : cl == 8 ? 20 : 16) ? cl : 0;
+    return tiles >= (kv8 ? 3 : 2) && tiles <= (cl == 8 ? 20 : 16) ? cl : 0;
 }
 
 cudaError_t launch_attention(const AttnArgs &a, cudaStream_t s)

@@ -240,7 +240,7 @@ void plan_attention(const int32_t *ctx_len_host, int batch, int nkv, int sm_coun
                     int stages = 3, double item_cost = 1.5);
 // Short caches: CTAs per (sequence, kv head) when one cluster each, merging inside the kernel, beats the items of
 // plan_attention and the merge kernel; 0 = the items.
-int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count, bool tensor_path);
+int plan_attention_cluster(const int32_t *ctx_len_host, int batch, int nq, int nkv, int sm_count, bool tensor_path, bool kv8);
 // 2-D uint8 tensor map (rows x cols bytes, cols contiguous), box (box_cols x box_rows), 128-byte swizzle.
 bool encode_u8_map_2d(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint32_t box_cols,
                       uint32_t box_rows);

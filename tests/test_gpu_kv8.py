@@ -32,7 +32,7 @@ def check_appended(dl, ref, name):
         assert (err <= bound).all(), f"{name}:{what} stored entry off by {float((err / bound).max()):.3f} of the bound"
 
 
-def kv8_check(oracle, shape, flags=0, budget=None, cache_seed=0):
+def kv8_check(oracle, shape, flags=0, budget=None, cache_seed=0, cluster=None):
     t = I.make_layers(shape, 1)[0]
     kv = I.make_int8_cache(shape, t["ctx_len"], seed=cache_seed)
     ref = oracle.layer_step(shape, t, int8_weights=bool(flags & P.FLAG_INT8_WEIGHTS), kv8=kv)
@@ -44,6 +44,7 @@ def kv8_check(oracle, shape, flags=0, budget=None, cache_seed=0):
         dl.run()
         assert dl.layer.last_status() == P.PRESERVE_OK
         assert dl.layer.last_status_code() == 0
+        assert cluster is None or dl.layer.attention_cluster_size() == cluster
         out, inter = dl.outputs(), dl.intermediates()
         for name in ("h", "x", "q", "o", "x2", "a"):
             G.assert_close(inter[name], ref[name], f"{shape.name}:{name}")
@@ -91,7 +92,7 @@ def test_int8_cache_matches_the_quantised_oracle(oracle, shape):
 
 
 @pytest.mark.parametrize("shape", [
-    # the cluster form of the attention: its largest range, the first beyond it, fewer tiles than CTAs, four CTAs
+    # short caches of up to 33 tiles, fewer tiles than a cluster has CTAs
     I.small_shape(name="kv8_cl_32_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=2047, ctx_min=0, seed=262),
     I.small_shape(name="kv8_cl_33_tiles", batch=1, n_q_heads=5, n_kv_heads=1, ctx=2048, seed=263),
     I.small_shape(name="kv8_cl_g7", batch=2, n_q_heads=7, n_kv_heads=1, ctx=512, ctx_min=64, seed=264),
@@ -99,6 +100,18 @@ def test_int8_cache_matches_the_quantised_oracle(oracle, shape):
 ], ids=lambda s: s.name)
 def test_int8_cluster_attention_matches_the_quantised_oracle(oracle, shape):
     kv8_check(oracle, shape)
+
+
+@pytest.mark.parametrize("shape,cluster", [
+    (I.small_shape(name="kv8_line_2_tiles", batch=3, n_q_heads=3, n_kv_heads=1, ctx=127, seed=266), 0),
+    (I.small_shape(name="kv8_line_3_tiles", batch=3, n_q_heads=3, n_kv_heads=1, ctx=128, seed=271), 8),
+    (I.small_shape(name="kv8_line_20_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=1279, seed=267), 8),
+    (I.small_shape(name="kv8_line_21_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=1280, seed=268), 0),
+    (I.small_shape(name="kv8_line_cl4", batch=10, n_q_heads=10, n_kv_heads=2, ctx=1023, seed=269), 4),
+    (I.small_shape(name="kv8_line_tensor_path", batch=20, n_q_heads=8, n_kv_heads=1, ctx=255, seed=270), 0),
+], ids=lambda v: getattr(v, "name", str(v)))
+def test_int8_attention_form_at_its_lines(oracle, shape, cluster):
+    kv8_check(oracle, shape, cluster=cluster)
 
 
 @pytest.mark.parametrize("idx", [0, 1, 3, 4])

@@ -15,7 +15,7 @@ import gpu_util as G
 pytestmark = pytest.mark.gpu
 
 
-def full_check(oracle, shape, flags=0, budget=None):
+def full_check(oracle, shape, flags=0, budget=None, cluster=None):
     t = I.make_layers(shape, 1)[0]
     ref = oracle.layer_step(shape, t, int8_weights=bool(flags & P.FLAG_INT8_WEIGHTS))
     dl = G.DeviceLayer(shape, t, flags=flags)
@@ -25,6 +25,7 @@ def full_check(oracle, shape, flags=0, budget=None):
         k_before, v_before = G.cuda_to_bits(dl.k_cache), G.cuda_to_bits(dl.v_cache)
         dl.run()
         assert dl.layer.last_status() == P.PRESERVE_OK
+        assert cluster is None or dl.layer.attention_cluster_size() == cluster
         out, inter = dl.outputs(), dl.intermediates()
         k_new, v_new = dl.appended_kv()
         for name in ("h", "x", "q", "o", "x2", "a"):
@@ -394,9 +395,8 @@ def test_batch_tile_follows_the_step_batch(oracle, batches, flags):
         dl.close()
 
 
-# attention with one cluster per (sequence, kv head): every sequence at most 32 tiles of 64 keys (8 CTAs of 4; 16 tiles
-# with 4 CTAs, from 19 sequence-heads up); the last tile of the range and the first beyond it, fewer tiles than
-# CTAs, groups whose 128 G outputs do not divide into whole heads, an empty cache
+# attention over short caches: groups whose 128 G outputs do not divide into whole heads, fewer tiles than
+# CTAs of a cluster, an empty cache, sequences of up to 33 tiles of 64 keys (LINE_SHAPES has the lines between the forms)
 CLUSTER_SHAPES = [
     I.small_shape(name="cl_g3_32_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=2047, ctx_min=0, seed=62),
     I.small_shape(name="cl_33_tiles", batch=1, n_q_heads=3, n_kv_heads=1, ctx=2048, seed=63),
@@ -412,3 +412,24 @@ CLUSTER_SHAPES = [
 @pytest.mark.parametrize("shape", CLUSTER_SHAPES, ids=[s.name for s in CLUSTER_SHAPES])
 def test_cluster_attention_matches_oracle(oracle, shape):
     full_check(oracle, shape)
+
+
+# (shape, CTAs of the cluster per (sequence, kv head); 0: work items and a merge kernel) on both sides of every line of
+# plan_attention_cluster, for 148 SMs
+LINE_SHAPES = [
+    (I.small_shape(name="line_1_tile", batch=3, n_q_heads=3, n_kv_heads=1, ctx=63, seed=270), 0),
+    (I.small_shape(name="line_2_tiles", batch=2, n_q_heads=8, n_kv_heads=1, ctx=64, seed=271), 8),
+    (I.small_shape(name="line_20_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=1279, seed=272), 8),
+    (I.small_shape(name="line_21_tiles", batch=2, n_q_heads=6, n_kv_heads=2, ctx=1280, seed=273), 0),
+    (I.small_shape(name="line_cl4_16_tiles", batch=10, n_q_heads=10, n_kv_heads=2, ctx=1023, seed=274), 4),
+    (I.small_shape(name="line_cl4_17_tiles", batch=10, n_q_heads=4, n_kv_heads=2, ctx=1024, seed=275), 0),
+    (I.small_shape(name="line_36_streams", batch=12, n_q_heads=3, n_kv_heads=3, ctx=130, seed=276), 4),
+    (I.small_shape(name="line_39_streams", batch=13, n_q_heads=3, n_kv_heads=3, ctx=130, seed=277), 0),
+    (I.small_shape(name="line_g9", batch=2, n_q_heads=9, n_kv_heads=1, ctx=200, seed=278), 0),
+    (I.small_shape(name="line_tensor_path", batch=18, n_q_heads=7, n_kv_heads=1, ctx=255, seed=279), 0),
+]
+
+
+@pytest.mark.parametrize("shape,cluster", LINE_SHAPES, ids=[s.name for s, _ in LINE_SHAPES])
+def test_attention_form_at_its_lines(oracle, shape, cluster):
+    full_check(oracle, shape, cluster=cluster)
