@@ -500,6 +500,10 @@ void plan_step(preserve_layer *L, const StepPtrs &sp, StepPlan *pl)
     // number that enters the graph signature changes as rarely as the launch does)
     if (pl->attn_items_per_stream < 4) pl->attn_items_per_stream = 4;
     if (pl->attn_items_per_stream > 32) pl->attn_items_per_stream = 32;
+    if (pl->attn_cluster) {      // neither enters a launch of the cluster form: no new graph when they change
+        pl->attn_grid = 0;
+        pl->attn_items_per_stream = 4;
+    }
 }
 
 // Queue one layer step on `s` (directly, or into an ongoing capture of `s`).

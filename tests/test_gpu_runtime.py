@@ -143,6 +143,28 @@ def test_layers_wired_output_to_input_without_link(oracle, batch):
             d.close()
 
 
+def test_ragged_short_caches_that_grow_replay_one_graph():
+    """Attention by clusters: sequences of different lengths cross tile boundaries one after another, and the step
+    keeps replaying the graph of its first token (the lengths are read on the device)."""
+    shape = I.small_shape(name="ragged_loop", batch=5, ctx=700, seed=79)
+    t = I.make_layers(shape, 1, nan_fill_tail=False)[0]
+    t["ctx_len"] = np.array([300, 317, 340, 401, 222], np.int32)
+    dl = G.DeviceLayer(shape, t)
+    stream = torch.cuda.Stream()
+    try:
+        for _ in range(140):
+            with torch.cuda.stream(stream):
+                dl.run(stream)
+                dl.ctx_dev += 1
+            assert dl.layer.attention_cluster_size() == 8
+            dl.ctx_host += 1
+        stream.synchronize()
+        assert dl.layer.last_status() == P.PRESERVE_OK
+        assert dl.layer.graph_captures() == 1
+    finally:
+        dl.close()
+
+
 WITHHOLD_CASES = [
     ("window", P.WITHHOLD_WINDOW, dict(batch=3, hidden=2048, ffn=256), 0),
     ("gemv", P.WITHHOLD_GEMV, dict(batch=4), 0),
