@@ -23,6 +23,7 @@ FLAG_INT8_WEIGHTS = 32
 FLAG_INT8_KV = 64
 DEBUG_WITHHOLD, DEBUG_WAIT_LIMIT_CYCLES = 0, 1
 WITHHOLD_WINDOW, WITHHOLD_GEMV, WITHHOLD_TENSOR, WITHHOLD_ATTENTION = 1, 2, 3, 4
+WITHHOLD_ATTENTION_HANDOVER, WITHHOLD_TENSOR_READY = 5, 6
 
 EXPORTS = (
     "preserve_layer_init", "preserve_set_prefetch_bytes", "preserve_set_plan_mode", "preserve_decode_step",

@@ -406,7 +406,7 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
         a.status = L->status;
         a.trace = trace;
         a.pdl = pdl;
-        a.inject = L->inject == INJECT_TC_RING && which == 0 ? INJECT_TC_RING : INJECT_NONE;
+        a.inject = (L->inject == INJECT_TC_RING || L->inject == INJECT_TC_READY) && which == 0 ? L->inject : INJECT_NONE;
         // The gate/up projection takes its input as one fp16 plane (an RMSNorm output is bounded, and 11
         // significant bits keep the SwiGLU output well inside the tolerance): half the activation
         // traffic and half the MMA work of the largest GEMM.  The QKV projection keeps two planes, hi + lo
@@ -684,7 +684,7 @@ int enqueue_step(preserve_layer *L, const StepPtrs &sp, const StepPlan &pl, bool
         a.status = L->status;
         a.trace = TRACE(2);
         a.pdl = pdl;
-        a.inject = L->inject == INJECT_ATTN_RING ? INJECT_ATTN_RING : INJECT_NONE;
+        a.inject = L->inject == INJECT_ATTN_RING || L->inject == INJECT_ATTN_SEND ? L->inject : INJECT_NONE;
         if (L->kv8) {
             a.kv8 = 1;
             a.k_codes = sp.k_cache;
@@ -1266,7 +1266,7 @@ int preserve_debug_set(preserve_layer_t *L, int32_t what, int64_t value)
     if (!L)
         return PRESERVE_EINVAL;
     if (what == PRESERVE_DEBUG_WITHHOLD) {
-        if (value < 0 || value > INJECT_ATTN_RING)
+        if (value < 0 || value > INJECT_TC_READY)
             return PRESERVE_EINVAL;
         L->inject = (int)value;
         return PRESERVE_OK;

@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
     pdl_launch_dependents();
     if constexpr (CL) {
         if (threadIdx.x == 0)
-            cluster_recv_init(rc, p.G, p.cl);
+            cluster_recv_init(rc, p.G, p.cl, p.inject == INJECT_ATTN_SEND && blockIdx.x == 0 ? 8 : 0);
         if (blockIdx.x == 0 && warp == 0)
             cluster_check_items(p.ctx_len, p.B, p.nkv, p.tiles_per_item, p.max_items, p.status);
         __syncthreads();

@@ -71,11 +71,12 @@ struct ClusterRecv {
     uint64_t bar;
     int gave_up;
 };
-__device__ __forceinline__ void cluster_recv_init(ClusterRecv &rc, int G, int cl)      // one thread, before the CTA's barrier
+// (by one thread, before the CTA's barrier; `more` bytes are expected that nobody sends: a test hook)
+__device__ __forceinline__ void cluster_recv_init(ClusterRecv &rc, int G, int cl, uint32_t more)
 {
     mbar_init(&rc.bar, 1);
     mbar_fence_init();
-    mbar_expect_tx(&rc.bar, (uint32_t)(G * 128 * 4 + cl * G * 8));
+    mbar_expect_tx(&rc.bar, (uint32_t)(G * 128 * 4 + cl * G * 8) + more);
     rc.gave_up = 0;
 }
 // balanced runs, the longer ones first (rank 0 is never empty)

@@ -61,7 +61,8 @@ struct GemmTcParams {
     EpilogueArgs epi;
     int *status;
     long long *trace;
-    int inject;         // test hook: the producer of CTA (0, 0) never fetches its first weight tile
+    int inject;         // test hook: the producer of CTA (0, 0) never fetches its first weight tile, or CTA (0, 1) never
+                        // tells CTA (0, 0) that its ring is free
     int planes;         // activation planes in the B operand: 2 = hi + lo, 1 = a single fp16 plane
     int f16;            // both operands are fp16 (else bf16)
     int epi_warps;      // 8 or 16
@@ -609,7 +610,8 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         cluster_wait();       // (the arrival at the top of the kernel: every rank's receive barrier exists)
         if (is_epi) {
             // (behind the wait for the accumulators: the ring has been read)
-            if (in_ring && warp == 2 && lane < p.splits && lane != s)
+            if (in_ring && warp == 2 && lane < p.splits && lane != s &&
+                !(p.inject == INJECT_TC_READY && tile == 0 && s == 1 && lane == 0))
                 mbar_arrive_cluster(cluster_map(&ready_bar, lane));
             // two chunks (four TMEM loads) in flight per wait
             const uint32_t red_row = smem_u32(red) + (uint32_t)row * 4u;

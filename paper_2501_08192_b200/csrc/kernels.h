@@ -57,7 +57,7 @@ inline cudaError_t ensure_dynamic_smem(Fn fn, PerDeviceSize &state, size_t bytes
 // consumer's bounded wait runs out and the give-up path runs.  Nothing faults or hangs: the wait
 // expires after the handle's wait limit and the kernel returns with a status code.
 enum Inject : int { INJECT_NONE = 0, INJECT_WINDOW_HANDOVER = 1, INJECT_GEMV_RING = 2, INJECT_TC_RING = 3,
-                    INJECT_ATTN_RING = 4 };
+                    INJECT_ATTN_RING = 4, INJECT_ATTN_SEND = 5, INJECT_TC_READY = 6 };
 
 // Device status block of a layer (ints): [0] status word (first writer wins), [2..3] the handle's
 // limit on any mbarrier wait in SM cycles (64-bit, 0 = the default below), [8] sink of the

@@ -174,20 +174,25 @@ def test_int8_cache_decode_loop_advances_over_a_tile_boundary(oracle):
         dl.close()
 
 
-def test_int8_cache_withheld_copy_ends_with_a_status(oracle):
-    """The producer of CTA 0 never fetches the key box of its first tile: the consumers' bounded wait
-    gives up, the step returns with a time-out status, and the handle works again afterwards."""
-    shape = I.small_shape(name="kv8_withhold", batch=2, ctx=100, seed=251)
+@pytest.mark.parametrize("what,ctx,cluster", [(P.WITHHOLD_ATTENTION, 100, 0), (P.WITHHOLD_ATTENTION, 200, 8),
+                                             (P.WITHHOLD_ATTENTION_HANDOVER, 200, 8)],
+                         ids=["items", "cluster", "handover"])
+def test_int8_cache_withheld_copy_ends_with_a_status(oracle, what, ctx, cluster):
+    """The producer of CTA 0 never fetches the key box of its first tile, or the first CTA of a cluster waits for
+    more than its peers hand over: the bounded wait gives up, the step returns with a time-out status, and the handle works
+    again afterwards."""
+    shape = I.small_shape(name="kv8_withhold", batch=2, ctx=ctx, seed=251)
     t = I.make_layers(shape, 1)[0]
     kv = I.make_int8_cache(shape, t["ctx_len"])
     ref = oracle.layer_step(shape, t, kv8=kv)
     dl = G.DeviceLayer(shape, t, kv8=kv)
     try:
         dl.layer.debug_set(P.DEBUG_WAIT_LIMIT_CYCLES, 1 << 21)
-        dl.layer.debug_set(P.DEBUG_WITHHOLD, P.WITHHOLD_ATTENTION)
+        dl.layer.debug_set(P.DEBUG_WITHHOLD, what)
         dl.run()
         torch.cuda.synchronize()
         assert dl.layer.last_status() == P.PRESERVE_ETIMEOUT
+        assert dl.layer.attention_cluster_size() == cluster
         dl.layer.debug_set(P.DEBUG_WITHHOLD, 0)
         dl.layer.clear_status()
         dl.run()

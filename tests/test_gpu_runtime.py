@@ -171,7 +171,14 @@ WITHHOLD_CASES = [
     ("tensor", P.WITHHOLD_TENSOR, dict(batch=20), 0),
     # batch 64: the split-K hand-over by bulk copies out of the senders' shared memory
     ("tensor_wide", P.WITHHOLD_TENSOR, dict(batch=64), 0),
+    # batch 128: a QKV projection whose receive area lies in the ring; one rank never says that its ring is free
+    ("tensor_ready", P.WITHHOLD_TENSOR_READY, dict(batch=128, hidden=1024), 0),
     ("attention", P.WITHHOLD_ATTENTION, dict(batch=4), 0),
+    # work items with a merge kernel (22 tiles), clusters (3 tiles), and a cluster whose first CTA waits for more
+    # than its peers hand over
+    ("attention_items", P.WITHHOLD_ATTENTION, dict(batch=4, ctx=1400, ctx_min=1300), 0),
+    ("attention_cluster", P.WITHHOLD_ATTENTION, dict(batch=4, ctx_min=140), 0),
+    ("attention_handover", P.WITHHOLD_ATTENTION_HANDOVER, dict(batch=4, ctx_min=140), 0),
     # int8 weights: the GEMV ring of codes, and the tcgen05 ring in front of the widening warps
     ("gemv_int8", P.WITHHOLD_GEMV, dict(batch=4), P.FLAG_INT8_WEIGHTS),
     ("tensor_int8", P.WITHHOLD_TENSOR, dict(batch=20), P.FLAG_INT8_WEIGHTS),
@@ -183,7 +190,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_survives(oracle, name, 
     """One producer withholds one issue; the consumer's wait (limit shortened to 2^21 SM cycles,
     about a millisecond) runs out, the kernels give up and return, the status says so, and after
     clearing it the same handle computes the right result again."""
-    shape = I.small_shape(name="timeout_" + name, ctx=150, ctx_min=9, seed=74, **kw)
+    shape = I.small_shape(name="timeout_" + name, **dict(dict(ctx=150, ctx_min=9, seed=74), **kw))
     t = I.make_layers(shape, 1)[0]
     ref = oracle.layer_step(shape, t, int8_weights=bool(flags & P.FLAG_INT8_WEIGHTS))
     dl = G.DeviceLayer(shape, t, flags=flags)
@@ -201,6 +208,8 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_survives(oracle, name, 
         assert t0.elapsed_time(t1) < 200.0          # milliseconds: a few expired waits, not a second each
         assert dl.layer.last_status() == P.PRESERVE_ETIMEOUT
         assert dl.layer.last_status() == P.PRESERVE_ETIMEOUT      # sticky until cleared
+        form = {"attention_items": 0, "attention_cluster": 8, "attention_handover": 8}.get(name)
+        assert form is None or dl.layer.attention_cluster_size() == form
         # back to normal: same handle, same buffers
         dl.layer.debug_set(P.DEBUG_WITHHOLD, 0)
         dl.layer.clear_status()
