@@ -370,10 +370,11 @@ def test_info_reports_plan_and_bytes():
 
 
 @pytest.mark.parametrize("flags", [0, P.FLAG_INT8_WEIGHTS], ids=["bf16", "w8"])
-@pytest.mark.parametrize("batches", [(128, (1, 16, 17, 33, 127)), (40, (40, 32, 5, 40))], ids=["max128", "max40"])
+@pytest.mark.parametrize("batches", [(128, (1, 16, 17, 33, 64, 80, 96, 112, 127)), (40, (40, 32, 5, 40))], ids=["max128", "max40"])
 def test_batch_tile_follows_the_step_batch(oracle, batches, flags):
-    """Tensor path with fewer sequences than max_batch: every width of the batch tile (its edges, and one layer
-    going from wide to narrow and back), same tolerance; two KV heads' caches behind the batch stay untouched."""
+    """Tensor path with fewer sequences than max_batch: every width of the batch tile (16, 32, .. 128; one layer
+    going from wide to narrow and back), same tolerance; of the caches exactly the slot ctx_len[b] of the
+    step's sequences changes, to the step's key and value."""
     most, steps = batches
     shape = I.small_shape(name=f"tile_{most}", batch=most, hidden=1024, ffn=640, ctx=70, ctx_min=3, seed=61)
     t = I.make_layers(shape, 1)[0]
@@ -386,11 +387,18 @@ def test_batch_tile_follows_the_step_batch(oracle, batches, flags):
             out = [G.GuardedOut((B, shape.hidden)) for _ in range(3)]
             io = dl.layer.make_io(B, dl.ctx_dev, dl.ctx_host, dl.partials, dl.peers, dl.residual, dl.k_cache,
                                   dl.v_cache, *[o.t for o in out])
+            before = [G.cuda_to_bits(c) for c in (dl.k_cache, dl.v_cache)]
             dl.layer.decode_step(io)
             assert dl.layer.last_status() == P.PRESERVE_OK
             for name, o in zip(("h2", "mlp_partial", "attn_partial"), out):
                 G.assert_close(G.cuda_to_f32(o.t), ref[name], f"batch {B}:{name}")
                 assert o.guards_intact()
+            rows, slots = np.arange(B), dl.ctx_host[:B]
+            for name, c, old in zip(("k_new", "v_new"), (dl.k_cache, dl.v_cache), before):
+                now = G.cuda_to_bits(c)
+                G.assert_close(I.bf16_bits_to_f32(now[rows, :, slots]), ref[name], f"batch {B}:{name}")
+                now[rows, :, slots] = old[rows, :, slots]
+                assert np.array_equal(now, old), f"batch {B}: {name} changed another slot"
     finally:
         dl.close()
 
