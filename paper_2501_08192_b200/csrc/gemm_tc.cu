@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
     // The whole warp walks the stages and waits; one elected lane issues.  The loop is warp-uniform for
     // the compiler (warp index by shuffle, descriptors from uniform values only), so that the operands of
     // the MMAs live in uniform registers.  Issued from a `lane == 0` branch every MMA cost
-    // that thread about 95 cycles whatever its width (four: 390, eight: 620, clock stamps), half of a stage's time:
+    // that thread 78-116 cycles whatever its width (four: 390, eight: 620, eight int8: 927, clock stamps), half of a stage's time:
     // 70B-shaped TP=8 layers at batch 16 72.8 -> 70.2 us, int8 weights at batch 64 125.9 -> 121.6 us per layer.
     auto run_mma = [&](int m_lo, int m_hi) {
         int st = 0, j = 0;               // ring stage and (int8 weights) widened slot of this use, with their phases
