@@ -348,7 +348,8 @@ PRESERVE_API int64_t preserve_graph_captures(const preserve_layer_t *layer);
  * GEMM never fetches its first weight tile; 4: the first attention CTA never fetches one box of
  * its first tile; 5: the first CTA of the first attention cluster waits for eight bytes that no peer hands
  * over (needs attention by clusters); 6: a CTA of the tcgen05 QKV GEMM never tells one peer that its ring is
- * free to receive (needs a receive area in the ring, e.g. batch 128) - so that the consumer's bounded wait runs out, the kernel gives up and returns,
+ * free to receive (needs a receive area in the ring, e.g. batch 128) - so that the consumer's
+ * bounded wait runs out, the kernel gives up and returns,
  * and preserve_last_status reports PRESERVE_ETIMEOUT.  Nothing faults or hangs. */
 #define PRESERVE_DEBUG_WITHHOLD          0
 #define PRESERVE_DEBUG_WAIT_LIMIT_CYCLES 1
