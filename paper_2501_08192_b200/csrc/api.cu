@@ -143,7 +143,6 @@ struct preserve_layer {
     int *ctx_dev;
 
     // tensor path
-    CUtensorMap wmap[4];
     CUtensorMap xmap[8][4];      // x, o, x2, a as B operands, for a batch tile of 16 * (first index + 1) rows
     int nb_pad;                  // max_batch rounded up to 16: rows per plane of the workspaces
 
@@ -396,7 +395,6 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
     const Dims d = layer_dims(L->cfg);
     if (L->tensor_path) {
         GemmTcArgs a = {};
-        a.w_map = L->wmap[which];
         (void)x;
         // The batch tile follows the step's batch, not max_batch: a server sized for 128 sequences that holds
         // 20 otherwise multiplies, fetches and hands over 128 columns in every projection.
@@ -416,7 +414,7 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
         a.x_fp16 = which >= 1 ? 1 : 2;
         a.w8 = L->w8 ? 1 : 0;
         a.scales = L->w8 ? L->scales + L->soff[which] : nullptr;
-        a.w8_codes = L->w8 ? L->arena + L->off[which] : nullptr;
+        a.w = L->arena + L->off[which];
         a.w8_tiles = L->w8 ? gemm_tc_w8_tiles(L->nb_pad, a.N, which >= 1) : 0;    // as the codes were packed
         CK(L, launch_gemm_tc(a, L->sm_count, s));
         return PRESERVE_OK;
@@ -1204,8 +1202,8 @@ int preserve_layer_init(const preserve_layer_config_t *cfg, const preserve_layer
         const void *xb[4] = {L->x, L->o, L->x2, L->a};
         for (int i = 0; i < 4; ++i) {
             // x (two fp16 planes: hi rows, lo rows) feeds the QKV projection; o, x2 and a are one fp16 plane each
-            // (int8 weights are fetched by plain bulk copies: no map over them)
-            bool ok = L->w8 || make_map_2d(&L->wmap[i], L->arena + L->off[i], d.k[i], d.n[i], 64, 128);
+            // (the weights are fetched by plain bulk copies: no maps over them)
+            bool ok = true;
             for (int nb = 16; ok && nb <= L->nb_pad; nb += 16)
                 ok = make_planes_map(&L->xmap[nb / 16 - 1][i], xb[i], d.k[i], L->nb_pad, i >= 1 ? 1 : 2, nb);
             if (!ok) {

@@ -8,8 +8,8 @@
 //
 // Per CTA: one 128-row tile of the packed weights (int8 weights, wide batches: two that share one activation
 // tile) x one slice of k.
-//   warp 0 (+ lane 0 of the first one or two epilogue warps): TMA producers - W tile (128 rows x 64,
-//               128B swizzle) and x tile (2 NB x 64) into a multi-stage shared-memory ring,
+//   warp 0 (+ lane 0 of the first one or two epilogue warps): producers - W tile (128 rows x 64, packed in the
+//               swizzled order of shared memory: one contiguous bulk copy) and x tile (2 NB x 64, TMA, 128B swizzle) into a multi-stage ring,
 //               mbarrier full/empty; the ring's stage uses are dealt round-robin to the issuing threads
 //               (three instead of one measured < 1 %)
 //   warp 1    : allocates TMEM, issues tcgen05.mma (kind::f16, bf16 in, fp32
@@ -47,7 +47,6 @@ constexpr int kTcTileM = 128;
 constexpr int kATileBytes = kTcTileM * kTcBlockK * 2;   // 16 KiB
 
 struct GemmTcParams {
-    CUtensorMap w_map;
     CUtensorMap x_map;
     int B, NB, N, K;
     int mt;             // int8 weights: 128-row weight tiles per CTA (1, or 2 that share one activation tile)
@@ -71,7 +70,7 @@ struct GemmTcParams {
     int w8_early;       // w8: the first ring fill's activation tiles complete their own barrier (codes widened before the wait)
     int w8_slots;       // 2..kTcMaxW8Slots widened tiles in tensor memory (mt * 64 columns each) behind the accumulators, at most `stages`
     const float *wscale;  // w8: one fp32 scale per packed weight row
-    const uint8_t *w8_codes;  // w8: the codes, one contiguous block of mt * 128 rows x 64 bytes per (tile, k-block)
+    const uint8_t *w;   // packed weights: the contiguous tile of (row tile, k block), mt * 16 KiB (pack.cu)
 };
 
 // int8 -> 16-bit widening of two weight codes, exact.  The packed matrix holds every code biased by
@@ -258,12 +257,8 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 mbar_expect_tx(&full[i], kEarly ? a_bytes : stage_bytes);
                 if (p.inject == INJECT_TC_RING && i == 0 && tile == 0 && s == 0)
                     continue;
-                if constexpr (W8)
-                    bulk_load_hint(smem + (size_t)i * stage_bytes, p.w8_codes + ((size_t)tile * p.kblocks + kb0 + i) * a_bytes,
-                                   a_bytes, &full[i], pol);
-                else
-                    tma_load_2d_hint(smem + (size_t)i * stage_bytes, &p.w_map, (kb0 + i) * kTcBlockK,
-                                     tile * mt * kTcTileM, &full[i], pol);
+                bulk_load_hint(smem + (size_t)i * stage_bytes, p.w + ((size_t)tile * p.kblocks + kb0 + i) * a_bytes, a_bytes,
+                               &full[i], pol);
             }
         }
         tma_prefetch_desc(&p.x_map);
@@ -286,6 +281,9 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
 
     const bool is_epi = warp >= 2;
     // ------------------------------------------------------------ TMA producers
+    // A weight tile is one contiguous 16 KiB run of the packed matrix (pack.cu), one bulk copy.  As 128 rows of 128 bytes
+    // out of a row-major matrix (a tiled TMA copy) the same stream was 7-12 % slower in DRAM: gate/up of hidden 8192, ffn 7168
+    // at batch 64 streams its 235 MB in 36.0 us instead of 40.2 (6.5 TB/s), at batch 128 (117 MB) 20.4 instead of 22.8.
     // Weights never depend on earlier kernels, the activations do: fill the whole ring with
     // weight tiles first (they stream in while the previous kernel finishes), then wait for the
     // previous kernel and add the activation tiles.  Producer j of NP owns the stage uses
@@ -324,10 +322,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             if (!mbar_wait(&empty[st], ph ^ 1, p.status, ST_TIMEOUT_EMPTY)) { poisoned = 1; break; }
             uint8_t *a_dst = smem + (size_t)st * stage_bytes;
             mbar_expect_tx(&full[st], stage_bytes);
-            if constexpr (W8)
-                bulk_load_hint(a_dst, p.w8_codes + ((size_t)tile * p.kblocks + kb) * a_bytes, a_bytes, &full[st], pol);
-            else
-                tma_load_2d_hint(a_dst, &p.w_map, kb * kTcBlockK, tile * mt * kTcTileM, &full[st], pol);
+            bulk_load_hint(a_dst, p.w + ((size_t)tile * p.kblocks + kb) * a_bytes, a_bytes, &full[st], pol);
             load_b(st, kb, false);
             st += NP;
             while (st >= p.stages) {
@@ -931,7 +926,6 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     if (a.NB < 16 || a.NB > 128 || a.NB % 16 || a.N % kTcTileM || a.K % (a.w8 ? 2 * kTcBlockK : kTcBlockK) || a.B > a.NB)
         return cudaErrorInvalidValue;
     GemmTcParams p;
-    p.w_map = a.w_map;
     p.x_map = a.x_map;
     p.B = a.B; p.NB = a.NB; p.N = a.N; p.K = a.K;
     p.kblocks = a.K / (a.w8 ? 2 * kTcBlockK : kTcBlockK);
@@ -948,12 +942,12 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     // (from 80 rows up) still lost 2-5 % of a layer at batch 65-112 (hidden 8192, 8 q heads, batch 112: 183.9 -> 176.1 us
     // per two layers; 32 q / 4 kv heads within 0.4 %) and nothing gained at batch 128.
     const int mt = a.w8 ? a.w8_tiles : 1;
-    if (a.w8 && (!a.w8_codes || !a.scales || mt < 1 || mt > 2))
+    if (!a.w || (a.w8 && (!a.scales || mt < 1 || mt > 2)))
         return cudaErrorInvalidValue;
     TcGeometry g;
     if (!tc_geometry(a, sm_count, mt, g))
         return cudaErrorInvalidValue;
-    p.w8_codes = static_cast<const uint8_t *>(a.w8_codes);
+    p.w = static_cast<const uint8_t *>(a.w);
     p.mt = mt;
     const int tiles = g.tiles, stage_bytes = g.stage_bytes, per_sm = g.per_sm, splits = g.splits, w8_slots = g.w8_slots;
     const size_t tile_bytes = g.tile_bytes, smem_cap = g.smem_cap;

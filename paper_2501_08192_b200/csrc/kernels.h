@@ -166,9 +166,8 @@ struct GemvArgs {
 };
 cudaError_t launch_gemv(const GemvArgs &a, int sm_count, cudaStream_t s);
 
-// ---- tcgen05 skinny GEMM (batch >= 16): W [N,K] K-major through TMA
+// ---- tcgen05 skinny GEMM (batch >= 16)
 struct GemmTcArgs {
-    CUtensorMap w_map;    // dims (K, N), box (64, 128), 128B swizzle
     CUtensorMap x_map;    // dims (K, rows, planes), box (64, NB, planes), 128B swizzle: the first NB rows of the hi and
                           // the lo plane - or, with x_fp16 = 1, of the one fp16 plane
     int x_fp16;           // 0: two bf16 planes; 2: two fp16 planes (hi rows then lo rows); 1: the activations are one fp16 plane (inputs that come out of an RMSNorm: bounded,
@@ -179,12 +178,11 @@ struct GemmTcArgs {
     long long *trace;
     int pdl;
     int inject;
-    // int8 weights: the codes come from w8_codes by plain bulk copies (w_map is unused); the
-    // kernel widens every tile to the activations' 16-bit format into tensor memory (the MMA's A operand)
+    const void *w;        // packed weights: contiguous tiles, fetched by plain bulk copies (launch_pack_rows, _w8)
+    // int8 weights: the kernel widens every tile to the activations' 16-bit format into tensor memory (the MMA's A operand)
     // and multiplies every accumulator row by its scale
     int w8;
     const float *scales;  // w8: [N] in packed row order
-    const void *w8_codes; // w8: the packed codes (launch_pack_rows_w8 with w8_tiles * 128 rows per block)
     int w8_tiles;         // w8: 128-row tiles per packed block and CTA (gemm_tc_w8_tiles of the largest batch)
 };
 // int8 weights: 128-row weight tiles per CTA for a matrix of N rows and a padded batch of NB (the packed
