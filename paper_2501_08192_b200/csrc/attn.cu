@@ -85,7 +85,7 @@ template <bool NARROW, bool CL = false>
 __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const __grid_constant__ AttnParams p)
 {
     extern __shared__ uint8_t smem_raw[];
-    AttnSmem &sm = *reinterpret_cast<AttnSmem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    AttnSmem &sm = *reinterpret_cast<AttnSmem *>(align_smem(smem_raw, 1024));
     __shared__ typename std::conditional<CL, ClusterRecv, int>::type rc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int streams = p.B * p.nkv;

@@ -141,7 +141,7 @@ template <bool CL>
 __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv_kv8(const __grid_constant__ AttnKv8Params p)
 {
     extern __shared__ uint8_t smem_raw[];
-    AttnKv8Smem &sm = *reinterpret_cast<AttnKv8Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    AttnKv8Smem &sm = *reinterpret_cast<AttnKv8Smem *>(align_smem(smem_raw, 1024));
     __shared__ typename std::conditional<CL, ClusterRecv, int>::type rc;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int streams = p.B * p.nkv;

@@ -64,6 +64,15 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// First multiple of `align` in dynamic shared memory.  (An offset and not a rounded address: the compiler then still
+// knows that the pointer is one into shared memory, and reads through it with ld.shared instead of generic loads: eight 8B-shaped
+// TP=8 layers at batch 8 266.6 -> 262.3 us, batch 5 with int8 261.0 -> 254.9, two 70B-shaped TP=4 layers with int8 at batch 64
+// 234.0 -> 228.6, one small layer 24.6 -> 23.6.)
+__device__ __forceinline__ uint8_t *align_smem(uint8_t *raw, uint32_t align)
+{
+    return raw + (-smem_u32(raw) & (align - 1));
+}
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {

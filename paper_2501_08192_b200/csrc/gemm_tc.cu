@@ -185,7 +185,7 @@ template <int KIND, int PUSH, bool W8 = false, bool EARLY = false>
 __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_constant__ GemmTcParams p)
 {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = align_smem(smem_raw, 1024);
     __shared__ uint64_t full[kTcMaxStages], empty[kTcMaxStages], accum_bar, push_bar, ready_bar;
     __shared__ uint64_t conv[kTcMaxW8Slots], slot_free[kTcMaxW8Slots];   // int8 weights: a widened tile is complete / has been consumed
     // int8 weights: the activation tiles of the ring's FIRST fill complete a barrier of their own, so that

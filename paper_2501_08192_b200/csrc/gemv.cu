@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
     __shared__ EpilogueTables tabs;
     __shared__ float scale_s[W8 ? kGemvWarps * RB * 16 : 1];   // W8: the scales of the group's rows
     extern __shared__ uint8_t gemv_smem_raw[];
-    uint8_t *wsm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(gemv_smem_raw) + 127) & ~uintptr_t(127));
+    uint8_t *wsm = align_smem(gemv_smem_raw, 128);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
