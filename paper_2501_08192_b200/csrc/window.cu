@@ -24,7 +24,7 @@ namespace cg = cooperative_groups;
 
 namespace prsv {
 
-constexpr int kWinMaxChunks = 2;   // 8-element chunks per thread
+constexpr int kWinMaxThreads = 512; // one 8-element chunk per thread: a row of 16384 is cut into at least four CTAs
 constexpr int kWinMaxCluster = 8;  // CTAs per row
 constexpr int kWinMaxCtas = 256;   // rows are cut into fewer, larger CTAs where there are many rows
 
@@ -79,7 +79,10 @@ __device__ __forceinline__ uint4 ld_volatile_v4(const void *p)
 }
 
 // (One instantiation for all four input forms: the two windows of a layer then run the same
-// instructions, which the second finds in the instruction caches.)
+// instructions, which the second finds in the instruction caches.  The same caches pay for every instruction that a
+// layer's kernels do without: one chunk per thread instead of up to two, and the rolled loop over the partials beyond
+// the first burst, make 16 KB of this kernel's 30; 70B-shaped TP=8 layers at batch 20 lose 1.7 %, 8B-shaped ones at
+// batch 5 with int8 weights 1.5 % of their time.)
 // LEAN, for big batches (hundreds of CTAs): one chunk per thread and the step's input buffers are only
 // hinted into L2 before the wait and loaded after it, so that a CTA holds few registers while it
 // waits - the grid then fits beside the early-launched GEMM CTAs in one wave instead of several.  For the same
@@ -96,26 +99,24 @@ __device__ __forceinline__ uint4 ld_volatile_v4(const void *p)
 // buffer only after it has passed window B of the same layer, by which time every peer has
 // announced its window-B buffer and therefore finished reading window A.
 template <bool LEAN, bool COMM = false>
-__global__ void __launch_bounds__(512, LEAN ? 2 : 1) k_window_reduce_rmsnorm(const __grid_constant__ WindowParams p)
+__global__ void __launch_bounds__(kWinMaxThreads, LEAN ? 2 : 1) k_window_reduce_rmsnorm(const __grid_constant__ WindowParams p)
 {
-    constexpr int kWinMaxChunks = LEAN ? 1 : prsv::kWinMaxChunks;
     const bool RESID_F32 = p.resid_f32 != 0, PART0_F32 = p.part0_f32 != 0;
     const int row = blockIdx.x / p.cluster, rank = blockIdx.x % p.cluster;
     const int chunks = (p.H >> 3) / p.cluster;   // uint4 chunks of this CTA's slice of the row
     const size_t row_off = (size_t)row * (p.H >> 3) + (size_t)rank * chunks;
     const int gain_off = rank * chunks;
-    float v[kWinMaxChunks][8];
-    uint4 gn[kWinMaxChunks];
+    float v[8];
+    uint4 gn = make_uint4(0, 0, 0, 0);
+    const int ch = threadIdx.x;
+    const bool mine = ch < chunks;
     float ss = 0.f;
 
     // the gain does not depend on the previous kernel: fetch it before waiting (LEAN: behind the sums, where
     // its registers are free again)
     auto load_gain = [&]() {
-#pragma unroll
-        for (int c = 0; c < kWinMaxChunks; ++c) {
-            const int ch = threadIdx.x + c * blockDim.x;
-            gn[c] = ch < chunks ? ld_cached(p.gain + gain_off + ch) : make_uint4(0, 0, 0, 0);
-        }
+        if (mine)
+            gn = ld_cached(p.gain + gain_off + ch);
     };
     if constexpr (!LEAN)
         load_gain();
@@ -141,20 +142,16 @@ __global__ void __launch_bounds__(512, LEAN ? 2 : 1) k_window_reduce_rmsnorm(con
     // previous kernel either: their loads - the only ones that go to HBM - are issued before the
     // wait, up to 8 partial buffers per chunk.
     constexpr int kBurst = LEAN ? 4 : 8;
-    uint4 pre[kWinMaxChunks][kBurst], pre_res[kWinMaxChunks];
+    uint4 pre[kBurst], pre_res;
     auto load_part = [&](int j, size_t at) { return COMM ? ld_volatile_v4(p.parts[j] + at) : ld_stream(p.parts[j] + at); };
     auto load_inputs = [&]() {
+        if (mine) {
+            if (!RESID_F32)
+                pre_res = ld_stream(reinterpret_cast<const uint4 *>(p.resid) + row_off + ch);
 #pragma unroll
-        for (int c = 0; c < kWinMaxChunks; ++c) {
-            const int ch = threadIdx.x + c * blockDim.x;
-            if (ch < chunks) {
-                if (!RESID_F32)
-                    pre_res[c] = ld_stream(reinterpret_cast<const uint4 *>(p.resid) + row_off + ch);
-#pragma unroll
-                for (int j = 0; j < kBurst; ++j)
-                    if (j < p.n_parts && !(PART0_F32 && j == 0))
-                        pre[c][j] = load_part(j, row_off + ch);
-            }
+            for (int j = 0; j < kBurst; ++j)
+                if (j < p.n_parts && !(PART0_F32 && j == 0))
+                    pre[j] = load_part(j, row_off + ch);
         }
     };
     if constexpr (LEAN && !COMM) {
@@ -211,51 +208,49 @@ __global__ void __launch_bounds__(512, LEAN ? 2 : 1) k_window_reduce_rmsnorm(con
     if constexpr (LEAN)
         load_inputs();
 
-#pragma unroll
-    for (int c = 0; c < kWinMaxChunks; ++c) {
-        const int ch = threadIdx.x + c * blockDim.x;
-        if (ch < chunks) {
-            if (RESID_F32) {
-                const float4 *r = reinterpret_cast<const float4 *>(p.resid) + (row_off + ch) * 2;
-                float4 a = r[0], b = r[1];
-                v[c][0] = a.x; v[c][1] = a.y; v[c][2] = a.z; v[c][3] = a.w;
-                v[c][4] = b.x; v[c][5] = b.y; v[c][6] = b.z; v[c][7] = b.w;
-            } else {
-                const uint4 r = pre_res[c];
-                v[c][0] = bf_lo(r.x); v[c][1] = bf_hi(r.x); v[c][2] = bf_lo(r.y); v[c][3] = bf_hi(r.y);
-                v[c][4] = bf_lo(r.z); v[c][5] = bf_hi(r.z); v[c][6] = bf_lo(r.w); v[c][7] = bf_hi(r.w);
-            }
-            if (PART0_F32) {     // partial 0 handed over in fp32 (own result / previous layer of a chain)
-                const float4 *r = reinterpret_cast<const float4 *>(p.parts[0]) + (row_off + ch) * 2;
-                float4 a = r[0], b = r[1];
-                v[c][0] += a.x; v[c][1] += a.y; v[c][2] += a.z; v[c][3] += a.w;
-                v[c][4] += b.x; v[c][5] += b.y; v[c][6] += b.z; v[c][7] += b.w;
-            }
-#pragma unroll
-            for (int j = 0; j < kBurst; ++j)
-                if (j < p.n_parts && !(PART0_F32 && j == 0)) {
-                    const uint4 r = pre[c][j];
-                    v[c][0] += bf_lo(r.x); v[c][1] += bf_hi(r.x); v[c][2] += bf_lo(r.y); v[c][3] += bf_hi(r.y);
-                    v[c][4] += bf_lo(r.z); v[c][5] += bf_hi(r.z); v[c][6] += bf_lo(r.w); v[c][7] += bf_hi(r.w);
-                }
-            // (more partial buffers than one burst: the rest in bursts)
-            for (int q0 = kBurst; q0 < p.n_parts; q0 += kBurst) {
-                uint4 r[kBurst];
-#pragma unroll
-                for (int j = 0; j < kBurst; ++j)
-                    if (q0 + j < p.n_parts)
-                        r[j] = load_part(q0 + j, row_off + ch);
-#pragma unroll
-                for (int j = 0; j < kBurst; ++j)
-                    if (q0 + j < p.n_parts) {
-                        v[c][0] += bf_lo(r[j].x); v[c][1] += bf_hi(r[j].x); v[c][2] += bf_lo(r[j].y); v[c][3] += bf_hi(r[j].y);
-                        v[c][4] += bf_lo(r[j].z); v[c][5] += bf_hi(r[j].z); v[c][6] += bf_lo(r[j].w); v[c][7] += bf_hi(r[j].w);
-                    }
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                ss += v[c][i] * v[c][i];
+    if (mine) {
+        if (RESID_F32) {
+            const float4 *r = reinterpret_cast<const float4 *>(p.resid) + (row_off + ch) * 2;
+            float4 a = r[0], b = r[1];
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+            v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+        } else {
+            const uint4 r = pre_res;
+            v[0] = bf_lo(r.x); v[1] = bf_hi(r.x); v[2] = bf_lo(r.y); v[3] = bf_hi(r.y);
+            v[4] = bf_lo(r.z); v[5] = bf_hi(r.z); v[6] = bf_lo(r.w); v[7] = bf_hi(r.w);
         }
+        if (PART0_F32) {     // partial 0 handed over in fp32 (own result / previous layer of a chain)
+            const float4 *r = reinterpret_cast<const float4 *>(p.parts[0]) + (row_off + ch) * 2;
+            float4 a = r[0], b = r[1];
+            v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
+            v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+        }
+#pragma unroll
+        for (int j = 0; j < kBurst; ++j)
+            if (j < p.n_parts && !(PART0_F32 && j == 0)) {
+                const uint4 r = pre[j];
+                v[0] += bf_lo(r.x); v[1] += bf_hi(r.x); v[2] += bf_lo(r.y); v[3] += bf_hi(r.y);
+                v[4] += bf_lo(r.z); v[5] += bf_hi(r.z); v[6] += bf_lo(r.w); v[7] += bf_hi(r.w);
+            }
+        // (more partial buffers than one burst)
+        constexpr int kRest = LEAN ? 4 : 2;
+#pragma unroll 1
+        for (int q0 = kBurst; q0 < p.n_parts; q0 += kRest) {
+            uint4 r[kRest];
+#pragma unroll
+            for (int j = 0; j < kRest; ++j)
+                if (q0 + j < p.n_parts)
+                    r[j] = load_part(q0 + j, row_off + ch);
+#pragma unroll
+            for (int j = 0; j < kRest; ++j)
+                if (q0 + j < p.n_parts) {
+                    v[0] += bf_lo(r[j].x); v[1] += bf_hi(r[j].x); v[2] += bf_lo(r[j].y); v[3] += bf_hi(r[j].y);
+                    v[4] += bf_lo(r[j].z); v[5] += bf_hi(r[j].z); v[6] += bf_lo(r[j].w); v[7] += bf_hi(r[j].w);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            ss += v[i] * v[i];
     }
 
     if constexpr (LEAN)
@@ -293,8 +288,9 @@ __global__ void __launch_bounds__(512, LEAN ? 2 : 1) k_window_reduce_rmsnorm(con
         row_total = 0.f;
         recv_short = !mbar_wait(&recv_bar, 0, p.status, ST_TIMEOUT_FULL);
         if (!recv_short)
-            for (int q = 0; q < p.cluster; ++q)
-                row_total += recv[q];
+#pragma unroll
+            for (int q = 0; q < kWinMaxCluster; ++q)
+                row_total += q < p.cluster ? recv[q] : 0.f;
     }
     const float inv = rsqrtf(row_total / (float)p.H + p.eps);
 
@@ -306,66 +302,62 @@ __global__ void __launch_bounds__(512, LEAN ? 2 : 1) k_window_reduce_rmsnorm(con
         }
     }
 
+    if (mine) {
+        if (p.h_f32) {
+            float4 *o = reinterpret_cast<float4 *>(p.h_f32) + (row_off + ch) * 2;
+            o[0] = make_float4(v[0], v[1], v[2], v[3]);
+            o[1] = make_float4(v[4], v[5], v[6], v[7]);
+        }
+        if (p.h_bf16) {
+            uint4 o;
+            o.x = pack_bf16(v[0], v[1]); o.y = pack_bf16(v[2], v[3]);
+            o.z = pack_bf16(v[4], v[5]); o.w = pack_bf16(v[6], v[7]);
+            p.h_bf16[row_off + ch] = o;
+        }
+        // x is kept as a pair of bf16 planes, x = hi + lo, so the GEMM that consumes it
+        // sees ~16 mantissa bits although its operands are bf16
+        const uint4 g = gn;
+        float xv[8];
+        xv[0] = v[0] * inv * bf_lo(g.x); xv[1] = v[1] * inv * bf_hi(g.x);
+        xv[2] = v[2] * inv * bf_lo(g.y); xv[3] = v[3] * inv * bf_hi(g.y);
+        xv[4] = v[4] * inv * bf_lo(g.z); xv[5] = v[5] * inv * bf_hi(g.z);
+        xv[6] = v[6] * inv * bf_lo(g.w); xv[7] = v[7] * inv * bf_hi(g.w);
+        if (p.x_fp16 == 2) {
+            // hi = fp16(x), lo = fp16(x - hi): the operand format of the tensor path's QKV projection
+            uint4 hi, lo;
+            uint32_t *hw = &hi.x, *lw = &lo.x;
 #pragma unroll
-    for (int c = 0; c < kWinMaxChunks; ++c) {
-        const int ch = threadIdx.x + c * blockDim.x;
-        if (ch < chunks) {
-            if (p.h_f32) {
-                float4 *o = reinterpret_cast<float4 *>(p.h_f32) + (row_off + ch) * 2;
-                o[0] = make_float4(v[c][0], v[c][1], v[c][2], v[c][3]);
-                o[1] = make_float4(v[c][4], v[c][5], v[c][6], v[c][7]);
+            for (int i = 0; i < 4; ++i) {
+                const float a0 = fminf(fmaxf(xv[2 * i], -65504.f), 65504.f);
+                const float a1 = fminf(fmaxf(xv[2 * i + 1], -65504.f), 65504.f);
+                const __half2 h2 = __floats2half2_rn(a0, a1);
+                const float2 hf = __half22float2(h2);
+                const __half2 l2 = __floats2half2_rn(a0 - hf.x, a1 - hf.y);
+                hw[i] = *reinterpret_cast<const uint32_t *>(&h2);
+                lw[i] = *reinterpret_cast<const uint32_t *>(&l2);
             }
-            if (p.h_bf16) {
-                uint4 o;
-                o.x = pack_bf16(v[c][0], v[c][1]); o.y = pack_bf16(v[c][2], v[c][3]);
-                o.z = pack_bf16(v[c][4], v[c][5]); o.w = pack_bf16(v[c][6], v[c][7]);
-                p.h_bf16[row_off + ch] = o;
-            }
-            // x is kept as a pair of bf16 planes, x = hi + lo, so the GEMM that consumes it
-            // sees ~16 mantissa bits although its operands are bf16
-            const uint4 g = gn[c];
-            float xv[8];
-            xv[0] = v[c][0] * inv * bf_lo(g.x); xv[1] = v[c][1] * inv * bf_hi(g.x);
-            xv[2] = v[c][2] * inv * bf_lo(g.y); xv[3] = v[c][3] * inv * bf_hi(g.y);
-            xv[4] = v[c][4] * inv * bf_lo(g.z); xv[5] = v[c][5] * inv * bf_hi(g.z);
-            xv[6] = v[c][6] * inv * bf_lo(g.w); xv[7] = v[c][7] * inv * bf_hi(g.w);
-            if (p.x_fp16 == 2) {
-                // hi = fp16(x), lo = fp16(x - hi): the operand format of the tensor path's QKV projection
-                uint4 hi, lo;
-                uint32_t *hw = &hi.x, *lw = &lo.x;
+            p.x_bf16[row_off + ch] = hi;
+            p.x_bf16[p.x_plane + row_off + ch] = lo;
+        } else if (p.x_fp16) {
+            // normalised activations are bounded (|x| <= sqrt(H) * |gain|): one fp16 plane carries 11
+            // significant bits; clamped to the fp16 range so that an absurd gain cannot make an infinity
+            uint4 o;
+            uint32_t *ow = &o.x;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float a0 = fminf(fmaxf(xv[2 * i], -65504.f), 65504.f);
-                    const float a1 = fminf(fmaxf(xv[2 * i + 1], -65504.f), 65504.f);
-                    const __half2 h2 = __floats2half2_rn(a0, a1);
-                    const float2 hf = __half22float2(h2);
-                    const __half2 l2 = __floats2half2_rn(a0 - hf.x, a1 - hf.y);
-                    hw[i] = *reinterpret_cast<const uint32_t *>(&h2);
-                    lw[i] = *reinterpret_cast<const uint32_t *>(&l2);
-                }
-                p.x_bf16[row_off + ch] = hi;
-                p.x_bf16[p.x_plane + row_off + ch] = lo;
-            } else if (p.x_fp16) {
-                // normalised activations are bounded (|x| <= sqrt(H) * |gain|): one fp16 plane carries 11
-                // significant bits; clamped to the fp16 range so that an absurd gain cannot make an infinity
-                uint4 o;
-                uint32_t *ow = &o.x;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const __half2 h2 = __floats2half2_rn(fminf(fmaxf(xv[2 * i], -65504.f), 65504.f),
-                                                         fminf(fmaxf(xv[2 * i + 1], -65504.f), 65504.f));
-                    ow[i] = *reinterpret_cast<const uint32_t *>(&h2);
-                }
-                p.x_bf16[row_off + ch] = o;
-            } else {
-                uint4 hi, lo;
-                split_bf16x2(xv[0], xv[1], hi.x, lo.x);
-                split_bf16x2(xv[2], xv[3], hi.y, lo.y);
-                split_bf16x2(xv[4], xv[5], hi.z, lo.z);
-                split_bf16x2(xv[6], xv[7], hi.w, lo.w);
-                p.x_bf16[row_off + ch] = hi;
-                p.x_bf16[p.x_plane + row_off + ch] = lo;
+            for (int i = 0; i < 4; ++i) {
+                const __half2 h2 = __floats2half2_rn(fminf(fmaxf(xv[2 * i], -65504.f), 65504.f),
+                                                     fminf(fmaxf(xv[2 * i + 1], -65504.f), 65504.f));
+                ow[i] = *reinterpret_cast<const uint32_t *>(&h2);
             }
+            p.x_bf16[row_off + ch] = o;
+        } else {
+            uint4 hi, lo;
+            split_bf16x2(xv[0], xv[1], hi.x, lo.x);
+            split_bf16x2(xv[2], xv[3], hi.y, lo.y);
+            split_bf16x2(xv[4], xv[5], hi.z, lo.z);
+            split_bf16x2(xv[6], xv[7], hi.w, lo.w);
+            p.x_bf16[row_off + ch] = hi;
+            p.x_bf16[p.x_plane + row_off + ch] = lo;
         }
     }
     if constexpr (COMM) {
@@ -430,9 +422,7 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
     // at batch 37-64 and cost up to 7 % there: three layers of hidden 6144, batch 48 155.5 -> 166.2 us, hidden 7168,
     // batch 56 179.0 -> 190.7; the two counts agree at hidden 2048, 4096 and 8192.)
     const bool comm = a.comm_rank >= 0;
-    const bool lean = (a.B * uncut > kWinMaxCtas || a.inputs_after_wait || comm) && chunks <= 512;
-    if ((a.inputs_after_wait || comm) && !lean)
-        return cudaErrorInvalidValue;
+    const bool lean = a.B * uncut > kWinMaxCtas || a.inputs_after_wait || comm;
     if (comm && (a.n_parts > 8 || a.part0_is_f32 || a.comm_rank >= a.n_parts))
         return cudaErrorInvalidValue;
     p.no_hint = a.inputs_after_wait;
@@ -445,11 +435,8 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
         p.comm_flags_peer[i] = a.comm_flags_peer[i];
     p.comm_epoch = a.comm_epoch;
     p.comm_done = a.comm_done;
-    int threads = (chunks + kWinMaxChunks - 1) / kWinMaxChunks;
-    if (chunks <= 512)
-        threads = chunks;
-    threads = ((threads + 31) / 32) * 32;
-    if (threads > 512 || threads * kWinMaxChunks < chunks)
+    const int threads = ((chunks + 31) / 32) * 32;
+    if (threads > kWinMaxThreads)
         return cudaErrorInvalidValue;
 
     cudaLaunchConfig_t cfg = {};
