@@ -79,8 +79,10 @@ __device__ __forceinline__ void load_epilogue_tables(const EpilogueArgs &e, Epil
 {
     if (e.kind != EPI_QKV)
         return;
+#pragma unroll 1
     for (int i = threadIdx.x; i < nb && i < 128; i += blockDim.x)
         t.pos[i] = e.ctx_len[b0 + i];
+#pragma unroll 1
     for (int i = threadIdx.x; i < kHeadDim / 2; i += blockDim.x)
         t.inv_freq[i] = e.inv_freq ? e.inv_freq[i] : 0.0;
 }
