@@ -454,6 +454,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_decode_splitkv(const _
             cluster_wait();          // (the arrival in the prologue: every rank's receive barrier exists)
         // two head dims per consumer thread, the heads of one parity per half of the threads
         const int d2 = threadIdx.x & 63;
+#pragma unroll 1
         for (int r = threadIdx.x >> 6; r < p.G; r += 2) {
             float M = -INFINITY;
 #pragma unroll
@@ -514,6 +515,7 @@ __global__ void __launch_bounds__(kMergeMaxWarps * 32) k_attn_merge(const __grid
     pdl_launch_dependents();
     // first item of this stream: parallel count over the streams before it (lengths are inputs)
     int cnt = 0;
+#pragma unroll 1
     for (int s2 = tid; s2 < sidx; s2 += blockDim.x) {
         const int nt = tiles_of(p.ctx_len[s2 / p.nkv]);
         cnt += (nt + p.tiles_per_item - 1) / p.tiles_per_item;
@@ -526,6 +528,7 @@ __global__ void __launch_bounds__(kMergeMaxWarps * 32) k_attn_merge(const __grid
     const int n_items = (tiles_of(p.ctx_len[b]) + p.tiles_per_item - 1) / p.tiles_per_item;
     __syncthreads();
     int base = 0;
+#pragma unroll 4
     for (int i = 0; i < n_warps; ++i)
         base += cnt_s[i];
     pdl_wait();    // the partials come from the split-KV kernel (every CTA waits, also those with nothing to do)
@@ -533,6 +536,7 @@ __global__ void __launch_bounds__(kMergeMaxWarps * 32) k_attn_merge(const __grid
     if (n_items > 1) {          // a single item was finished by the split-KV kernel itself
         float Mg = -INFINITY, L = 0.f;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
         for (int e = warp; e < n_items && base + e < p.max_items; e += n_warps) {
             const size_t ent = (size_t)(base + e) * p.G + row;
             const float2 ml = *reinterpret_cast<const float2 *>(p.part_ml + ent * 2);

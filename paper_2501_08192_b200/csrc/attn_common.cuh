@@ -18,12 +18,16 @@ __device__ __forceinline__ void consumer_barrier()
 
 __device__ __forceinline__ int tiles_of(int ctx) { return (ctx + 1 + kTileKeys - 1) / kTileKeys; }
 
+// (Loops that run once per kernel or item are kept rolled: unrolled by default they were 6 KB of each attention
+// kernel's 33-48, and what a layer's kernels execute competes for the instruction caches.)
+
 // First item index of every stream, computed identically by every CTA: the lengths are
 // fetched by all threads at once (one memory round trip), then warp 0 scans them.
 template <typename Params>
 __device__ __forceinline__ void build_item_table(const Params &p, int *item_base)
 {
     const int streams = p.B * p.nkv;
+#pragma unroll 1
     for (int i = threadIdx.x; i < streams; i += blockDim.x) {
         const int nt = tiles_of(p.ctx_len[i / p.nkv]);
         item_base[i + 1] = (nt + p.tiles_per_item - 1) / p.tiles_per_item;
@@ -31,6 +35,7 @@ __device__ __forceinline__ void build_item_table(const Params &p, int *item_base
     __syncthreads();
     if (threadIdx.x < 32) {
         int carry = 0;
+#pragma unroll 1
         for (int base = 0; base < streams; base += 32) {
             const int i = base + threadIdx.x;
             int v = i < streams ? item_base[i + 1] : 0;
@@ -104,13 +109,16 @@ __device__ __forceinline__ void cluster_finish(ClusterRecv &rc, int G, int cl, i
     } else {
         trace_waited(tr);
         const int L = G * 128 / cl;
+#pragma unroll 1
         for (int i = 2 * tid; i < L; i += 2 * kConsumerWarps * 32) {
             const int e = rank * L + i, r = e >> 7;
             float M = -INFINITY;
+#pragma unroll 4
             for (int c = 0; c < cl; ++c)
                 M = fmaxf(M, rc.ml[c * G + r][0]);
             float2 acc = make_float2(0.f, 0.f);
             float l = 0.f;
+#pragma unroll 4
             for (int c = 0; c < cl; ++c) {                    // rank order
                 const float mc = rc.ml[c * G + r][0];
                 const float w = mc == -INFINITY ? 0.f : exp2f(mc - M);
@@ -141,6 +149,7 @@ __device__ __forceinline__ void cluster_finish(ClusterRecv &rc, int G, int cl, i
 __device__ __forceinline__ void cluster_check_items(const int *ctx_len, int B, int nkv, int tiles_per_item, int max_items, int *status)
 {
     int n = 0;
+#pragma unroll 1
     for (int b = threadIdx.x & 31; b < B; b += 32)
         n += nkv * ((tiles_of(ctx_len[b]) + tiles_per_item - 1) / tiles_per_item);
 #pragma unroll
