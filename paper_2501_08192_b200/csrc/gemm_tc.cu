@@ -210,8 +210,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
     const int b_bytes = p.planes * p.NB * kBlk * 2;
     const int stage_bytes = a_bytes + b_bytes;
     const int acc_cols = p.planes * p.NB;      // TMEM columns of one weight tile's accumulator
-    const int kb0 = (int)((long long)p.kblocks * s / p.splits);
-    const int kb1 = (int)((long long)p.kblocks * (s + 1) / p.splits);
+    const int kb0 = p.kblocks * s / p.splits, kb1 = p.kblocks * (s + 1) / p.splits;
 
     // MMA-issuing threads (see run_mma): two for the int8 kernels with two weight tiles and sixteen epilogue warps
     // (the last of them is then not needed as a converter)
@@ -219,12 +218,14 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
     trace_start(p.trace);
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
+#pragma unroll 1
         for (int i = 0; i < p.stages; ++i) {
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], n_issuers);
         }
         mbar_init(&accum_bar, n_issuers);
         if (kEarly) {
+#pragma unroll 1
             for (int i = 0; i < p.stages; ++i)
                 mbar_init(&fullb[i], 1);
         }
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             const uint64_t pol = policy_evict_first();   // every weight byte is read once per step
             const int n_kb = kb1 - kb0;
             const int pre = n_kb < p.stages ? n_kb : p.stages;
+#pragma unroll 1
             for (int i = 0; i < pre; ++i) {
                 mbar_expect_tx(&full[i], kEarly ? a_bytes : stage_bytes);
                 if (p.inject == INJECT_TC_RING && i == 0 && tile == 0 && s == 0)
@@ -309,14 +311,17 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 tma_load_3d(b_dst, &p.x_map, kb_ * kBlk, 0, 0, &full[st_]);
             }
         };
+#pragma unroll 1
         for (int i = prod; i < pre; i += NP)
             load_b(i, kb0 + i, kEarly);
         int it = prod;
+#pragma unroll 1
         while (it < pre)
             it += NP;
         // (stage and phase of use `it` are kept incrementally: no division on this thread's path)
         int st = it % p.stages;
         uint32_t ph = (uint32_t)(it / p.stages) & 1;
+#pragma unroll 1
         for (; it < n_kb; it += NP) {
             const int kb = kb0 + it;
             if (!mbar_wait(&empty[st], ph ^ 1, p.status, ST_TIMEOUT_EMPTY)) { poisoned = 1; break; }
@@ -325,6 +330,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             bulk_load_hint(a_dst, p.w + ((size_t)tile * p.kblocks + kb) * a_bytes, a_bytes, &full[st], pol);
             load_b(st, kb, false);
             st += NP;
+#pragma unroll 1
             while (st >= p.stages) {
                 st -= p.stages;
                 ph ^= 1;
@@ -346,6 +352,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         int st = 0, j = 0;               // ring stage and (int8 weights) widened slot of this use, with their phases
         uint32_t ph = 0, phj = 0;
         const uint32_t smem_base = smem_u32(smem);
+#pragma unroll 1
         for (int kb = kb0; kb < kb1; ++kb) {
             // (int8 weights: the widened tile of this use completes after the stage has landed)
             bool got = W8 ? mbar_wait(&conv[j], phj, p.status, ST_TIMEOUT_FULL)
@@ -360,6 +367,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             const uint64_t bdesc = make_smem_desc(st_addr + a_bytes);
             const uint32_t more = kb > kb0 ? 1u : 0u;
             if (elect_one()) {
+#pragma unroll 1
                 for (int m = m_lo; m < m_hi; ++m) {
                     // each 128-row weight tile has its own accumulator (planes * NB TMEM columns)
                     if constexpr (W8) {
@@ -389,13 +397,17 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             if (++st == p.stages) { st = 0; ph ^= 1; }
         }
     };
-    if (warp == 0) {
-        if (lane == 0)
-            run_producer(0);
-    } else if (warp == 1) {
-        run_mma(0, n_issuers == 2 ? 1 : mt);
+    // (int8 weights: below, in one copy with the roles of the epilogue warps - 7 KB less code, 1 % of a layer at batch 64; for
+    // 16-bit weights, whose producer and issuer should start at once, that was 1 % slower at batch 16 and 20)
+    if constexpr (!W8) {
+        if (warp == 0) {
+            if (lane == 0)
+                run_producer(0);
+        } else if (warp == 1) {
+            run_mma(0, 1);
+        }
+        __syncwarp();
     }
-    __syncwarp();
 
     // ---------------------------------------------------------------- epilogue
     // Accumulator column b holds the hi-plane product of batch row b, column NB + b the
@@ -455,17 +467,14 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             apply_epilogue_t<KIND>(p.epi, tabs, b, true, p.N, b, pair, v0, v1);
         }
     };
-    // the first epilogue warps lend their lane 0 to the ring (the warp reconverges behind the block)
-    if (is_epi && warp - 1 < p.producers) {
+    // the first epilogue warps lend their lane 0 to the ring, the last one may issue MMAs (the warps reconverge behind the block)
+    const bool issuer2 = W8 && n_issuers == 2 && warp == 1 + p.epi_warps;
+    if ((W8 && warp == 0) || (is_epi && warp - 1 < p.producers)) {
         if (lane == 0)
-            run_producer(warp - 1);
-        __syncwarp();
-    }
-    else if (is_epi && W8 && n_issuers == 2 && warp == 1 + p.epi_warps) {
-        run_mma(1, 2);
-        __syncwarp();
-    }
-    else if (is_epi && W8) {
+            run_producer(warp == 0 ? 0 : warp - 1);
+    } else if (W8 && (warp == 1 || issuer2)) {
+        run_mma(issuer2 ? 1 : 0, issuer2 || n_issuers == 1 ? mt : 1);
+    } else if (W8) {
         // ---------------------------------------------------- int8 weights: widen every tile
         // Tile use `itc` is widened from its ring stage into tensor-memory slot itc % slots, where the
         // MMA takes it as its A operand: row r of a weight tile in TMEM lane r, 64 columns per 128 k.
@@ -545,8 +554,8 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             if (++j == p.w8_slots) { j = 0; phj ^= 1; reuse = true; }
             if (++st == p.stages) { st = 0; ph ^= 1; }
         }
-        __syncwarp();
     }
+    __syncwarp();
     bool have = false;
     if (is_epi) {
         have = mbar_wait(&accum_bar, 0, p.status, ST_TIMEOUT_MMA);
@@ -610,6 +619,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 mbar_arrive_cluster(cluster_map(&ready_bar, lane));
             // two chunks (four TMEM loads) in flight per wait
             const uint32_t red_row = smem_u32(red) + (uint32_t)row * 4u;
+#pragma unroll 1
             for (int j = sub; j < mt * nchunks; j += 2 * kSubs) {
                 const int j1 = j + kSubs;
                 const bool two = j1 < mt * nchunks;
@@ -682,6 +692,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 }
                 int m = 0, cl = warp - 2;
                 while (cl >= cols) { cl -= cols; ++m; }
+#pragma unroll 1
                 for (int k = 0; m < mt; ++k) {
                     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -727,6 +738,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
         const uint32_t src_stride = (uint32_t)mt * kTcTileM * cols * 4u;          // bytes per source rank
         cluster_wait();       // (the arrival at the top of the kernel: every rank's receive barrier exists)
         if (is_epi) {
+#pragma unroll 1
             for (int j = sub; j < mt * nchunks; j += kSubs) {
                 const int m = j / nchunks, c = j % nchunks;
                 float v[16];
@@ -763,6 +775,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 const int hp = cols / 2;                   // column pairs per m
                 int m = 0, c2 = sub;
                 while (c2 >= hp) { c2 -= hp; ++m; }
+#pragma unroll 1
                 for (int k = 0; m < mt; ++k) {
                     const uint32_t a = row_a + m * mstr + c2 * 8u;
                     float mine[2] = {0.f, 0.f};
@@ -788,6 +801,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 finish(std::integral_constant<int, 8>());
         }
     } else if (is_epi) {
+#pragma unroll 1
         for (int j = sub; j < mt * nchunks; j += kSubs) {
             const int m = j / nchunks, c = j % nchunks;
             const int pair = ((tile * mt + m) * kTcTileM + row) >> 1;
