@@ -31,12 +31,13 @@
 // finishes the outputs - or, when a CTA handles several groups, through
 // distributed shared memory with every rank finishing its share of the outputs.
 // The fused epilogues live in epilogue.cuh.
-// The kernel runs four times a layer for microseconds, so its instructions are a cost of their own: one copy of the
-// epilogues, loops outside the weight stream rolled, no 64-bit divisions and no cooperative-groups calls make 30 KB of
-// 50: four layers of hidden 2688 at batch 3 110.2 -> 104.8 us, eight 8B-shaped TP=8 layers at batch 5 with int8 weights
-// 251.6 -> 243.2, at batch 8 within 0.5 %.  (A refill of the ring once per burst instead of once per slot makes
-// 26 KB and costs 2 % at batch 8.  A further instantiation beside this one - four row blocks per warp for gate/up - made every
-// other kernel of the layer slower while this one had 50 KB: batch 8 266 -> 289 us.)
+// The kernel runs four times a layer for microseconds, so the instructions it executes are a cost of their own (they compete
+// with the other kernels' for the instruction caches): loops outside the weight stream are rolled and the hand-over
+// without clusters' helpers is in plain instructions - four layers of hidden 2688 at batch 3 106.0 -> 101.5 us, eight
+// 8B-shaped TP=8 layers at batch 5 with int8 244.3 -> 234.2, at batch 8 258.7 -> 253.9, layers of hidden 8192 at batch 8 within 0.6 %.
+// (One copy of the epilogues for the three hand-over forms makes 30 KB of 39 and costs up to 2 % of the longer
+// streams.  A further instantiation beside this one - four row blocks per warp for gate/up - made every other kernel of the
+// layer slower: batch 8 266 -> 289 us.)
 #include "epilogue.cuh"
 
 namespace prsv {
@@ -107,10 +108,11 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
 
     // this warp's run of k-chunks: part ki of ks = splits * warps_k equal parts (same for every group)
     const int ks = p.splits * p.warps_k, ki = s * p.warps_k + wk;
-    const int c_begin = p.kchunks * ki / ks;
-    const int c_end = p.kchunks * (ki + 1) / ks;
+    const int c_begin = (int)((long long)p.kchunks * ki / ks);
+    const int c_end = (int)((long long)p.kchunks * (ki + 1) / ks);
     uint8_t *ring = wsm + (size_t)warp * (p.slots * kUnitChunks * 1024);
     const uint32_t slot_mask = (uint32_t)p.slots - 1;
+    const uint32_t ring_a = smem_u32(ring);
 
     trace_start(p.trace);
     pdl_launch_dependents();    // the next kernel may start its own weight fetch right away
@@ -257,8 +259,9 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                         const uint32_t ph = (n_consumed >> (p.slots == 4 ? 2 : p.slots - 1)) & 1;
                         ok = mbar_wait(&bars[warp][slot], ph, p.status, ST_TIMEOUT_FULL);
                         if (ok) {
-                            const uint4 *wtile =
-                                reinterpret_cast<const uint4 *>(ring + slot * (kUnitChunks * 1024)) + lane * 2;
+                            // (explicit ld.shared by 32-bit address, in program order: 1-2 % of a layer from batch 5 up
+                            // against loads that the compiler places)
+                            const uint32_t wt = ring_a + (uint32_t)(slot * (kUnitChunks * 1024)) + lane * 32u;
                             // PACK: a unit's products are summed by the tensor cores from zero and added to the
                             // running sum in fp32.  (The tensor cores' own accumulation truncates: over a
                             // warp's whole run the SwiGLU output of hidden 8192 was 3.1e-6 off its float64 value, with
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
 #pragma unroll
                             for (int u = 0; u < kUnitChunks; ++u)
                                 if (uu * kUnitChunks + u < nb) {
-                                    const uint4 wl = wtile[u * 64], wh = wtile[u * 64 + 1];
+                                    const uint4 wl = lds_u32x4(wt + u * 1024), wh = lds_u32x4(wt + u * 1024 + 16);
                                     compute(PACK ? d : acc[r], wl, wh, xq[uu * kUnitChunks + u]);
                                 }
                             if constexpr (PACK) {
@@ -324,26 +327,20 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
             const int b = i % NB, row = (i / NB) % 16, rl = i / (16 * NB);
             const int wrow = rl / RB, r = rl % RB;       // warp row of the CTA, row block of that warp
             float v = 0.f;
-#pragma unroll 1
-            for (int k = 0; k < p.warps_k; k += 4) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)          // (four loads in flight)
-                    v += k + j < p.warps_k ? red[(wrow * p.warps_k + k + j) & (kGemvWarps - 1)][r * 16 + row][b] : 0.f;
-            }
+            for (int k = 0; k < p.warps_k; ++k)
+                v += red[wrow * p.warps_k + k][r * 16 + row][b];
             cta_part[rl][row][b] = v;
         }
 
         // ---- sum over the cluster ranks (fixed order)
-        const bool pull = p.splits > 1 && !p.push;
-        const float *recv = reinterpret_cast<const float *>(wsm + p.recv_off);
-        __syncthreads();
-        if (pull) {
-            cluster_sync();
-        } else if (p.push) {
+        const int n_out = rbs_per_cta * 8 * NB;          // (row block, pair, batch row) triples of the group
+        if (p.splits > 1 && p.push) {
             // One-sided: ranks 1.. store their partial sums into rank 0's shared memory, signalling its
             // barrier with the bytes, and are done; rank 0 waits for all the bytes and finishes every
             // output.  No cluster barrier on the critical path.  (One group per CTA in this mode.)
+            __syncthreads();
             cluster_wait();       // (the arrival in the prologue: rank 0's barrier exists)
+            float *recv = reinterpret_cast<float *>(wsm + p.recv_off);
             if (s != 0) {
                 const uint32_t dst = cluster_map(recv + (size_t)(s - 1) * part_floats, 0);
                 const uint32_t bar = cluster_map(&push_bar, 0);
@@ -355,47 +352,64 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                 const bool got = mbar_wait(&push_bar, 0, p.status, ST_TIMEOUT_FULL);
                 push_short = !got;
                 ok = got && ok;
-            }
-        }
-        // ---- finish: (row block, pair, batch row) triples of the group; without a hand-over every rank takes its share.
-        // (One copy of the epilogues for all three forms: they are most of the kernel's instructions.)
-        const int n_out = rbs_per_cta * 8 * NB;
-        const int ranks = pull ? p.splits : 1;
 #pragma unroll 1
-        for (int i = threadIdx.x * ranks + (pull ? s : 0); i < n_out && (pull || s == 0); i += blockDim.x * ranks) {
-            const int b = i % NB, r = (i / NB) % 8, rl = i / (8 * NB);
-            if (b >= p.B)
-                continue;
-            const int at = (rl * 16 + r) * NB + b;
-            float v0 = 0.f, v1 = 0.f;
-            if (pull) {
+                for (int i = threadIdx.x; i < n_out; i += blockDim.x) {
+                    const int b = i % NB, r = (i / NB) % 8, rl = i / (8 * NB);
+                    if (b >= p.B)
+                        continue;
+                    float v0 = cta_part[rl][r][b], v1 = cta_part[rl][r + 8][b];
+#pragma unroll 1
+                    for (int q = 1; q < p.splits; ++q) {
+                        v0 += recv[(size_t)(q - 1) * part_floats + (rl * 16 + r) * NB + b];
+                        v1 += recv[(size_t)(q - 1) * part_floats + (rl * 16 + r + 8) * NB + b];
+                    }
+                    if constexpr (W8) {
+                        v0 *= scale_s[rl * 16 + r];
+                        v1 *= scale_s[rl * 16 + r + 8];
+                    }
+                    apply_epilogue(p.epi, tabs, b, false, p.N, p.b0 + b, (grp * rbs_per_cta + rl) * 8 + r, v0, v1);
+                }
+            }
+        } else if (p.splits > 1) {
+            // every rank finishes its share of the outputs, reading all ranks' partial sums
+            cluster_sync();
+#pragma unroll 1
+            for (int i = threadIdx.x * p.splits + s; i < n_out; i += blockDim.x * p.splits) {
+                const int b = i % NB, r = (i / NB) % 8, rl = i / (8 * NB);
+                if (b >= p.B)
+                    continue;
+                float v0 = 0.f, v1 = 0.f;
 #pragma unroll 1
                 for (int q = 0; q < p.splits; ++q) {
-                    const uint32_t remote = cluster_map(&cta_part[0][0][0] + at, q);
+                    const uint32_t remote = cluster_map(&cta_part[0][0][0] + (rl * 16 + r) * NB + b, q);
                     v0 += ld_cluster_f32(remote);
                     v1 += ld_cluster_f32(remote + 8 * NB * 4);
                 }
-            } else {
-                v0 = cta_part[rl][r][b];
-                v1 = cta_part[rl][r + 8][b];
-#pragma unroll 1
-                for (int q = 0; q < p.splits - 1; ++q) {
-                    v0 += recv[(size_t)q * part_floats + at];
-                    v1 += recv[(size_t)q * part_floats + at + 8 * NB];
+                if constexpr (W8) {
+                    v0 *= scale_s[rl * 16 + r];
+                    v1 *= scale_s[rl * 16 + r + 8];
                 }
+                apply_epilogue(p.epi, tabs, b, false, p.N, p.b0 + b, (grp * rbs_per_cta + rl) * 8 + r, v0, v1);
             }
-            if constexpr (W8) {
-                v0 *= scale_s[rl * 16 + r];
-                v1 *= scale_s[rl * 16 + r + 8];
-            }
-            apply_epilogue(p.epi, tabs, b, false, p.N, p.b0 + b, (grp * rbs_per_cta + rl) * 8 + r, v0, v1);
-        }
-        if (pull)
             cluster_sync();   // peers' shared memory must outlive the reads; also fences red/cta_part reuse
-        else if (!p.push)
-            __syncthreads();
-        if (!p.push)
             load_scales(grp + gridDim.x);
+        } else {
+            __syncthreads();
+#pragma unroll 1
+            for (int i = threadIdx.x; i < n_out; i += blockDim.x) {
+                const int b = i % NB, r = (i / NB) % 8, rl = i / (8 * NB);
+                if (b >= p.B)
+                    continue;
+                float v0 = cta_part[rl][r][b], v1 = cta_part[rl][r + 8][b];
+                if constexpr (W8) {
+                    v0 *= scale_s[rl * 16 + r];
+                    v1 *= scale_s[rl * 16 + r + 8];
+                }
+                apply_epilogue(p.epi, tabs, b, false, p.N, p.b0 + b, (grp * rbs_per_cta + rl) * 8 + r, v0, v1);
+            }
+            __syncthreads();
+            load_scales(grp + gridDim.x);
+        }
     }
     if (p.push && s == 0) {
         // Rank 0 gave up waiting for a rank's partial sums: that rank may still store them into this
