@@ -610,6 +610,7 @@ int enqueue_step(preserve_layer *L, const StepPtrs &sp, const StepPlan &pl, bool
         w.B = B; w.H = H;
         w.trace = TRACE(0);
         w.delay_ns = L->window_delay_ns;
+        w.sm_count = L->sm_count;
         w.status = L->status;
         // Launched directly, the first kernel of a call must not start before everything queued on
         // the stream earlier has finished: it reads its input buffers ahead of the dependency wait,
@@ -746,6 +747,7 @@ int enqueue_step(preserve_layer *L, const StepPtrs &sp, const StepPlan &pl, bool
         w.B = B; w.H = H;
         w.trace = TRACE(5);
         w.delay_ns = L->window_delay_ns;
+        w.sm_count = L->sm_count;
         w.status = L->status;
         w.pdl = pdl;
         w.inputs_after_wait = sp.late_b;

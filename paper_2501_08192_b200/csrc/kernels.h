@@ -88,6 +88,7 @@ struct WindowArgs {
     long long *trace;              // optional timeline slot (kTraceSlots values), see common.cuh
     int delay_ns;                  // modelled communication latency added to the window (0 = none)
     int *status;                   // device status block (bounded waits report here)
+    int sm_count;
     int pdl;                       // launch with the programmatic-serialization attribute
     int inputs_after_wait;         // the step's input buffers may still be written by an earlier kernel of the
                                    // same call: read them only after the dependency wait

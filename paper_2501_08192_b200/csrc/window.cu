@@ -83,8 +83,7 @@ __device__ __forceinline__ uint4 ld_volatile_v4(const void *p)
 // layer's kernels do without: one chunk per thread instead of up to two, and the rolled loop over the partials beyond
 // the first burst, make 16 KB of this kernel's 30; 70B-shaped TP=8 layers at batch 20 lose 1.7 %, 8B-shaped ones at
 // batch 5 with int8 weights 1.5 % of their time.)
-// LEAN, for big batches (hundreds of CTAs): one chunk per thread and the step's input buffers are only
-// hinted into L2 before the wait and loaded after it, so that a CTA holds few registers while it
+// LEAN, for big batches (see the launcher): the step's input buffers are only hinted into L2 before the wait and loaded after it, so that a CTA holds few registers while it
 // waits - the grid then fits beside the early-launched GEMM CTAs in one wave instead of several.  For the same
 // reason the partial buffers come in bursts of four and the gain last (at most 64 registers; at 42 it spills).
 // COMM: the real communication window - the partial-sum buffers are the ranks' exchange buffers
@@ -416,13 +415,13 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
     while (cl < uncut && ((a.H / 8) / cl > 512 || a.B * cl * 2 <= kWinMaxCtas)) cl *= 2;
     p.cluster = cl;
     const int chunks = a.H / 8 / cl;
-    // LEAN (inputs read after the wait, at most 64 registers: 389.1 -> 378.1 us there) for big batches, where the
-    // CTAs would be more than 256 without the limit above, and whenever an input buffer may still be
-    // written by an earlier kernel of the same call.  (Counted in threads instead, from 32768 up, it took in hidden 5120-7168
-    // at batch 37-64 and cost up to 7 % there: three layers of hidden 6144, batch 48 155.5 -> 166.2 us, hidden 7168,
-    // batch 56 179.0 -> 190.7; the two counts agree at hidden 2048, 4096 and 8192.)
+    // LEAN (inputs read after the wait, 64 registers) for grids that do not find room in one wave otherwise - at 72
+    // registers a CTA of up to 448 threads fits an SM twice, a larger one once - and whenever an input buffer may still be
+    // written by an earlier kernel of the same call.  Three layers, LEAN -> not: hidden 8192, batch 33 175.9 -> 168.4 us,
+    // batch 64 196.1 -> 190.8, batch 72 197.9 -> 192.3 (144 CTAs of 512 threads); batch 80 (160 CTAs) 199.5 -> 201.0, batch 128
+    // 230.8 -> 245.3; hidden 4096, batch 128 (256 CTAs of 256) 186.3 -> 183.0; hidden 5120, batch 112 188.8 -> 184.0.
     const bool comm = a.comm_rank >= 0;
-    const bool lean = a.B * uncut > kWinMaxCtas || a.inputs_after_wait || comm;
+    const bool lean = a.B * cl > a.sm_count * (chunks > 448 ? 1 : 2) || a.inputs_after_wait || comm;
     if (comm && (a.n_parts > 8 || a.part0_is_f32 || a.comm_rank >= a.n_parts))
         return cudaErrorInvalidValue;
     p.no_hint = a.inputs_after_wait;

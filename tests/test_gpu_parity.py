@@ -83,6 +83,14 @@ def test_small_shapes_match_oracle(oracle, shape):
     full_check(oracle, shape)
 
 
+@pytest.mark.parametrize("batch,hidden", [(72, 8192), (80, 8192), (128, 8192), (128, 4096), (100, 5120)])
+def test_window_forms_at_their_line(oracle, batch, hidden):
+    """The window kernel holds its inputs while it waits as long as its grid fits the SMs in one wave (148 SMs: 144 CTAs of
+    512 threads, 256 of 256, 200 of 320) and reads them after the wait beyond that (160 and 256 CTAs of 512 threads)."""
+    full_check(oracle, I.small_shape(name="window_form", batch=batch, hidden=hidden, ffn=128, ctx=20, ctx_min=3, n_q_heads=2,
+                                     n_kv_heads=2, tp_degree=3, seed=58))
+
+
 @pytest.mark.parametrize("idx", [0, 1, 3, 4])
 def test_benchmark_configs_match_oracle(oracle, idx):
     # (with the side-stream L2 prefetch running: a budget of 16 MiB per window; the library's default
