@@ -617,59 +617,79 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             if (in_ring && warp == 2 && lane < p.splits && lane != s &&
                 !(p.inject == INJECT_TC_READY && tile == 0 && s == 1 && lane == 0))
                 mbar_arrive_cluster(cluster_map(&ready_bar, lane));
-            // two chunks (four TMEM loads) in flight per wait
+            // The columns of the other ranks first, so that they travel while this rank's own are staged.  Two chunks (four
+            // TMEM loads) in flight per wait.
             const uint32_t red_row = smem_u32(red) + (uint32_t)row * 4u;
+            const int own_c0 = (s * cols + 15) / 16, own_n = max((s + 1) * cols / 16 - own_c0, 0);     // chunks that are all this rank's
+            auto stage = [&](bool own) {
+                const int n_c = own ? own_n : nchunks - own_n;
+                auto chunk = [&](int j, int &m, int &c) {
+                    m = j / n_c;
+                    c = j - m * n_c;
+                    c = own ? c + own_c0 : c < own_c0 ? c : c + own_n;
+                };
 #pragma unroll 1
-            for (int j = sub; j < mt * nchunks; j += 2 * kSubs) {
-                const int j1 = j + kSubs;
-                const bool two = j1 < mt * nchunks;
-                const int m0 = j / nchunks, c0 = j % nchunks;
-                const int m1 = two ? j1 / nchunks : m0, c1 = two ? j1 % nchunks : c0;
-                uint32_t h0[16], l0[16], h1[16], l1[16];
-                if (have) {
-                    tc_ld16_issue(t_lane + m0 * acc_cols + c0 * 16, h0);
-                    tc_ld16_issue(t_lane + m1 * acc_cols + c1 * 16, h1);
-                    if (p.planes == 2) {
-                        tc_ld16_issue(t_lane + m0 * acc_cols + p.NB + c0 * 16, l0);
-                        tc_ld16_issue(t_lane + m1 * acc_cols + p.NB + c1 * 16, l1);
+                for (int j = sub; j < mt * n_c; j += 2 * kSubs) {
+                    const bool two = j + kSubs < mt * n_c;
+                    int m0, c0, m1, c1;
+                    chunk(j, m0, c0);
+                    chunk(two ? j + kSubs : j, m1, c1);
+                    uint32_t h0[16], l0[16], h1[16], l1[16];
+                    if (have) {
+                        tc_ld16_issue(t_lane + m0 * acc_cols + c0 * 16, h0);
+                        tc_ld16_issue(t_lane + m1 * acc_cols + c1 * 16, h1);
+                        if (p.planes == 2) {
+                            tc_ld16_issue(t_lane + m0 * acc_cols + p.NB + c0 * 16, l0);
+                            tc_ld16_issue(t_lane + m1 * acc_cols + p.NB + c1 * 16, l1);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i)
+                                l0[i] = l1[i] = 0u;
+                        }
+                        tc_ld_wait4(h0, l0, h1, l1);
                     } else {
 #pragma unroll
                         for (int i = 0; i < 16; ++i)
-                            l0[i] = l1[i] = 0u;
+                            h0[i] = l0[i] = h1[i] = l1[i] = 0u;
                     }
-                    tc_ld_wait4(h0, l0, h1, l1);
-                } else {
+                    const uint32_t a0 = red_row + (uint32_t)((m0 * p.NB + c0 * 16) * kTcTileM) * 4u;
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
-                        h0[i] = l0[i] = h1[i] = l1[i] = 0u;
+                        sts_f32(a0 + i * (kTcTileM * 4), (__uint_as_float(h0[i]) + __uint_as_float(l0[i])) * wscale_of(m0));
+                    if (two) {
+                        const uint32_t a1 = red_row + (uint32_t)((m1 * p.NB + c1 * 16) * kTcTileM) * 4u;
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            sts_f32(a1 + i * (kTcTileM * 4), (__uint_as_float(h1[i]) + __uint_as_float(l1[i])) * wscale_of(m1));
+                    }
                 }
-                const uint32_t a0 = red_row + (uint32_t)((m0 * p.NB + c0 * 16) * kTcTileM) * 4u;
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    sts_f32(a0 + i * (kTcTileM * 4), (__uint_as_float(h0[i]) + __uint_as_float(l0[i])) * wscale_of(m0));
-                if (two) {
-                    const uint32_t a1 = red_row + (uint32_t)((m1 * p.NB + c1 * 16) * kTcTileM) * 4u;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        sts_f32(a1 + i * (kTcTileM * 4), (__uint_as_float(h1[i]) + __uint_as_float(l1[i])) * wscale_of(m1));
+            };
+            // (one copy of the code for both passes)
+#pragma unroll 1
+            for (int pass = 0; pass < (own_n > 0 ? 2 : 1); ++pass) {
+                stage(pass == 1);
+                if (pass == 0) {
+                    fence_proxy_async_smem();
+                    asm volatile("bar.sync 1, %0;" ::"r"(kSubs * 128) : "memory");
+                    // copy e is issued by lane e / n_warps of epilogue warp e % n_warps: spread over the warps,
+                    // the (splits - 1) * mt copies go out side by side
+                    const int n_ewarps = kSubs * 4;
+                    const int e = lane < 8 ? (warp - 2) + lane * n_ewarps : 1 << 30;
+                    if (e < (p.splits - 1) * mt && in_ring && !mbar_wait(&ready_bar, 0, p.status, ST_TIMEOUT_MMA)) {
+                        poisoned = 1;      // (a peer that is this late gets nothing: its own wait records it)
+                    } else if (e < (p.splits - 1) * mt) {
+                        const int slot_q = e / mt, m = e % mt;
+                        const int q = slot_q < s ? slot_q : slot_q + 1;      // owner
+                        const int my_slot = s < q ? s : s - 1;               // where the owner keeps this rank's share
+                        bulk_copy_to_cluster(cluster_map(recv + ((size_t)(my_slot * mt + m) * cols) * kTcTileM, q),
+                                             smem_u32(red + ((size_t)m * p.NB + q * cols) * kTcTileM),
+                                             (uint32_t)cols * kTcTileM * 4u, cluster_map(&push_bar, q));
+                    }
+                    __syncwarp();
                 }
             }
-            fence_proxy_async_smem();
-            asm volatile("bar.sync 1, %0;" ::"r"(kSubs * 128) : "memory");
-            // copy e is issued by lane e / n_warps of epilogue warp e % n_warps: spread over the warps,
-            // the (splits - 1) * mt copies go out side by side
-            const int n_ewarps = kSubs * 4;
-            const int e = lane < 8 ? (warp - 2) + lane * n_ewarps : 1 << 30;
-            if (e < (p.splits - 1) * mt && in_ring && !mbar_wait(&ready_bar, 0, p.status, ST_TIMEOUT_MMA)) {
-                poisoned = 1;      // (a peer that is this late gets nothing: its own wait records it)
-            } else if (e < (p.splits - 1) * mt) {
-                const int slot_q = e / mt, m = e % mt;
-                const int q = slot_q < s ? slot_q : slot_q + 1;      // owner
-                const int my_slot = s < q ? s : s - 1;               // where the owner keeps this rank's share
-                bulk_copy_to_cluster(cluster_map(recv + ((size_t)(my_slot * mt + m) * cols) * kTcTileM, q),
-                                     smem_u32(red + ((size_t)m * p.NB + q * cols) * kTcTileM),
-                                     (uint32_t)cols * kTcTileM * 4u, cluster_map(&push_bar, q));
-            }
+            if (own_n > 0)
+                asm volatile("bar.sync 1, %0;" ::"r"(kSubs * 128) : "memory");    // own columns staged by all epilogue warps
             if (!mbar_wait(&push_bar, 0, p.status, ST_TIMEOUT_MMA))
                 poisoned = 1;
         }
