@@ -415,6 +415,7 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
         a.w8 = L->w8 ? 1 : 0;
         a.scales = L->w8 ? L->scales + L->soff[which] : nullptr;
         a.w = L->arena + L->off[which];
+        a.w8_early = L->cfg.hidden < 8192;
         a.w8_tiles = L->w8 ? gemm_tc_w8_tiles(L->nb_pad, a.N, which >= 1) : 0;    // as the codes were packed
         CK(L, launch_gemm_tc(a, L->sm_count, s));
         return PRESERVE_OK;

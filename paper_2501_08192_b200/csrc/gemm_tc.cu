@@ -987,8 +987,12 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     const size_t tile_bytes = g.tile_bytes, smem_cap = g.smem_cap;
     int stages = g.stages;
     p.w8_slots = w8_slots;
-    // (measured: pays for narrow batches - two CTAs per SM, few stages per CTA - and costs ~1 % on wide ones)
-    p.w8_early = a.w8 && g.w8_two;
+    // Codes widened before the dependency wait: always for narrow batches (two CTAs per SM, few stages per CTA), and for wide ones
+    // where the layer's weights are small enough for it to matter - two layers of hidden 2048, batch 20 of 128 78.7 -> 71.7 us,
+    // hidden 4096, batch 48 103.8 -> 97.9, hidden 7168, batch 48 147.2 -> 140.5, batch 128 within 1 %; hidden 8192, batch 48 and
+    // 64 1.6 % and 1.8 % slower.  One answer for all projections of a layer: two instantiations side by side cost more
+    // than either (the caches of instructions).
+    p.w8_early = a.w8 && (g.w8_two || a.w8_early);
     p.w8 = a.w8;
     p.wscale = a.scales;
     p.splits = splits;

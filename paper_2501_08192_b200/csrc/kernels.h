@@ -184,6 +184,7 @@ struct GemmTcArgs {
     // and multiplies every accumulator row by its scale
     int w8;
     const float *scales;  // w8: [N] in packed row order
+    int w8_early;         // w8, wide batches: widen the ring's first codes before the dependency wait
     int w8_tiles;         // w8: 128-row tiles per packed block and CTA (gemm_tc_w8_tiles of the largest batch)
 };
 // int8 weights: 128-row weight tiles per CTA for a matrix of N rows and a padded batch of NB (the packed

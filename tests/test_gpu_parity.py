@@ -137,6 +137,13 @@ def test_int8_weights_on_benchmark_configs(oracle, idx):
         assert np.array_equal(bits[k], again[k]), k          # prefetch never changes results, int8 included
 
 
+@pytest.mark.parametrize("batch,hidden", [(33, 8064), (33, 8192), (128, 8064), (128, 8192)])
+def test_int8_weights_of_wide_batches_at_the_line_of_early_widening(oracle, batch, hidden):
+    """Wide batches widen the first codes of a projection before its dependency wait below hidden 8192."""
+    full_check(oracle, I.small_shape(name="w8_early", batch=batch, hidden=hidden, ffn=256, ctx=40, ctx_min=3, n_q_heads=2,
+                                     n_kv_heads=1, seed=59), flags=P.FLAG_INT8_WEIGHTS)
+
+
 def test_int8_weights_on_either_path_report_one_byte_per_weight():
     for flags, tensor in ((P.FLAG_INT8_WEIGHTS, 1), (P.FLAG_INT8_WEIGHTS | P.FLAG_FORCE_GEMV, 0)):
         s = I.small_shape(batch=20, ctx=50, seed=151)
