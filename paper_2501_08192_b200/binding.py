@@ -433,7 +433,7 @@ def preserve_measure_stream(buf, n_bytes: int, passes: int, path: int, ctas: int
 
 def preserve_measure_stream_tma(buf, n_bytes: int, passes: int, ctas: int, stages: int, box_rows: int,
                                 producers: int, status, stream=None) -> float:
-    """GB/s of 2-D tiled TMA loads (the tcgen05 GEMM's weight loads) over `buf` (see preserve.h)."""
+    """GB/s of 2-D tiled TMA loads (weight tiles out of a row-major matrix) over `buf` (see preserve.h)."""
     out = C.c_float()
     _check(lib().preserve_measure_stream_tma(_ptr(buf), n_bytes, passes, ctas, stages, box_rows, producers,
                                              _ptr(status), _stream_ptr(stream), C.byref(out)),

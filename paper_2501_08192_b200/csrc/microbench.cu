@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(32 * kStreamMaxProducers) k_stream_bulk(const 
     }
 }
 
-// path 3: the tcgen05 GEMM's weight loads - 2-D tiled TMA copies (128-byte swizzle) of boxes of 64 columns x
+// path 3: weight tiles out of a row-major matrix - 2-D tiled TMA copies (128-byte swizzle) of boxes of 64 columns x
 // `rows` rows out of a [n_rows, 8192] bf16 matrix (row stride 16 KiB): CTA c walks the 128 column blocks of
 // row tile c mod n_tiles, `passes` times; producer w of the CTA takes the column blocks w, w + producers, ...
 struct StreamTmaParams {
