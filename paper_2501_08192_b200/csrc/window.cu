@@ -14,6 +14,7 @@
 // produces (this shard's own partial sum, the fp32 residual) is read after it.
 // The kernel stays narrow (at most 8 B small CTAs): during a real allreduce the
 // SMs idle, which is what leaves HBM bandwidth to the prefetch stream.
+#include <atomic>
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
@@ -388,6 +389,28 @@ __global__ void __launch_bounds__(kWinMaxThreads, LEAN ? 2 : 1) k_window_reduce_
     trace_end(p.trace);
 }
 
+// CTAs of `threads` threads of the held-inputs form that an SM has room for, counted up to two.  Asked of the device
+// (once per block size): it follows from the registers that the compiler gave the kernel - at 72, blocks of up to
+// 448 threads fit twice - and a few more after an edit would put grids of that size into two waves.
+static cudaError_t held_ctas_per_sm(int threads, int *ctas)
+{
+    static std::atomic<int> known[kMaxDevices][kWinMaxThreads / 32 + 1];
+    const int dev = current_device_index();
+    if (dev < 0)
+        return cudaErrorInvalidDevice;
+    std::atomic<int> &k = known[dev][threads / 32];
+    int n = k.load(std::memory_order_relaxed);
+    if (n == 0) {
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_window_reduce_rmsnorm<false, false>, threads, 0);
+        if (e != cudaSuccess)
+            return e;
+        n = n < 1 ? 1 : n > 2 ? 2 : n;
+        k.store(n, std::memory_order_relaxed);
+    }
+    *ctas = n;
+    return cudaSuccess;
+}
+
 cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
 {
     WindowParams p;
@@ -415,13 +438,21 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
     while (cl < uncut && ((a.H / 8) / cl > 512 || a.B * cl * 2 <= kWinMaxCtas)) cl *= 2;
     p.cluster = cl;
     const int chunks = a.H / 8 / cl;
-    // LEAN (inputs read after the wait, 64 registers) for grids that do not find room in one wave otherwise - at 72
-    // registers a CTA of up to 448 threads fits an SM twice, a larger one once - and whenever an input buffer may still be
-    // written by an earlier kernel of the same call.  Three layers, LEAN -> not: hidden 8192, batch 33 175.9 -> 168.4 us,
-    // batch 64 196.1 -> 190.8, batch 72 197.9 -> 192.3 (144 CTAs of 512 threads); batch 80 (160 CTAs) 199.5 -> 201.0, batch 128
-    // 230.8 -> 245.3; hidden 4096, batch 128 (256 CTAs of 256) 186.3 -> 183.0; hidden 5120, batch 112 188.8 -> 184.0.
+    const int threads = ((chunks + 31) / 32) * 32;
+    if (threads > kWinMaxThreads)
+        return cudaErrorInvalidValue;
+    // LEAN (inputs read after the wait, 64 registers) for grids whose CTAs do not all fit the SMs at once otherwise (two per SM
+    // at most are counted on), and whenever an input buffer may still be written by an earlier kernel of the same
+    // call.  Three layers, LEAN -> not: hidden 8192, batch 33 175.9 -> 168.4 us, batch 64 196.1 -> 190.8, batch 72 197.9 -> 192.3
+    // (144 CTAs of 512 threads); batch 80 (160 CTAs) 199.5 -> 201.0, batch 128 230.8 -> 245.3; hidden 4096, batch 128 (256 CTAs of 256)
+    // 186.3 -> 183.0; hidden 5120, batch 112 188.8 -> 184.0; hidden 6144 (384 threads), batch 75 / 96 / 128 203.6 / 220.2 / 230.4 ->
+    // 202.3 / 219.1 / 230.1; hidden 7168 (448 threads) 216.2 / 233.5 / 244.0 -> 216.4 / 235.2 / 245.9.
     const bool comm = a.comm_rank >= 0;
-    const bool lean = a.B * cl > a.sm_count * (chunks > 448 ? 1 : 2) || a.inputs_after_wait || comm;
+    int held = 1;
+    const cudaError_t he = held_ctas_per_sm(threads, &held);
+    if (he != cudaSuccess)
+        return he;
+    const bool lean = a.B * cl > a.sm_count * held || a.inputs_after_wait || comm;
     if (comm && (a.n_parts > 8 || a.part0_is_f32 || a.comm_rank >= a.n_parts))
         return cudaErrorInvalidValue;
     p.no_hint = a.inputs_after_wait;
@@ -434,9 +465,6 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
         p.comm_flags_peer[i] = a.comm_flags_peer[i];
     p.comm_epoch = a.comm_epoch;
     p.comm_done = a.comm_done;
-    const int threads = ((chunks + 31) / 32) * 32;
-    if (threads > kWinMaxThreads)
-        return cudaErrorInvalidValue;
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.B * cl);

@@ -71,8 +71,7 @@ SMALL = [
     I.small_shape(name="h384_b7", batch=7, hidden=384, ffn=224, ctx=33, seed=49),
     # window rows split over a cluster of CTAs
     I.small_shape(name="h2048_b3", batch=3, hidden=2048, ffn=256, ctx=40, tp_degree=5, seed=50),
-    # 40 rows of 8192: the window kernel's big-batch form (inputs loaded after the wait); tensor path with a
-    # 48-column batch tile and the bulk split-K hand-over
+    # 40 rows of 8192 in 160 window CTAs; tensor path with a 48-column batch tile and the bulk split-K hand-over
     I.small_shape(name="h8192_b40", batch=40, hidden=8192, ffn=256, ctx=50, ctx_min=3, n_q_heads=2, n_kv_heads=2,
                   tp_degree=3, seed=57),
 ]
@@ -83,10 +82,12 @@ def test_small_shapes_match_oracle(oracle, shape):
     full_check(oracle, shape)
 
 
-@pytest.mark.parametrize("batch,hidden", [(72, 8192), (80, 8192), (128, 8192), (128, 4096), (100, 5120)])
+@pytest.mark.parametrize("batch,hidden", [(72, 8192), (74, 8192), (75, 8192), (80, 8192), (128, 8192), (128, 4096), (100, 5120),
+                                          (100, 6144), (100, 7168), (100, 7296), (74, 7296), (75, 7296)])
 def test_window_forms_at_their_line(oracle, batch, hidden):
-    """The window kernel holds its inputs while it waits as long as its grid fits the SMs in one wave (148 SMs: 144 CTAs of
-    512 threads, 256 of 256, 200 of 320) and reads them after the wait beyond that (160 and 256 CTAs of 512 threads)."""
+    """The window kernel holds its inputs while it waits as long as its grid fits the SMs in one wave and reads them after the
+    wait beyond that: on 148 SMs up to 148 CTAs of 480 or 512 threads (hidden 7296 and 8192, batch 74; not 75), and
+    200 to 256 CTAs of 256 to 448 threads, of which an SM takes two."""
     full_check(oracle, I.small_shape(name="window_form", batch=batch, hidden=hidden, ffn=128, ctx=20, ctx_min=3, n_q_heads=2,
                                      n_kv_heads=2, tp_degree=3, seed=58))
 
