@@ -81,9 +81,15 @@ __device__ __forceinline__ uint4 ld_volatile_v4(const void *p)
 
 // (One instantiation for all four input forms: the two windows of a layer then run the same
 // instructions, which the second finds in the instruction caches.  The same caches pay for every instruction that a
-// layer's kernels do without: one chunk per thread instead of up to two, and the rolled loop over the partials beyond
-// the first burst, make 16 KB of this kernel's 30; 70B-shaped TP=8 layers at batch 20 lose 1.7 %, 8B-shaped ones at
+// layer's kernels do without: one chunk per thread instead of up to two, and no code for partials beyond the
+// first burst, make 16 KB of this kernel's 30; 70B-shaped TP=8 layers at batch 20 lose 1.7 %, 8B-shaped ones at
 // batch 5 with int8 weights 1.5 % of their time.)
+// MANY: more than eight partial-sum buffers (tensor-parallel degree 9 to 16), an instantiation of its own so that the usual
+// degrees do not carry it: the buffers beyond the first eight are hinted into L2 before the wait and
+// come in a second burst after it.  (Two at a time and without the hint a window of degree 16 paid four round trips to
+// memory behind its wait.  Three layers at degree 16: hidden 1024, batch 4 75.0 -> 64.8 us, hidden 4096, batch 8 117.2 ->
+// 106.5, hidden 8192, batch 16 158.7 -> 147.7, batch 33 201.6 -> 184.4, batch 64 212.0 -> 198.6; degree 9, batch 64 200.5 -> 193.2;
+// the hint alone or bursts of four 2-8 % slower; degrees up to 8 unchanged.)
 // LEAN, for big batches (see the launcher): the step's input buffers are only hinted into L2 before the wait and loaded after it, so that a CTA holds few registers while it
 // waits - the grid then fits beside the early-launched GEMM CTAs in one wave instead of several.  For the same
 // reason the partial buffers come in bursts of four and the gain last (at most 64 registers; at 42 it spills).
@@ -98,7 +104,7 @@ __device__ __forceinline__ uint4 ld_volatile_v4(const void *p)
 // needs no new arguments.  Buffers are reused window after window: a rank overwrites its window-A
 // buffer only after it has passed window B of the same layer, by which time every peer has
 // announced its window-B buffer and therefore finished reading window A.
-template <bool LEAN, bool COMM = false>
+template <bool LEAN, bool COMM = false, bool MANY = false>
 __global__ void __launch_bounds__(kWinMaxThreads, LEAN ? 2 : 1) k_window_reduce_rmsnorm(const __grid_constant__ WindowParams p)
 {
     const bool RESID_F32 = p.resid_f32 != 0, PART0_F32 = p.part0_f32 != 0;
@@ -165,6 +171,12 @@ __global__ void __launch_bounds__(kWinMaxThreads, LEAN ? 2 : 1) k_window_reduce_
         }
     } else if constexpr (!LEAN) {
         load_inputs();
+        if constexpr (MANY) {
+            if ((ch & 7) == 0 && mine)
+#pragma unroll 1
+                for (int j = kBurst; j < p.n_parts; ++j)
+                    line_prefetch_l2(p.parts[j] + row_off + ch);
+        }
     }
 
     if (p.cluster > 1)
@@ -232,21 +244,21 @@ __global__ void __launch_bounds__(kWinMaxThreads, LEAN ? 2 : 1) k_window_reduce_
                 v[0] += bf_lo(r.x); v[1] += bf_hi(r.x); v[2] += bf_lo(r.y); v[3] += bf_hi(r.y);
                 v[4] += bf_lo(r.z); v[5] += bf_hi(r.z); v[6] += bf_lo(r.w); v[7] += bf_hi(r.w);
             }
-        // (more partial buffers than one burst)
-        constexpr int kRest = LEAN ? 4 : 2;
+        if constexpr (LEAN || MANY) {      // the partial buffers beyond the first burst
 #pragma unroll 1
-        for (int q0 = kBurst; q0 < p.n_parts; q0 += kRest) {
-            uint4 r[kRest];
+            for (int q0 = kBurst; q0 < p.n_parts; q0 += kBurst) {
+                uint4 r[kBurst];
 #pragma unroll
-            for (int j = 0; j < kRest; ++j)
-                if (q0 + j < p.n_parts)
-                    r[j] = load_part(q0 + j, row_off + ch);
+                for (int j = 0; j < kBurst; ++j)
+                    if (q0 + j < p.n_parts)
+                        r[j] = load_part(q0 + j, row_off + ch);
 #pragma unroll
-            for (int j = 0; j < kRest; ++j)
-                if (q0 + j < p.n_parts) {
-                    v[0] += bf_lo(r[j].x); v[1] += bf_hi(r[j].x); v[2] += bf_lo(r[j].y); v[3] += bf_hi(r[j].y);
-                    v[4] += bf_lo(r[j].z); v[5] += bf_hi(r[j].z); v[6] += bf_lo(r[j].w); v[7] += bf_hi(r[j].w);
-                }
+                for (int j = 0; j < kBurst; ++j)
+                    if (q0 + j < p.n_parts) {
+                        v[0] += bf_lo(r[j].x); v[1] += bf_hi(r[j].x); v[2] += bf_lo(r[j].y); v[3] += bf_hi(r[j].y);
+                        v[4] += bf_lo(r[j].z); v[5] += bf_hi(r[j].z); v[6] += bf_lo(r[j].w); v[7] += bf_hi(r[j].w);
+                    }
+            }
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -391,7 +403,8 @@ __global__ void __launch_bounds__(kWinMaxThreads, LEAN ? 2 : 1) k_window_reduce_
 
 // CTAs of `threads` threads of the held-inputs form that an SM has room for, counted up to two.  Asked of the device
 // (once per block size): it follows from the registers that the compiler gave the kernel - at 72, blocks of up to
-// 448 threads fit twice - and a few more after an edit would put grids of that size into two waves.
+// 448 threads fit twice, at the 82 of MANY up to 352 - and a few more after an edit would put grids of that size into two waves.
+template <bool MANY>
 static cudaError_t held_ctas_per_sm(int threads, int *ctas)
 {
     static std::atomic<int> known[kMaxDevices][kWinMaxThreads / 32 + 1];
@@ -401,7 +414,7 @@ static cudaError_t held_ctas_per_sm(int threads, int *ctas)
     std::atomic<int> &k = known[dev][threads / 32];
     int n = k.load(std::memory_order_relaxed);
     if (n == 0) {
-        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_window_reduce_rmsnorm<false, false>, threads, 0);
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_window_reduce_rmsnorm<false, false, MANY>, threads, 0);
         if (e != cudaSuccess)
             return e;
         n = n < 1 ? 1 : n > 2 ? 2 : n;
@@ -448,8 +461,9 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
     // 186.3 -> 183.0; hidden 5120, batch 112 188.8 -> 184.0; hidden 6144 (384 threads), batch 75 / 96 / 128 203.6 / 220.2 / 230.4 ->
     // 202.3 / 219.1 / 230.1; hidden 7168 (448 threads) 216.2 / 233.5 / 244.0 -> 216.4 / 235.2 / 245.9.
     const bool comm = a.comm_rank >= 0;
+    const bool many = a.n_parts > 8;
     int held = 1;
-    const cudaError_t he = held_ctas_per_sm(threads, &held);
+    const cudaError_t he = many ? held_ctas_per_sm<true>(threads, &held) : held_ctas_per_sm<false>(threads, &held);
     if (he != cudaSuccess)
         return he;
     const bool lean = a.B * cl > a.sm_count * held || a.inputs_after_wait || comm;
@@ -485,7 +499,9 @@ cudaError_t launch_window(const WindowArgs &a, cudaStream_t s)
     p.part0_f32 = a.part0_is_f32;
     if (comm)
         return cudaLaunchKernelEx(&cfg, k_window_reduce_rmsnorm<true, true>, p);
-    return lean ? cudaLaunchKernelEx(&cfg, k_window_reduce_rmsnorm<true, false>, p)
+    if (lean)
+        return cudaLaunchKernelEx(&cfg, k_window_reduce_rmsnorm<true, false>, p);
+    return many ? cudaLaunchKernelEx(&cfg, k_window_reduce_rmsnorm<false, false, true>, p)
                 : cudaLaunchKernelEx(&cfg, k_window_reduce_rmsnorm<false, false>, p);
 }
 

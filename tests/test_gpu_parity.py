@@ -92,6 +92,15 @@ def test_window_forms_at_their_line(oracle, batch, hidden):
                                      n_kv_heads=2, tp_degree=3, seed=58))
 
 
+@pytest.mark.parametrize("tp,batch,hidden", [(8, 33, 8192), (9, 64, 8192), (16, 8, 8192), (16, 33, 8192), (16, 64, 8192), (16, 74, 8192),
+                                             (16, 75, 8192), (16, 100, 5632), (16, 100, 6144), (12, 100, 7168), (13, 4, 1024)])
+def test_windows_of_more_than_eight_partials(oracle, tp, batch, hidden):
+    """Up to eight partial-sum buffers are requested ahead of the wait, up to eight more in a second burst after it - or, in the
+    form for grids beyond one wave (from 75 rows of 8192, and here 100 of 6144 and 7168), all of them after it."""
+    full_check(oracle, I.small_shape(name="window_parts", batch=batch, hidden=hidden, ffn=128, ctx=20, ctx_min=3, n_q_heads=2,
+                                     n_kv_heads=2, tp_degree=tp, seed=60))
+
+
 @pytest.mark.parametrize("idx", [0, 1, 3, 4])
 def test_benchmark_configs_match_oracle(oracle, idx):
     # (with the side-stream L2 prefetch running: a budget of 16 MiB per window; the library's default
