@@ -291,18 +291,6 @@ __device__ __forceinline__ void cluster_wait()
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Cluster barrier with release / acquire order: what every CTA wrote before it is visible to all behind it.
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr)
-{
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
-    return v;
-}
-
 // Bulk copy from this CTA's shared memory into another CTA's of the cluster; the bytes are signalled
 // on the destination CTA's mbarrier.  Addresses 16-byte aligned, size a multiple of 16.  The source
 // must stay valid until the destination's barrier has completed.

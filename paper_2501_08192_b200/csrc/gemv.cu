@@ -28,14 +28,13 @@
 // Split-K partial sums are added in a fixed order, so results are bit-stable: warps
 // through shared memory; cluster ranks one-sidedly - ranks 1.. store their sums
 // into rank 0's shared memory (st.async + mbarrier complete_tx) and rank 0
-// finishes the outputs - or, when a CTA handles several groups, through
-// distributed shared memory with every rank finishing its share of the outputs.
+// finishes the outputs.
 // The fused epilogues live in epilogue.cuh.
 // The kernel runs four times a layer for microseconds, so the instructions it executes are a cost of their own (they compete
-// with the other kernels' for the instruction caches): loops outside the weight stream are rolled and the hand-over
-// without clusters' helpers is in plain instructions - four layers of hidden 2688 at batch 3 106.0 -> 101.5 us, eight
+// with the other kernels' for the instruction caches): loops outside the weight stream are rolled -
+// four layers of hidden 2688 at batch 3 106.0 -> 101.5 us, eight
 // 8B-shaped TP=8 layers at batch 5 with int8 244.3 -> 234.2, at batch 8 258.7 -> 253.9, layers of hidden 8192 at batch 8 within 0.6 %.
-// (One copy of the epilogues for the three hand-over forms makes 30 KB of 39 and costs up to 2 % of the longer
+// (One copy of the epilogues for the forms with and without ranks along k costs up to 2 % of the longer
 // streams.  A further instantiation beside this one - four row blocks per warp for gate/up - made every other kernel of the
 // layer slower: batch 8 266 -> 289 us.)
 #include "epilogue.cuh"
@@ -46,6 +45,7 @@ constexpr int kGemvWarps = 8;
 constexpr int kRingSlots = 4;
 constexpr int kUnitChunks = 2;                       // tiles per ring slot (2 KiB)
 constexpr int kGemvSmemBytes = kGemvWarps * kRingSlots * kUnitChunks * 1024;
+constexpr int kGemvRecvBytes = 7 * 2 * 16 * 16 * 4;    // most that rank 0 receives: seven ranks, two row blocks, 16 batch rows
 
 struct GemvParams {
     const uint4 *w;
@@ -59,8 +59,7 @@ struct GemvParams {
     int splits;          // cluster size along k
     int groups;          // row-block groups = row_blocks / (8 / warps_k)
     int slots;           // ring slots per warp actually used (1, 2 or 4): no more than the warp's run needs
-    int push;            // cluster reduction by one-sided hand-over to rank 0 (else every rank reads all ranks)
-    int recv_off;        // push: offset of rank 0's receive area in dynamic shared memory
+    int recv_off;        // splits > 1: offset of rank 0's receive area in dynamic shared memory
     int *status;
     long long *trace;
     const uint8_t *next_w;
@@ -92,7 +91,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
     constexpr int XF = W8 ? 2 : 1;          // uint4 of activations per tile, lane and (batch row, plane): 8 k each
     constexpr int NX = NT * XF;             // activation fragments (uint4) per tile and lane
     __shared__ float red[kGemvWarps][RB * 16][NB];       // per-warp partials
-    __shared__ float cta_part[kGemvWarps * RB][16][NB];  // per-row-block CTA partials (read across the cluster)
+    __shared__ float cta_part[kGemvWarps * RB][16][NB];  // per-row-block CTA partials
     __shared__ uint64_t bars[kGemvWarps][kRingSlots];
     __shared__ uint64_t push_bar;
     __shared__ EpilogueTables tabs;
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
     __syncwarp();
 
     const int part_floats = rbs_per_cta * 16 * NB;   // one rank's partial sums of a group
-    if (p.push) {
+    if (p.splits > 1) {
         // rank 0 will receive the other ranks' partial sums: its barrier must exist (and expect them)
         // before anybody sends - a cluster barrier, split: arrive here, wait just before the sends, so
         // that a CTA which starts late does not spend the barrier's latency ahead of its dependency wait
@@ -334,10 +333,10 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
 
         // ---- sum over the cluster ranks (fixed order)
         const int n_out = rbs_per_cta * 8 * NB;          // (row block, pair, batch row) triples of the group
-        if (p.splits > 1 && p.push) {
+        if (p.splits > 1) {
             // One-sided: ranks 1.. store their partial sums into rank 0's shared memory, signalling its
             // barrier with the bytes, and are done; rank 0 waits for all the bytes and finishes every
-            // output.  No cluster barrier on the critical path.  (One group per CTA in this mode.)
+            // output.  No cluster barrier on the critical path.  (One group per CTA: see the launcher.)
             __syncthreads();
             cluster_wait();       // (the arrival in the prologue: rank 0's barrier exists)
             float *recv = reinterpret_cast<float *>(wsm + p.recv_off);
@@ -370,29 +369,6 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                     apply_epilogue(p.epi, tabs, b, false, p.N, p.b0 + b, (grp * rbs_per_cta + rl) * 8 + r, v0, v1);
                 }
             }
-        } else if (p.splits > 1) {
-            // every rank finishes its share of the outputs, reading all ranks' partial sums
-            cluster_sync();
-#pragma unroll 1
-            for (int i = threadIdx.x * p.splits + s; i < n_out; i += blockDim.x * p.splits) {
-                const int b = i % NB, r = (i / NB) % 8, rl = i / (8 * NB);
-                if (b >= p.B)
-                    continue;
-                float v0 = 0.f, v1 = 0.f;
-#pragma unroll 1
-                for (int q = 0; q < p.splits; ++q) {
-                    const uint32_t remote = cluster_map(&cta_part[0][0][0] + (rl * 16 + r) * NB + b, q);
-                    v0 += ld_cluster_f32(remote);
-                    v1 += ld_cluster_f32(remote + 8 * NB * 4);
-                }
-                if constexpr (W8) {
-                    v0 *= scale_s[rl * 16 + r];
-                    v1 *= scale_s[rl * 16 + r + 8];
-                }
-                apply_epilogue(p.epi, tabs, b, false, p.N, p.b0 + b, (grp * rbs_per_cta + rl) * 8 + r, v0, v1);
-            }
-            cluster_sync();   // peers' shared memory must outlive the reads; also fences red/cta_part reuse
-            load_scales(grp + gridDim.x);
         } else {
             __syncthreads();
 #pragma unroll 1
@@ -411,7 +387,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
             load_scales(grp + gridDim.x);
         }
     }
-    if (p.push && s == 0) {
+    if (p.splits > 1 && s == 0) {
         // Rank 0 gave up waiting for a rank's partial sums: that rank may still store them into this
         // CTA's shared memory, and a store into a CTA that has exited is a fault.  Stay until every other
         // rank has left (its stores were issued before that), then give the stores in flight a bounded
@@ -433,7 +409,7 @@ static cudaError_t launch_variant(GemvParams &p, int sm_count, int pdl, cudaStre
 {
     static PerDeviceSize smem_limit;      // per instantiation and device
     {
-        cudaError_t e = ensure_dynamic_smem(k_gemv_splitk<NB, PACK, RB, W8>, smem_limit, kGemvSmemBytes + 32 * 1024 + 128);
+        cudaError_t e = ensure_dynamic_smem(k_gemv_splitk<NB, PACK, RB, W8>, smem_limit, kGemvSmemBytes + kGemvRecvBytes + 128);
         if (e != cudaSuccess)
             return e;
     }
@@ -465,10 +441,12 @@ static cudaError_t launch_variant(GemvParams &p, int sm_count, int pdl, cudaStre
     const int chunks_per_warp = (p.kchunks + p.splits * p.warps_k - 1) / (p.splits * p.warps_k);
     const int units = groups_per_cta * RB * ((chunks_per_warp + kUnitChunks - 1) / kUnitChunks);
     p.slots = units >= 4 ? 4 : (units >= 2 ? 2 : 1);
-    // one-sided cluster reduction when every CTA has a single group and rank 0's receive area is small
     const size_t ring_bytes = (size_t)kGemvWarps * p.slots * kUnitChunks * 1024;
     const size_t recv_bytes = (size_t)(p.splits - 1) * (kGemvWarps / p.warps_k * RB) * 16 * NB * 4;
-    p.push = p.splits > 1 && groups_per_cta == 1 && recv_bytes <= 32 * 1024;
+    // Ranks along k mean one group per CTA (the doubling above keeps groups * splits within the slots) and eight warps
+    // along k (fewer only where k is too short to be split again): at most 14 KiB to receive.
+    if (p.splits > 1 && (groups_per_cta != 1 || recv_bytes > kGemvRecvBytes))
+        return cudaErrorInvalidValue;
     p.recv_off = (int)ring_bytes;
     p.next_slice = 0;
     if (p.next_w && p.next_bytes) {
@@ -478,7 +456,7 @@ static cudaError_t launch_variant(GemvParams &p, int sm_count, int pdl, cudaStre
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(clusters, p.splits, 1);
     cfg.blockDim = dim3(kGemvWarps * 32);
-    cfg.dynamicSmemBytes = ring_bytes + (p.push ? recv_bytes : 0) + 128;
+    cfg.dynamicSmemBytes = ring_bytes + recv_bytes + 128;
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     int n = pdl_attr(at, pdl);
