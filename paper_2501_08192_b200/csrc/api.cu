@@ -411,12 +411,12 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
         // (fp16 each, its weights stored as fp16 like the others: with int8 weights the codes then take the
         // cheap fp16 widening): rounding of q is amplified by the softmax (measured: one fp16 plane put the
         // 70B-shaped chain's attention partial sums at 1.02 of the bound).
-        a.x_fp16 = which >= 1 ? 1 : 2;
+        a.planes = which >= 1 ? 1 : 2;
         a.w8 = L->w8 ? 1 : 0;
         a.scales = L->w8 ? L->scales + L->soff[which] : nullptr;
         a.w = L->arena + L->off[which];
         a.w8_early = L->cfg.hidden < 8192;
-        a.w8_tiles = L->w8 ? gemm_tc_w8_tiles(L->nb_pad, a.N, which >= 1) : 0;    // as the codes were packed
+        a.w8_tiles = L->w8 ? gemm_tc_w8_tiles(L->nb_pad, a.N, a.planes) : 0;    // as the codes were packed
         CK(L, launch_gemm_tc(a, L->sm_count, s));
         return PRESERVE_OK;
     }
@@ -1133,8 +1133,8 @@ int preserve_layer_init(const preserve_layer_config_t *cfg, const preserve_layer
             // (tensor path: blocks of one or two 128-row tiles, as the GEMM will take them per CTA)
             const int nbp = ((c.max_batch + 15) / 16) * 16;
             auto pack8 = [&](const void *const *srcs, const int *cols, int n, int i, int kind) -> cudaError_t {
-                return L->tensor_path ? launch_pack_rows_w8(srcs, cols, n, d.k[i], kind, L->arena + L->off[i],
-                                                            L->scales + L->soff[i], gemm_tc_w8_tiles(nbp, d.n[i], i >= 1),
+                return L->tensor_path ? launch_pack_tiles_w8(srcs, cols, n, d.k[i], kind, L->arena + L->off[i],
+                                                            L->scales + L->soff[i], gemm_tc_w8_tiles(nbp, d.n[i], i >= 1 ? 1 : 2),
                                                             nullptr)
                                       : launch_pack_gemv_w8(srcs, cols, n, d.k[i], kind, L->arena + L->off[i],
                                                             L->scales + L->soff[i], nullptr);
@@ -1144,12 +1144,11 @@ int preserve_layer_init(const preserve_layer_config_t *cfg, const preserve_layer
             CKI(pack8(s_gu, c_gu, 2, 2, EPI_SWIGLU));
             CKI(pack8(s_dn, c_dn, 1, 3, EPI_PLAIN));
         } else {
-            auto pack = L->tensor_path ? launch_pack_rows : launch_pack_gemv;
-            // (tensor path: Wgate|up meets the fp16 RMSNorm output x2 and is stored as fp16)
-            CKI(pack(s_qkv, c_qkv, 3, d.k[0], EPI_QKV, L->arena + L->off[0], L->tensor_path ? 1 : 0, nullptr));
-            CKI(pack(s_o, c_o, 1, d.k[1], EPI_PLAIN, L->arena + L->off[1], 1, nullptr));
-            CKI(pack(s_gu, c_gu, 2, d.k[2], EPI_SWIGLU, L->arena + L->off[2], 1, nullptr));
-            CKI(pack(s_dn, c_dn, 1, d.k[3], EPI_PLAIN, L->arena + L->off[3], 1, nullptr));
+            auto pack = L->tensor_path ? launch_pack_tiles : launch_pack_gemv;
+            CKI(pack(s_qkv, c_qkv, 3, d.k[0], EPI_QKV, L->arena + L->off[0], nullptr));
+            CKI(pack(s_o, c_o, 1, d.k[1], EPI_PLAIN, L->arena + L->off[1], nullptr));
+            CKI(pack(s_gu, c_gu, 2, d.k[2], EPI_SWIGLU, L->arena + L->off[2], nullptr));
+            CKI(pack(s_dn, c_dn, 1, d.k[3], EPI_PLAIN, L->arena + L->off[3], nullptr));
         }
     }
     // rotary frequencies theta^(-2i/d)

@@ -1,7 +1,7 @@
 // Skinny GEMM on the 5th-generation tensor cores for decode batches >= 16:
 //     y[b, n] = sum_k x[b, k] * W[n, k]
 // computed "swapped": the weight tile is the M = 128 operand, the batch (padded
-// to a multiple of 16; present twice - the hi and the lo bf16 plane of the
+// to a multiple of 16; present twice - the hi and the lo fp16 plane of the
 // activations, x = hi + lo - or once, as one fp16 plane) is the N operand, so one tcgen05.mma per 16 k covers a
 // 128 x 16-k slab of weights for every batch row at once and the CUDA cores stay
 // out of the weight stream entirely.
@@ -12,7 +12,7 @@
 //               swizzled order of shared memory: one contiguous bulk copy) and x tile (2 NB x 64, TMA, 128B swizzle) into a multi-stage ring,
 //               mbarrier full/empty; the ring's stage uses are dealt round-robin to the issuing threads
 //               (three instead of one measured < 1 %)
-//   warp 1    : allocates TMEM, issues tcgen05.mma (kind::f16, bf16 in, fp32
+//   warp 1    : allocates TMEM, issues tcgen05.mma (kind::f16, fp16 in, fp32
 //               accumulate in TMEM), tcgen05.commit frees ring slots
 //   warps 2.. : epilogue (8 or 16 warps) - tcgen05.ld the accumulator (lane = output row; the warps of
 //               a TMEM lane group share the column chunks), split-K reduction across the cluster as a
@@ -22,7 +22,7 @@
 // The kernel is instantiated per (epilogue kind, hand-over form): the tail of one instantiation is
 // a few KB of instructions, which matters for a kernel that runs for microseconds.
 // int8 weights (W8 instantiations): the ring carries the codes of 128 k per stage; the epilogue warps
-// that issue no copies widen them (exactly) to the activations' 16-bit format and store them into
+// that issue no copies widen them (exactly) to fp16 and store them into
 // tensor memory (tcgen05.st), where the MMA takes them as its A operand - shared memory stays all
 // ring, and nothing widened ever passes through it.  See the converter block below.
 // Every mbarrier wait is bounded; a wait that gives up records a status code,
@@ -63,7 +63,6 @@ struct GemmTcParams {
     int inject;         // test hook: the producer of CTA (0, 0) never fetches its first weight tile, or CTA (0, 1) never
                         // tells CTA (0, 0) that its ring is free
     int planes;         // activation planes in the B operand: 2 = hi + lo, 1 = a single fp16 plane
-    int f16;            // both operands are fp16 (else bf16)
     int epi_warps;      // 8 or 16
     int producers;      // 1..kTcMaxProducers threads that issue the ring's TMA loads (stage uses dealt round-robin)
     int w8;             // the weight tiles arrive as int8 codes and are widened into tensor memory (the MMA's A operand)
@@ -73,38 +72,26 @@ struct GemmTcParams {
     const uint8_t *w;   // packed weights: the contiguous tile of (row tile, k block), mt * 16 KiB (pack.cu)
 };
 
-// int8 -> 16-bit widening of two weight codes, exact.  The packed matrix holds every code biased by
+// int8 -> fp16 widening of two weight codes, exact.  The packed matrix holds every code biased by
 // 128 (an unsigned byte), so no sign handling is left for the kernel.  SEL places the bytes: 0x4140 =
-// bytes (0, 1) of the word, 0x4342 = bytes (2, 3).
-// fp16: the byte lands in the mantissa of 1024.0, i.e. the number 1152 + code; subtract 1152.
-// bf16 (7 mantissa bits): the low seven bits land in the mantissa of 128.0, i.e. 128 + (byte & 127);
-// subtract 128 when the byte's top bit is set (code >= 0), 256 when it is not.
-template <uint32_t SEL, bool F16>
+// bytes (0, 1) of the word, 0x4342 = bytes (2, 3).  A byte lands in the mantissa of 1024.0, i.e. the number
+// 1152 + code; subtract 1152.
+template <uint32_t SEL>
 __device__ __forceinline__ uint32_t widen_u8x2(uint32_t biased)
 {
-    uint32_t r;
-    if constexpr (F16) {
-        r = __byte_perm(biased, 0x64646464u, SEL);
-        const uint32_t off = 0x64806480u;      // (1152.0, 1152.0)
-        asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(off));
-    } else {
-        const uint32_t w = __byte_perm(biased, 0x43434343u, SEL);
-        const uint32_t minuend = w & 0xff7fff7fu, subtrahend = (w & 0x00800080u) ^ 0x43804380u;
-        asm("sub.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(minuend), "r"(subtrahend));
-    }
+    uint32_t r = __byte_perm(biased, 0x64646464u, SEL);
+    const uint32_t off = 0x64806480u;      // (1152.0, 1152.0)
+    asm("sub.f16x2 %0, %0, %1;" : "+r"(r) : "r"(off));
     return r;
 }
-// One widening pass of a converter thread over a tile: `n` tasks of 16 codes (one 16-byte load, two
-// 16-byte stores); consecutive tasks of a thread are `src_step` / `dst_step` bytes apart.
 // 16 codes (one 16-byte word group) widened to eight 32-bit registers: k elements 2c (low half) and
 // 2c + 1 (high half) in register c - the packing of a 16-bit A operand in tensor memory.
-template <bool F16>
 __device__ __forceinline__ void widen16(uint4 w, uint32_t (&r)[8])
 {
-    r[0] = widen_u8x2<0x4140, F16>(w.x); r[1] = widen_u8x2<0x4342, F16>(w.x);
-    r[2] = widen_u8x2<0x4140, F16>(w.y); r[3] = widen_u8x2<0x4342, F16>(w.y);
-    r[4] = widen_u8x2<0x4140, F16>(w.z); r[5] = widen_u8x2<0x4342, F16>(w.z);
-    r[6] = widen_u8x2<0x4140, F16>(w.w); r[7] = widen_u8x2<0x4342, F16>(w.w);
+    r[0] = widen_u8x2<0x4140>(w.x); r[1] = widen_u8x2<0x4342>(w.x);
+    r[2] = widen_u8x2<0x4140>(w.y); r[3] = widen_u8x2<0x4342>(w.y);
+    r[4] = widen_u8x2<0x4140>(w.z); r[5] = widen_u8x2<0x4342>(w.z);
+    r[6] = widen_u8x2<0x4140>(w.w); r[7] = widen_u8x2<0x4342>(w.w);
 }
 // registers -> 8 consecutive TMEM columns of this thread's lane (asynchronous; tc_st_wait completes it)
 __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t (&r)[8])
@@ -505,7 +492,6 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             n_min = n < n_min ? n : n_min;
         }
         const int G = n_min < p.w8_slots ? n_min : p.w8_slots;
-        const bool f16 = p.f16 != 0;
         const int row = quad * 32 + lane;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(mt * acc_cols);
         const uint32_t src_lane = (uint32_t)row * 128;
@@ -528,7 +514,10 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
                 tc_fence_after();
                 const uint8_t *a8 = smem + (size_t)st * stage_bytes + src_lane;
                 const uint32_t slot_addr = lane_addr + (uint32_t)(j * mt * 64);
-                for (int mh = 0; mh < 2 * mt; ++mh) {      // (weight tile, half of its 128 k): four 16-byte groups
+                // (weight tile, half of its 128 k): four 16-byte groups.  (Nothing but the widening in here: with a run-time
+                // choice of the 16-bit format per group, two 70B-shaped TP=4 layers at batch 64 took 223.2 us instead of 210.5,
+                // two TP=8 layers at batch 32 129.0 instead of 118.7.)
+                for (int mh = 0; mh < 2 * mt; ++mh) {
                     const int m = mh >> 1, q0 = (mh & 1) * 4;
                     uint4 w[4];
 #pragma unroll
@@ -537,10 +526,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         uint32_t r[8];
-                        if (f16)
-                            widen16<true>(w[q], r);
-                        else
-                            widen16<false>(w[q], r);
+                        widen16(w[q], r);
                         tc_st8(slot_addr + (uint32_t)(m * 64 + (q0 + q) * 8), r);
                     }
                 }
@@ -883,7 +869,7 @@ static cudaError_t launch_instance(cudaLaunchConfig_t &cfg, const GemmTcParams &
 // int8 weights: 128-row weight tiles per CTA (1 or 2).  The two widened tiles behind the ring cost
 // mt * 32 KiB; one weight tile per CTA when that is what lets two CTAs share an SM (the second streams
 // while the first is in its epilogue).  The packed codes are laid out for this number (pack.cu).
-int gemm_tc_w8_tiles(int NB, int N, int x_fp16)
+int gemm_tc_w8_tiles(int NB, int N, int planes)
 {
     // Narrow batches: one tile, so that two CTAs can share an SM's tensor memory (and the grid has
     // twice the CTAs to fill the SMs with).  Wide batches: two tiles (one activation tile serves both)
@@ -891,7 +877,7 @@ int gemm_tc_w8_tiles(int NB, int N, int x_fp16)
     // accumulators plus at least two widened tiles of 2 * 64 columns (128 k).
     if (NB <= 32)
         return 1;
-    const int acc = (x_fp16 ? 1 : 2) * NB;
+    const int acc = planes * NB;
     return (N % (2 * kTcTileM) == 0 && 2 * acc + 2 * 2 * 64 <= 512) ? 2 : 1;
 }
 
@@ -906,7 +892,7 @@ struct TcGeometry {
 };
 bool tc_geometry(const GemmTcArgs &a, int sm_count, int mt, TcGeometry &g)
 {
-    const int planes = a.x_fp16 == 1 ? 1 : 2;
+    const int planes = a.planes;
     const int kblocks = a.K / (a.w8 ? 2 * kTcBlockK : kTcBlockK);
     g.tiles = a.N / (kTcTileM * mt);
     // int8 weights: a stage holds the codes (half a 16-bit tile) and the activations; the widened tiles
@@ -957,7 +943,8 @@ bool tc_geometry(const GemmTcArgs &a, int sm_count, int mt, TcGeometry &g)
 
 cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
 {
-    if (a.NB < 16 || a.NB > 128 || a.NB % 16 || a.N % kTcTileM || a.K % (a.w8 ? 2 * kTcBlockK : kTcBlockK) || a.B > a.NB)
+    if (a.NB < 16 || a.NB > 128 || a.NB % 16 || a.N % kTcTileM || a.K % (a.w8 ? 2 * kTcBlockK : kTcBlockK) || a.B > a.NB ||
+        a.planes < 1 || a.planes > 2)
         return cudaErrorInvalidValue;
     GemmTcParams p;
     p.x_map = a.x_map;
@@ -967,9 +954,8 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     p.status = a.status;
     p.trace = a.trace;
     p.inject = a.inject;
-    const int planes = a.x_fp16 == 1 ? 1 : 2;
+    const int planes = a.planes;
     p.planes = planes;
-    p.f16 = a.x_fp16 ? 1 : 0;
     // 16-bit weights: one 128-row weight tile per CTA.  Two that share one activation tile halve the activations' traffic
     // and double the partial tile that the CTA's epilogue has to stage, send and finish: at batch 96 and 128 four
     // 70B-shaped TP=8 layers took 420.7 us with pairs, 387.2 without, and pairs for the two-plane QKV projection alone
@@ -999,10 +985,9 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     int cols = 32;
     while (cols < mt * planes * a.NB + w8_slots * mt * 64) cols *= 2;
     p.tmem_cols = cols;
-    // instruction descriptor: fp32 accumulate; A (weights) and B (activations) in the same 16-bit format -
-    // both bf16 (B = hi + lo planes) or both fp16 (B = one plane); N = columns of the B tile, M = 128
-    const uint32_t fmt = a.x_fp16 ? 0u : 1u;
-    p.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)((planes * a.NB) >> 3) << 17) |
+    // instruction descriptor: fp32 accumulate; A (weights) and B (activations) both fp16 (format 0);
+    // N = columns of the B tile, M = 128
+    p.idesc = (1u << 4) | ((uint32_t)((planes * a.NB) >> 3) << 17) |
               ((uint32_t)(kTcTileM >> 4) << 24);
 
     // The split-K hand-over: st.async pieces when the receive area (one partial tile per CTA) is small -

@@ -133,9 +133,12 @@ struct EpilogueArgs {
 // PLAIN has no pairing (identity order).  The packers and the epilogues agree through
 // packed_row_to_feature() in pack.cu / epilogue.cuh.
 cudaError_t launch_pack_gemv(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind,
-                             void *dst, int to_fp16, cudaStream_t s);
-cudaError_t launch_pack_rows(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind,
-                             void *dst, int to_fp16, cudaStream_t s);
+                             void *dst, cudaStream_t s);
+// the tensor path: fp16 (exact for bf16 weights of magnitude 2^-17 .. 65504) in tiles of 128 rows x 64 k, each 16 KiB in
+// one piece at ((row tile) * K / 64 + k block) * 16384, in the 128-byte swizzle of shared memory: row r at r * 128,
+// its eight 16-byte groups in the order q ^ (r % 8)
+cudaError_t launch_pack_tiles(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind,
+                              void *dst, cudaStream_t s);
 // int8 weights for the GEMV path: symmetric per-output-channel quantisation (scale = max |w| / 127 of the
 // output feature's column, code = round-to-nearest-even(w / scale), both in fp32), codes in fragment-major
 // 1 KiB tiles of 16 rows x 64 k, scales [N] in packed row order.
@@ -145,8 +148,8 @@ cudaError_t launch_pack_gemv_w8(const void *const *srcs, const int *src_cols, in
 // (unsigned bytes), in contiguous blocks of (tiles * 128 rows) x 128 k, block (row tile, k block) at
 // ((row tile) * K / 128 + k block) * tiles * 16384 - a CTA's stream of k blocks is one contiguous run; inside a
 // row the eight 16-byte groups are permuted by the row index (pack.cu)
-cudaError_t launch_pack_rows_w8(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind,
-                                void *dst_codes, float *dst_scales, int tiles, cudaStream_t s);
+cudaError_t launch_pack_tiles_w8(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind,
+                                 void *dst_codes, float *dst_scales, int tiles, cudaStream_t s);
 
 // ---- split-K GEMV (batch < 16): y[b,n] = sum_k x[b,k] W[n,k]; W in fragment-major tiles
 struct GemvArgs {
@@ -169,18 +172,16 @@ cudaError_t launch_gemv(const GemvArgs &a, int sm_count, cudaStream_t s);
 
 // ---- tcgen05 skinny GEMM (batch >= 16)
 struct GemmTcArgs {
-    CUtensorMap x_map;    // dims (K, rows, planes), box (64, NB, planes), 128B swizzle: the first NB rows of the hi and
-                          // the lo plane - or, with x_fp16 = 1, of the one fp16 plane
-    int x_fp16;           // 0: two bf16 planes; 2: two fp16 planes (hi rows then lo rows); 1: the activations are one fp16 plane (inputs that come out of an RMSNorm: bounded,
-                          // 11 significant bits suffice) instead of bf16 hi + lo planes
+    CUtensorMap x_map;    // dims (K, rows, planes), box (64, NB, planes), 128B swizzle: the first NB rows of every plane
+    int planes;           // fp16 planes of the activations: 2 = hi rows then lo rows, 1 where 11 significant bits suffice
     int B, NB, N, K;      // NB = batch rows per plane (multiple of 16)
     EpilogueArgs epi;
     int *status;
     long long *trace;
     int pdl;
     int inject;
-    const void *w;        // packed weights: contiguous tiles, fetched by plain bulk copies (launch_pack_rows, _w8)
-    // int8 weights: the kernel widens every tile to the activations' 16-bit format into tensor memory (the MMA's A operand)
+    const void *w;        // packed weights: contiguous tiles, fetched by plain bulk copies (launch_pack_tiles, _w8)
+    // int8 weights: the kernel widens every tile to fp16 into tensor memory (the MMA's A operand)
     // and multiplies every accumulator row by its scale
     int w8;
     const float *scales;  // w8: [N] in packed row order
@@ -189,7 +190,7 @@ struct GemmTcArgs {
 };
 // int8 weights: 128-row weight tiles per CTA for a matrix of N rows and a padded batch of NB (the packed
 // layout depends on it)
-int gemm_tc_w8_tiles(int NB, int N, int x_fp16);
+int gemm_tc_w8_tiles(int NB, int N, int planes);
 cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s);
 
 // ---- split-KV decode attention + merge

@@ -23,7 +23,6 @@ struct PackParams {
     int cols[3];
     int n_srcs;
     int N, K, kind;
-    int to_fp16;      // store the weights as fp16 (tensor path, matrices whose activations are one fp16 plane)
     bf16 *dst;
 };
 
@@ -57,13 +56,12 @@ __global__ void __launch_bounds__(256) k_pack_tiles(const __grid_constant__ Pack
     const bf16 *from = p.src[src] + (size_t)k0 * p.cols[src] + col;
 #pragma unroll 8
     for (int k = threadIdx.x >> 7; k < 64; k += 2) {
-        // Both operands of a tcgen05 kind::f16 MMA must have the same 16-bit format, so a matrix that is
-        // multiplied with fp16 activations is stored as fp16: exact for every bf16 weight of magnitude
+        // Both operands of a tcgen05 kind::f16 MMA must have the same 16-bit format, and the activations are fp16
+        // planes, so the weights are stored as fp16: exact for every bf16 weight of magnitude
         // 2^-17 .. 65504 (fp16 has the longer mantissa); smaller ones round to a multiple of 2^-24 (error
         // <= 2^-25, far below one bf16 ulp of any output), larger ones saturate
         const bf16 v = from[(size_t)k * p.cols[src]];
-        tile[k * kPackPitch + row] = p.to_fp16 ? __half_as_ushort(__float2half_rn(fminf(fmaxf(__bfloat162float(v), -65504.f), 65504.f)))
-                                               : __bfloat16_as_ushort(v);
+        tile[k * kPackPitch + row] = __half_as_ushort(__float2half_rn(fminf(fmaxf(__bfloat162float(v), -65504.f), 65504.f)));
     }
     __syncthreads();
     uint4 *dst = reinterpret_cast<uint4 *>(p.dst) + ((size_t)blockIdx.y * (p.K >> 6) + blockIdx.x) * 1024;
@@ -78,7 +76,7 @@ __global__ void __launch_bounds__(256) k_pack_tiles(const __grid_constant__ Pack
 }
 
 static cudaError_t launch_pack(bool tensor, const void *const *srcs, const int *src_cols, int n_srcs, int K,
-                               int kind, void *dst, int to_fp16, cudaStream_t s)
+                               int kind, void *dst, cudaStream_t s)
 {
     PackParams p = {};
     int N = 0;
@@ -91,7 +89,6 @@ static cudaError_t launch_pack(bool tensor, const void *const *srcs, const int *
     p.N = N;
     p.K = K;
     p.kind = kind;
-    p.to_fp16 = to_fp16;
     p.dst = reinterpret_cast<bf16 *>(dst);
     if (tensor) {
         if (N % 128 || K % 64)
@@ -104,7 +101,7 @@ static cudaError_t launch_pack(bool tensor, const void *const *srcs, const int *
     return cudaGetLastError();
 }
 
-// ---- int8 weights (GEMV path: fragment-major tiles; tensor path: [N, K] K-major rows of codes)
+// ---- int8 weights (GEMV path: fragment-major tiles; tensor path: contiguous blocks of codes, see launch_pack_tiles_w8)
 struct PackW8Params {
     const bf16 *src[3];
     int cols[3];
@@ -190,8 +187,8 @@ cudaError_t launch_pack_gemv_w8(const void *const *srcs, const int *src_cols, in
 {
     return launch_pack_w8(0, srcs, src_cols, n_srcs, K, kind, dst_codes, dst_scales, s);
 }
-cudaError_t launch_pack_rows_w8(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind,
-                                void *dst_codes, float *dst_scales, int tiles, cudaStream_t s)
+cudaError_t launch_pack_tiles_w8(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind,
+                                 void *dst_codes, float *dst_scales, int tiles, cudaStream_t s)
 {
     if ((tiles != 1 && tiles != 2) || K % 128)
         return cudaErrorInvalidValue;
@@ -199,15 +196,14 @@ cudaError_t launch_pack_rows_w8(const void *const *srcs, const int *src_cols, in
 }
 
 cudaError_t launch_pack_gemv(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind, void *dst,
-                             int to_fp16, cudaStream_t s)
+                             cudaStream_t s)
 {
-    (void)to_fp16;      // the GEMV path keeps bf16 weights and hi + lo bf16 activations
-    return launch_pack(false, srcs, src_cols, n_srcs, K, kind, dst, 0, s);
+    return launch_pack(false, srcs, src_cols, n_srcs, K, kind, dst, s);
 }
-cudaError_t launch_pack_rows(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind, void *dst,
-                             int to_fp16, cudaStream_t s)
+cudaError_t launch_pack_tiles(const void *const *srcs, const int *src_cols, int n_srcs, int K, int kind, void *dst,
+                              cudaStream_t s)
 {
-    return launch_pack(true, srcs, src_cols, n_srcs, K, kind, dst, to_fp16, s);
+    return launch_pack(true, srcs, src_cols, n_srcs, K, kind, dst, s);
 }
 
 }  // namespace prsv
