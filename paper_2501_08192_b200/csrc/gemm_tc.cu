@@ -609,8 +609,8 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
             const int own_c0 = (s * cols + 15) / 16, own_n = max((s + 1) * cols / 16 - own_c0, 0);     // chunks that are all this rank's
             auto stage = [&](bool own) {
                 const int n_c = own ? own_n : nchunks - own_n;
-                auto chunk = [&](int j, int &m, int &c) {
-                    m = j / n_c;
+                auto chunk = [&](int j, int &m, int &c) {      // (16-bit weights: one tile, nothing to divide)
+                    m = W8 ? j / n_c : 0;
                     c = j - m * n_c;
                     c = own ? c + own_c0 : c < own_c0 ? c : c + own_n;
                 };
