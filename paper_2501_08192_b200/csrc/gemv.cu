@@ -90,6 +90,11 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
     constexpr int NT = PACK ? 1 : 2 * NTB;  // hi planes then lo planes of the activations
     constexpr int XF = W8 ? 2 : 1;          // uint4 of activations per tile, lane and (batch row, plane): 8 k each
     constexpr int NX = NT * XF;             // activation fragments (uint4) per tile and lane
+    // Ranks whose partial sums rank 0 adds per iteration.  One (see above); at int8 weights and 9 to 15 rows the rolled loop costs
+    // the stream registers that it does not have: 44 bytes of spills, 1 % behind the unrolled loop of old.  Three layers,
+    // one -> four: hidden 8192, batch 9 / 12 / 15 229.6 / 237.4 / 243.5 -> 217.3 / 225.6 / 231.6 us, hidden 4096, batch 12 157.8 -> 145.6;
+    // other batches and 16-bit weights 0.1-0.6 % slower with four.
+    constexpr int kUnrollRanks = W8 && NB == 16 ? 4 : 1;
     __shared__ float red[kGemvWarps][RB * 16][NB];       // per-warp partials
     __shared__ float cta_part[kGemvWarps * RB][16][NB];  // per-row-block CTA partials
     __shared__ uint64_t bars[kGemvWarps][kRingSlots];
@@ -357,7 +362,7 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) k_gemv_splitk(const __grid
                     if (b >= p.B)
                         continue;
                     float v0 = cta_part[rl][r][b], v1 = cta_part[rl][r + 8][b];
-#pragma unroll 1
+#pragma unroll kUnrollRanks
                     for (int q = 1; q < p.splits; ++q) {
                         v0 += recv[(size_t)(q - 1) * part_floats + (rl * 16 + r) * NB + b];
                         v1 += recv[(size_t)(q - 1) * part_floats + (rl * 16 + r + 8) * NB + b];
