@@ -415,7 +415,7 @@ int launch_gemm(preserve_layer *L, int which, const void *x, int B, const Epilog
         a.w8 = L->w8 ? 1 : 0;
         a.scales = L->w8 ? L->scales + L->soff[which] : nullptr;
         a.w = L->arena + L->off[which];
-        a.w8_early = L->cfg.hidden < 8192;
+        a.w8_early = gemm_tc_w8_early(a.NB, L->wbytes[0] + L->wbytes[1] + L->wbytes[2] + L->wbytes[3]);
         a.w8_tiles = L->w8 ? gemm_tc_w8_tiles(L->nb_pad, a.N, a.planes) : 0;    // as the codes were packed
         CK(L, launch_gemm_tc(a, L->sm_count, s));
         return PRESERVE_OK;

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kTcMaxThreads, 1) k_gemm_tcgen05(const __grid_
     // the tensor pipe's front end spend per stage does not depend on what the stage carries, and an int8
     // stage of 64 k carries half the bytes
     constexpr int kBlk = W8 ? 2 * kTcBlockK : kTcBlockK;
-    // int8 weights, narrow batches: the codes of the ring's first fill are widened before the activations exist
+    // int8 weights: the codes of the ring's first fill are widened before the activations exist (gemm_tc_w8_early)
     constexpr bool kEarly = W8 && EARLY;
     const int mt = W8 ? p.mt : 1;     // 128-row weight tiles per CTA
     const int a_bytes = mt * kATileBytes;
@@ -881,6 +881,18 @@ int gemm_tc_w8_tiles(int NB, int N, int planes)
     return (N % (2 * kTcTileM) == 0 && 2 * acc + 2 * 2 * 64 <= 512) ? 2 : 1;
 }
 
+// int8 weights: whether the projections of a step widen the codes of their ring's first fill before the dependency wait.
+// One answer for all four of a layer: two instantiations side by side cost more than either (the caches of
+// instructions).  It pays for batches up to 48 and, beyond, where the layer is small: with long streams the first
+// fill is a small part of them, and the MMA thread's second barrier per stage costs more than it gives.
+// Two layers, not early -> early, us: hidden 8192, ffn 3584, 20 sequences of 128 (QKV alone -> all) 128.8 -> 128.0, ffn 7168, batch 33 171.1 -> 171.5,
+// hidden 7168, ffn 3584, batch 33 136.7 -> 135.1, hidden 2048, batch 33 102.0 -> 100.4; hidden 2048 (18 MB), batch 64 / 96 / 128 122.3 /
+// 150.1 / 152.5 -> 119.4 / 148.3 / 152.2, hidden 7424, ffn 2048 (80 MB) 163.2 / 202.0 / 220.5 -> 161.8 / 200.0 / 219.6; hidden 8192, ffn 1024
+// (63 MB, most of it QKV and O) 160.6 / 197.3 / 219.2 -> 161.5 / 197.9 / 220.3; hidden 4096, ffn 7168 (107 MB) 184.3 / 225.7 / 213.2
+// -> 184.8 / 226.3 / 213.2; hidden 7296, ffn 3584 (112 MB) 150.3 / 183.0 / 214.7 -> 151.4 / 185.9 / 217.1; hidden 8192, ffn 7168 (214 MB) 189.0 /
+// 231.7 / 268.7 -> 190.3 / 233.2 / 270.7.
+bool gemm_tc_w8_early(int NB, size_t layer_bytes) { return NB <= 48 || layer_bytes <= (size_t(80) << 20); }
+
 namespace {
 // How a GEMM is cut into CTAs when each takes `mt` weight tiles.
 struct TcGeometry {
@@ -973,12 +985,7 @@ cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s)
     const size_t tile_bytes = g.tile_bytes, smem_cap = g.smem_cap;
     int stages = g.stages;
     p.w8_slots = w8_slots;
-    // Codes widened before the dependency wait: always for narrow batches (two CTAs per SM, few stages per CTA), and for wide ones
-    // where the layer's weights are small enough for it to matter - two layers of hidden 2048, batch 20 of 128 78.7 -> 71.7 us,
-    // hidden 4096, batch 48 103.8 -> 97.9, hidden 7168, batch 48 147.2 -> 140.5, batch 128 within 1 %; hidden 8192, batch 48 and
-    // 64 1.6 % and 1.8 % slower.  One answer for all projections of a layer: two instantiations side by side cost more
-    // than either (the caches of instructions).
-    p.w8_early = a.w8 && (g.w8_two || a.w8_early);
+    p.w8_early = a.w8 && a.w8_early;
     p.w8 = a.w8;
     p.wscale = a.scales;
     p.splits = splits;

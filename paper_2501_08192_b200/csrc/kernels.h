@@ -185,12 +185,14 @@ struct GemmTcArgs {
     // and multiplies every accumulator row by its scale
     int w8;
     const float *scales;  // w8: [N] in packed row order
-    int w8_early;         // w8, wide batches: widen the ring's first codes before the dependency wait
+    int w8_early;         // w8: widen the ring's first codes before the dependency wait (gemm_tc_w8_early)
     int w8_tiles;         // w8: 128-row tiles per packed block and CTA (gemm_tc_w8_tiles of the largest batch)
 };
 // int8 weights: 128-row weight tiles per CTA for a matrix of N rows and a padded batch of NB (the packed
 // layout depends on it)
 int gemm_tc_w8_tiles(int NB, int N, int planes);
+// int8 weights: whether a step's projections widen the first codes early (NB columns; weight bytes of the layer)
+bool gemm_tc_w8_early(int NB, size_t layer_bytes);
 cudaError_t launch_gemm_tc(const GemmTcArgs &a, int sm_count, cudaStream_t s);
 
 // ---- split-KV decode attention + merge

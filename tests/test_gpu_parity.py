@@ -149,9 +149,18 @@ def test_int8_weights_on_benchmark_configs(oracle, idx):
 
 @pytest.mark.parametrize("batch,hidden", [(33, 8064), (33, 8192), (128, 8064), (128, 8192)])
 def test_int8_weights_of_wide_batches_at_the_line_of_early_widening(oracle, batch, hidden):
-    """Wide batches widen the first codes of a projection before its dependency wait below hidden 8192."""
+    """Wide batches of hidden 8064 and 8192: layers of at most 80 MiB of codes widen their first codes before the dependency
+    wait, here all of them."""
     full_check(oracle, I.small_shape(name="w8_early", batch=batch, hidden=hidden, ffn=256, ctx=40, ctx_min=3, n_q_heads=2,
                                      n_kv_heads=1, seed=59), flags=P.FLAG_INT8_WEIGHTS)
+
+
+@pytest.mark.parametrize("batch,hidden,ffn", [(48, 8192, 3200), (49, 8192, 3072), (49, 8192, 3200), (64, 7296, 3584), (128, 8192, 3200)])
+def test_int8_weights_at_the_lines_of_early_widening(oracle, batch, hidden, ffn):
+    """The first codes of all projections of a step are widened before the dependency wait up to 48 sequences, and beyond in
+    layers of at most 80 MiB of codes (ffn 3072 here; hidden 7296: O and down with two CTAs per SM, not early)."""
+    full_check(oracle, I.small_shape(name="w8_early", batch=batch, hidden=hidden, ffn=ffn, ctx=40, ctx_min=3, n_q_heads=2,
+                                     n_kv_heads=1, seed=61), flags=P.FLAG_INT8_WEIGHTS)
 
 
 def test_int8_weights_on_either_path_report_one_byte_per_weight():
