@@ -561,7 +561,7 @@ def measure_streams(P, torch, stream, quick: bool = True):
                 rows.append({"buffer_mib": nbytes >> 20, "source": kind,
                              "path": f"cp.async.bulk {chunk} B x{stages} stages x{producers} lanes of one warp",
                              "ctas_per_sm": 1, "gbs": round(g, 1), "gbs_per_sm": round(g / sms, 2)})
-        # the tcgen05 GEMM's kind of load: 2-D tiled TMA boxes of 64 columns x 128 / 256 rows
+        # weight tiles out of a row-major matrix: 2-D tiled TMA boxes of 64 columns x 128 / 256 rows
         for nbytes, kind in ((32 << 20, "l2"), (1 << 30, "hbm")):
             passes = 40 if kind == "l2" else 2
             for box_rows, stages, producers in ((256, 4, 1), (256, 2, 3), (128, 6, 1), (128, 4, 3)):

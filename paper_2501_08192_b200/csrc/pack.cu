@@ -45,7 +45,7 @@ __global__ void k_pack_gemv(const __grid_constant__ PackParams p)
 
 // One CTA per tile of 128 packed rows x 64 k: read along the source rows, turned in shared memory, written in one piece.
 // (Written element by element the tiles of four 70B-shaped TP=8 layers took 115 ms to prepare, as rows 70 ms.)
-constexpr int kPackPitch = 130;      // elements per k row in shared memory: no bank conflicts along either side
+constexpr int kPackPitch = 129;      // elements per k row in shared memory: odd, so that neither side has bank conflicts
 __global__ void __launch_bounds__(256) k_pack_tiles(const __grid_constant__ PackParams p)
 {
     __shared__ uint16_t tile[64 * kPackPitch];
