@@ -48,9 +48,9 @@ MIN_LAYER_STEPS = 200        # timed layer-steps per setting, whatever --steps s
 NCU_TRAFFIC = {
     ("gate_up_proj", 1): (44220000, "profiles/ncu_full_gemv_attn_window_config1_small.md (includes 14.68 MB of the "
                                     "down projection's weights that this kernel's CTAs prefetch into L2)"),
-    ("gate_up_proj", 2): (121910000, "profiles/ncu_full_gemm_tcgen05_config3_small.md"),
+    ("gate_up_proj", 2): (120834304, "profiles/ncu_full_gemm_tcgen05_config3_small.md"),
     ("attn_splitkv", 4): (542870000, "profiles/ncu_full_attn_splitkv_config5.md"),
-    ("gate_up_proj", 3): (240296448, "profiles/ncu_full_gemm_tcgen05_gate_up_config4.md (read 236.03 MB + write 4.27 MB, "
+    ("gate_up_proj", 3): (239228416, "profiles/ncu_full_gemm_tcgen05_gate_up_config4.md (read 235.98 MB + write 3.25 MB, "
                                      "full-size launch, 2-layer rotation)"),
 }
 
