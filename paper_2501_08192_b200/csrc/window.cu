@@ -14,7 +14,6 @@
 // produces (this shard's own partial sum, the fp32 residual) is read after it.
 // The kernel stays narrow (at most 8 B small CTAs): during a real allreduce the
 // SMs idle, which is what leaves HBM bandwidth to the prefetch stream.
-#include <atomic>
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
@@ -407,18 +406,18 @@ __global__ void __launch_bounds__(kWinMaxThreads, LEAN ? 2 : 1) k_window_reduce_
 template <bool MANY>
 static cudaError_t held_ctas_per_sm(int threads, int *ctas)
 {
-    static std::atomic<int> known[kMaxDevices][kWinMaxThreads / 32 + 1];
+    static PerDeviceSize known[kWinMaxThreads / 32 + 1];      // (two threads that race here find the same number)
     const int dev = current_device_index();
     if (dev < 0)
         return cudaErrorInvalidDevice;
-    std::atomic<int> &k = known[dev][threads / 32];
-    int n = k.load(std::memory_order_relaxed);
+    size_t &k = known[threads / 32].v[dev];
+    int n = (int)k;
     if (n == 0) {
         const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_window_reduce_rmsnorm<false, false, MANY>, threads, 0);
         if (e != cudaSuccess)
             return e;
         n = n < 1 ? 1 : n > 2 ? 2 : n;
-        k.store(n, std::memory_order_relaxed);
+        k = (size_t)n;
     }
     *ctas = n;
     return cudaSuccess;
