@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(kMergeMaxWarps * 32) k_attn_merge(const __grid
     pdl_launch_dependents();
     // first item of this stream: parallel count over the streams before it (lengths are inputs)
     int cnt = 0;
-#pragma unroll 1
+#pragma unroll 4
     for (int s2 = tid; s2 < sidx; s2 += blockDim.x) {
         const int nt = tiles_of(p.ctx_len[s2 / p.nkv]);
         cnt += (nt + p.tiles_per_item - 1) / p.tiles_per_item;

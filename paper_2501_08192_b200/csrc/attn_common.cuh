@@ -18,8 +18,11 @@ __device__ __forceinline__ void consumer_barrier()
 
 __device__ __forceinline__ int tiles_of(int ctx) { return (ctx + 1 + kTileKeys - 1) / kTileKeys; }
 
-// (Loops that run once per kernel or item are kept rolled: unrolled by default they were 6 KB of each attention
-// kernel's 33-48, and what a layer's kernels execute competes for the instruction caches.)
+// (Loops that run a few times per kernel or item are kept rolled: unrolled by default they were 6 KB of each attention
+// kernel's 33-48, and what a layer's kernels execute competes for the instruction caches.  Not the loops over the streams,
+// here and in the merge kernel, up to 64 dependent rounds: rolled, three layers of hidden 4096 with 16 kv heads at
+// batch 128 and 40 tokens took 286.3 us instead of 268.2, at batch 64 185.1 instead of 176.6, 8 kv heads at batch 64 and 200 tokens 200.0
+// instead of 194.1; int8 cache 314.1 / 295.8, 232.7 / 225.1 and 198.4 / 194.2; up to 128 streams the same.)
 
 // First item index of every stream, computed identically by every CTA: the lengths are
 // fetched by all threads at once (one memory round trip), then warp 0 scans them.
@@ -27,7 +30,7 @@ template <typename Params>
 __device__ __forceinline__ void build_item_table(const Params &p, int *item_base)
 {
     const int streams = p.B * p.nkv;
-#pragma unroll 1
+#pragma unroll 4
     for (int i = threadIdx.x; i < streams; i += blockDim.x) {
         const int nt = tiles_of(p.ctx_len[i / p.nkv]);
         item_base[i + 1] = (nt + p.tiles_per_item - 1) / p.tiles_per_item;
@@ -35,7 +38,7 @@ __device__ __forceinline__ void build_item_table(const Params &p, int *item_base
     __syncthreads();
     if (threadIdx.x < 32) {
         int carry = 0;
-#pragma unroll 1
+#pragma unroll 4
         for (int base = 0; base < streams; base += 32) {
             const int i = base + threadIdx.x;
             int v = i < streams ? item_base[i + 1] : 0;

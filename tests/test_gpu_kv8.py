@@ -114,6 +114,12 @@ def test_int8_attention_form_at_its_lines(oracle, shape, cluster):
     kv8_check(oracle, shape, cluster=cluster)
 
 
+@pytest.mark.parametrize("batch,heads", [(33, 16), (97, 7), (128, 16)])
+def test_int8_work_items_of_many_streams(oracle, batch, heads):
+    kv8_check(oracle, I.small_shape(name="kv8_many_streams", batch=batch, hidden=256, ffn=128, ctx=150, ctx_min=1, n_q_heads=heads,
+                                    n_kv_heads=heads, seed=272))
+
+
 @pytest.mark.parametrize("idx", [0, 1, 3, 4])
 def test_int8_cache_on_benchmark_configs(oracle, idx):
     bits = kv8_check(oracle, I.CONFIGS[idx], budget=16 << 20)

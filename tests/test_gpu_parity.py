@@ -101,6 +101,14 @@ def test_windows_of_more_than_eight_partials(oracle, tp, batch, hidden):
                                      n_kv_heads=2, tp_degree=tp, seed=60))
 
 
+@pytest.mark.parametrize("batch,heads", [(33, 16), (97, 7), (120, 16), (128, 16)])
+def test_work_items_of_many_streams(oracle, batch, heads):
+    """Every attention and merge CTA finds its work items by a scan over all (sequence, kv head) pairs, 32 at a time: 17, 22, 60
+    and 64 rounds, of which the last is full or not."""
+    full_check(oracle, I.small_shape(name="many_streams", batch=batch, hidden=256, ffn=128, ctx=150, ctx_min=1, n_q_heads=heads,
+                                     n_kv_heads=heads, seed=62))
+
+
 @pytest.mark.parametrize("idx", [0, 1, 3, 4])
 def test_benchmark_configs_match_oracle(oracle, idx):
     # (with the side-stream L2 prefetch running: a budget of 16 MiB per window; the library's default
